@@ -152,6 +152,57 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_
     }
 }
 
+// The same wait by a whole converged warp: every lane polls, the vote keeps the warp
+// converged (as elect.sync and the issue of tcgen05 / TMA instructions behind it need)
+// and makes the outcome warp-uniform.  `ready`: an earlier mbar_try_wait on the same
+// phase, polled while the previous stage's instructions were in flight, so that a phase
+// already complete costs no wait here.  ONE: only lane 0 polls (beside warps that keep the
+// load pipes busy, the router GEMM's norm jobs, whole-warp polling cost that GEMM 30 %).
+template <bool ONE = false>
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint64_t limit_ns,
+                                               const volatile int* abort_flag, bool ready = false) {
+    if (ONE) {
+        int ok = 1;
+        if ((threadIdx.x & 31) == 0) ok = ready || mbar_wait(bar, parity, limit_ns, abort_flag);
+        return __shfl_sync(0xffffffffu, ok, 0) != 0;
+    }
+    if (__all_sync(0xffffffffu, ready || mbar_try_wait(bar, parity))) return true;
+    const uint64_t t0 = globaltimer_ns();
+    for (uint32_t i = 1;; ++i) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if ((i & 127u) == 0u) {
+            const bool stop = (abort_flag && *abort_flag) || globaltimer_ns() - t0 > limit_ns;
+            if (__any_sync(0xffffffffu, stop)) return false;
+        }
+    }
+}
+// One poll that does not suspend the thread.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// True in one lane of a converged warp, always the same one.  Code that one lane runs
+// behind this predicate is known to ptxas to run in a single lane, so the instructions
+// with warp-uniform operands (tcgen05.mma and commit, TMA and bulk copies) need no loop
+// over the active lanes, which they do behind a condition on threadIdx.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
 // ------------------------------------------------------------- cp.async
 
 // 16-byte global->shared copy; src_bytes < 16 zero-fills the rest (0: all zeros,

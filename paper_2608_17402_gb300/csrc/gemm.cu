@@ -29,8 +29,9 @@
 //               TMEM lanes 32 (w%4)..+31, every other 32-column chunk), fused math,
 //               and 16-byte stores / reductions of each thread's own row
 //   warp 8      TMEM allocation (both CTAs, jointly); leader lane 0 issues the MMAs
-//   warp 9      lane 0: TMA loads of the B half and, for contiguous A rows, of A;
-//               the leader posts the byte count of both CTAs on its full barrier
+//   warp 9      TMA loads of the B half and, for contiguous A rows, of A; the leader
+//               posts the byte count of both CTAs on its full barrier.  With contiguous A
+//               warp 18 takes turns with it, stage by stage
 //   warps 10-17 token gather: 16-byte cp.async of A rows straight into the 128-byte
 //               swizzled K-major layout; each thread hands the completion of its
 //               copies to the stage's local afull barrier and moves on
@@ -318,10 +319,14 @@ __device__ __forceinline__ int rows_half(const Tile& t, uint32_t rank) {
 
 // --------------------------------------------------------------- producers
 
-// TMA producer (warp 9, lane 0): the CTA's half of B, and A when its rows are
-// contiguous.  The leader posts the byte count of both CTAs on its full barrier.
-template <bool GATHER, bool TRAIN>
-__device__ void producer_tma(const GemmArgs& p, const Smem& sm, int64_t n_work,
+// TMA producers (all lanes of a warp in step, one elected lane issues): the CTA's half of
+// B, and A when its rows are contiguous.  `np` warps take the stages in turn, warp `pid`
+// every np-th one.  The byte-count arrival, the copies and the wait of one stage are a chain
+// of about 725 cycles in one warp (clock sums in the kernel), longer than the 512 cycles of
+// the stage's MMAs: two producers took the down-projection at T = 8192, d = 1280, h = 854
+// from 141 to 137 us.  With gathered A, where the gather paces the ring, one is enough.  The leader posts the byte count of both CTAs on its full barrier.
+template <bool GATHER, bool TRAIN, bool ONE>
+__device__ void producer_tma(const GemmArgs& p, const Smem& sm, int64_t n_work, int pid, int np,
                              volatile int* abort_flag) {
     tma_prefetch_desc(&p.tmB);
     if (p.g_split < p.G || p.swiglu) tma_prefetch_desc(&p.tmB2);
@@ -340,15 +345,17 @@ __device__ void producer_tma(const GemmArgs& p, const Smem& sm, int64_t n_work,
     // gathering: plus the 16-byte signal with which the peer publishes its A half
     const uint32_t stage_tx = 2 * cta_bytes + (gather ? 16u : 0u);
     const uint32_t full_leader = peer_addr(sm.full, 0);
-    int s = 0;
+    int s = 0, turn = 0;
     uint32_t ph = 0;
+    bool ready = false;
     int64_t w = sm.pair;
-    Tile t{};
-    if (w < n_work) t = decode_tile(p, w);
+    if (w >= n_work) return;
+    Tile t = decode_tile(p, w);
     for (; w < n_work; w += sm.npairs) {
         const int64_t wn = w + sm.npairs;
-        TileLd nl{};
-        if (wn < n_work) nl = tile_load(p, wn);   // checked after this item's loads
+        // checked after this item's loads (loaded whether there is a next item or not: a
+        // conditional load would be waited for here, where its two values merge)
+        const TileLd nl = tile_load(p, wn < n_work ? wn : w);
         // B of this group: groups >= g_split from their own map; with swiglu the second
         // CTA of the pair loads the up projection (W3) beside the gate's (W1) columns
         const bool tail = t.g >= p.g_split;
@@ -358,42 +365,49 @@ __device__ void producer_tma(const GemmArgs& p, const Smem& sm, int64_t n_work,
         const int gb = (TRAIN && p.item_table == 2) ? 0 : (tail ? t.g - p.g_split : t.g);
         const int ncol0 = p.swiglu ? t.n0 : t.n0 + (int)(sm.rank * half_n);
         for (int kb = t.kb0; kb < t.kb1; ++kb) {
-            if (!mbar_wait(sm.empty + 8 * s, ph ^ 1u, p.limit_ns, abort_flag)) {
-                set_abort(abort_flag, p.status, SITE_GEMM_WAIT_EMPTY, (int)sm.pair, 1);
-                return;
-            }
-            const uint32_t bar = full_leader + 8 * s;
-            if (sm.rank == 0) mbar_arrive_expect_tx(sm.full + 8 * s, stage_tx);
-            const uint32_t b_dst = sm.b0 + s * GM_B_BYTES;
-            const int kk = kb * GM_BK;
-            if (TRAIN && p.b_kmajor) {   // half_n rows of the CTA's columns, 64 K values each
-                tma_load_3d_pair(b_dst, tmb, bar, kk, ncol0, gb);
-            } else {
-                for (uint32_t j = 0; j < nboxh; ++j)
-                    tma_load_3d_pair(b_dst + j * (GM_BK * 128), tmb, bar, ncol0 + (int)(64 * j), kk, gb);
-            }
-            if (!gather) {
-                if (TRAIN && p.a_mn) {   // two 64-row halves of the CTA's 128 output rows, 64 K rows each
-                    const int m = t.m0 + (int)sm.rank * GM_HALF;
-                    tma_load_3d_pair(sm.a0 + s * GM_A_BYTES, &p.tmA, bar, m, kk, 0);
-                    tma_load_3d_pair(sm.a0 + s * GM_A_BYTES + GM_BK * 128, &p.tmA, bar, m + 64, kk, 0);
-                } else {
-                    const int col = p.a_kperiod ? kk % p.a_kperiod : kk;
-                    tma_load_2d_pair(sm.a0 + s * GM_A_BYTES, &p.tmA, bar, col,
-                                     t.row0 + (int)sm.rank * GM_HALF);
+            if (turn == pid) {
+                if (!mbar_wait_warp<ONE>(sm.empty + 8 * s, ph ^ 1u, p.limit_ns, abort_flag, ready)) {
+                    set_abort(abort_flag, p.status, SITE_GEMM_WAIT_EMPTY, (int)sm.pair, 1);
+                    return;
                 }
+                if (elect_one()) {
+                    const uint32_t bar = full_leader + 8 * s;
+                    if (sm.rank == 0) mbar_arrive_expect_tx(sm.full + 8 * s, stage_tx);
+                    const uint32_t b_dst = sm.b0 + s * GM_B_BYTES;
+                    const int kk = kb * GM_BK;
+                    if (TRAIN && p.b_kmajor) {   // half_n rows of the CTA's columns, 64 K values each
+                        tma_load_3d_pair(b_dst, tmb, bar, kk, ncol0, gb);
+                    } else {
+                        for (uint32_t j = 0; j < nboxh; ++j)
+                            tma_load_3d_pair(b_dst + j * (GM_BK * 128), tmb, bar, ncol0 + (int)(64 * j), kk, gb);
+                    }
+                    if (!gather) {
+                        if (TRAIN && p.a_mn) {   // two 64-row halves of the CTA's 128 output rows, 64 K rows each
+                            const int m = t.m0 + (int)sm.rank * GM_HALF;
+                            tma_load_3d_pair(sm.a0 + s * GM_A_BYTES, &p.tmA, bar, m, kk, 0);
+                            tma_load_3d_pair(sm.a0 + s * GM_A_BYTES + GM_BK * 128, &p.tmA, bar, m + 64, kk, 0);
+                        } else {
+                            const int col = p.a_kperiod ? kk % p.a_kperiod : kk;
+                            tma_load_2d_pair(sm.a0 + s * GM_A_BYTES, &p.tmA, bar, col,
+                                             t.row0 + (int)sm.rank * GM_HALF);
+                        }
+                    }
+                }
+                __syncwarp();
             }
+            if (++turn == np) turn = 0;
             if (++s == sm.nstages) {
                 s = 0;
                 ph ^= 1u;
             }
+            ready = !ONE && turn == pid && mbar_test(sm.empty + 8 * s, ph ^ 1u);
         }
         if (wn < n_work) t = tile_finish(p, nl);
     }
 }
 
 // Table rows of this thread's GM_GATHER_ROWS rows of tile t (r = rb + GM_GATHER_RSTEP j of
-// the CTA's half; -1 past the tile), loaded one item ahead of their use.
+// the CTA's half; past the tile row 0's, unused), loaded one item ahead of their use.
 __device__ __forceinline__ void gather_rows_load(const GemmArgs& p, const Tile& t, uint32_t rank,
                                                  int rb, int (&raw)[GM_GATHER_ROWS]) {
     const int nh = rows_half(t, rank);
@@ -401,7 +415,7 @@ __device__ __forceinline__ void gather_rows_load(const GemmArgs& p, const Tile& 
     for (int j = 0; j < GM_GATHER_ROWS; ++j) {
         const int r = rb + GM_GATHER_RSTEP * j;
         const int gr = t.row0 + (int)rank * GM_HALF + r;
-        raw[j] = (r < nh) ? (p.a_ident ? gr : __ldg(p.a_rows + gr)) : -1;
+        raw[j] = p.a_ident ? gr : __ldg(p.a_rows + (r < nh ? gr : 0));
     }
 }
 
@@ -414,7 +428,7 @@ __device__ __forceinline__ void gather_rows_finish(const GemmArgs& p, const Tile
 #pragma unroll
     for (int j = 0; j < GM_GATHER_ROWS; ++j) {
         const int r = rb + GM_GATHER_RSTEP * j;
-        const int idx = r < nh ? raw[j] / p.a_div : -1;
+        const int idx = p.a_div == 1 ? raw[j] : raw[j] / p.a_div;
         if (r < nh && idx >= 0 && idx < p.a_nrows) {
             src[j] = p.A + (int64_t)idx * p.lda;
         } else {
@@ -434,74 +448,68 @@ __device__ __forceinline__ void gather_rows_finish(const GemmArgs& p, const Tile
 __device__ void producer_gather(const GemmArgs& p, const Smem& sm, int64_t n_work,
                                 volatile int* abort_flag) {
     const int pt = threadIdx.x - GM_WARP_GATHER * 32;   // 0 .. GM_GATHER_WARPS * 32 - 1
-    const int lane = threadIdx.x & 31;
     const int c = pt & 7, rb = pt >> 3;                  // 16-byte chunk, first row
     // gathered rows are re-read by every expert of their tokens: keep them in L2
     const uint64_t keep_pol = l2_policy_evict_last();
     int s = 0;
     uint32_t ph = 0;
-    bool ok = true;
+    bool ready = false;
     int64_t w = sm.pair;
     // The per-item set-up is pipelined so that no load is waited on at an item start:
     // item w's row pointers are ready when it starts; the next item's table rows were
     // loaded one item earlier, after its tile entry (loaded earlier still) was checked.
+    // Past the last item the last one is loaded again (unused): conditional loads would be
+    // waited for where their values merge, several thousand cycles an item.
+    if (w >= n_work) return;
     const __nv_bfloat16* src[GM_GATHER_ROWS];
     int nraw[GM_GATHER_ROWS];
-    Tile t{}, tn{};
-    TileLd nnl{};
-    if (w < n_work) {
-        t = decode_tile(p, w);
+    const int64_t w1 = w + sm.npairs < n_work ? w + sm.npairs : w;
+    const TileLd l0 = tile_load(p, w), l1 = tile_load(p, w1);
+    TileLd nnl = tile_load(p, w1 + sm.npairs < n_work ? w1 + sm.npairs : w1);
+    Tile t = tile_finish(p, l0), tn = tile_finish(p, l1);
+    {
         int raw[GM_GATHER_ROWS];
         gather_rows_load(p, t, sm.rank, rb, raw);
+        gather_rows_load(p, tn, sm.rank, rb, nraw);
         gather_rows_finish(p, t, sm.rank, rb, raw, src);
     }
-    if (w + sm.npairs < n_work) {
-        tn = decode_tile(p, w + sm.npairs);
-        gather_rows_load(p, tn, sm.rank, rb, nraw);
-    }
-    if (w + 2 * sm.npairs < n_work) nnl = tile_load(p, w + 2 * sm.npairs);
-    for (; w < n_work && ok; w += sm.npairs) {
-        const int64_t wn = w + sm.npairs;
+    const uint32_t dst_t = sm.a0 + rb * 128 + ((c ^ (rb & 7)) << 4);
+    static_assert(GM_GATHER_RSTEP % 8 == 0, "the swizzle phase is the same for all rows of a thread");
+    for (; w < n_work; w += sm.npairs) {
         for (int kb = t.kb0; kb < t.kb1; ++kb) {
-            int good = 1;
-            if (lane == 0) good = mbar_wait(sm.empty + 8 * s, ph ^ 1u, p.limit_ns, abort_flag);
-            good = __shfl_sync(0xffffffffu, good, 0);
-            if (!good) {
-                if (lane == 0) set_abort(abort_flag, p.status, SITE_GEMM_WAIT_EMPTY, (int)sm.pair, 0);
-                ok = false;
-                break;
+            if (!mbar_wait_warp(sm.empty + 8 * s, ph ^ 1u, p.limit_ns, abort_flag, ready)) {
+                set_abort(abort_flag, p.status, SITE_GEMM_WAIT_EMPTY, (int)sm.pair, 0);
+                cp_async_wait_all();
+                return;
             }
-            const uint32_t dst0 = sm.a0 + s * GM_A_BYTES;
+            const uint32_t dst0 = dst_t + s * GM_A_BYTES;
             const int kk = kb * GM_BK + c * 8;
             const bool col_ok = kk < p.K;
 #pragma unroll
             for (int j = 0; j < GM_GATHER_ROWS; ++j) {
-                const int r = rb + GM_GATHER_RSTEP * j;
-                const uint32_t dst = dst0 + r * 128 + ((c ^ (r & 7)) << 4);
                 const bool v = col_ok && src[j] != nullptr;
-                cp_async16_hint(dst, v ? (const void*)(src[j] + kk) : (const void*)p.A, v ? 16u : 0u,
-                                keep_pol);
+                cp_async16_hint(dst0 + j * (GM_GATHER_RSTEP * 128), v ? (const void*)(src[j] + kk) : (const void*)p.A,
+                                v ? 16u : 0u, keep_pol);
             }
             cp_async_arrive_noinc(sm.afull + 8 * s);
             if (++s == sm.nstages) {
                 s = 0;
                 ph ^= 1u;
             }
+            ready = mbar_test(sm.empty + 8 * s, ph ^ 1u);
         }
-        if (wn < n_work) {   // advance: item wn's pointers, item wn + npairs's table rows
-            gather_rows_finish(p, tn, sm.rank, rb, nraw, src);
-            t = tn;
-            if (wn + sm.npairs < n_work) {
-                tn = tile_finish(p, nnl);
-                gather_rows_load(p, tn, sm.rank, rb, nraw);
-                if (wn + 2 * sm.npairs < n_work) nnl = tile_load(p, wn + 2 * sm.npairs);
-            }
-        }
+        // advance: the next item's pointers, the table rows of the one after, a further entry
+        gather_rows_finish(p, tn, sm.rank, rb, nraw, src);
+        t = tn;
+        tn = tile_finish(p, nnl);
+        gather_rows_load(p, tn, sm.rank, rb, nraw);
+        const int64_t w3 = w + 3 * sm.npairs;
+        nnl = tile_load(p, w3 < n_work ? w3 : w);
     }
     cp_async_wait_all();
 }
 
-// Warp GM_WARP_FWD, lane 0, in both CTAs: once all of this CTA's gather threads'
+// Warp GM_WARP_FWD (one elected lane), in both CTAs: once all of this CTA's gather threads'
 // copies of a stage have landed (its afull barrier), make them visible to the async
 // proxy that tcgen05.mma reads shared memory through, and publish the stage on the
 // leader's full barrier: a local arrival in the leader; from the peer, a 16-byte
@@ -515,29 +523,34 @@ __device__ void gather_forwarder(const GemmArgs& p, const Smem& sm, int64_t n_wo
     const uint32_t sink_leader = peer_addr(sm.sink, 0);
     int s = 0;
     uint32_t ph = 0;
+    bool ready = false;
     for (int64_t w = sm.pair; w < n_work; w += sm.npairs) {
         int kb0, kb1;   // the item's stages; its table entry is not needed here
         tile_kb(p, (int)(w % p.ksplit), kb0, kb1);
         for (int kb = kb0; kb < kb1; ++kb) {
-            if (!mbar_wait(sm.afull + 8 * s, ph, p.limit_ns, abort_flag)) {
+            if (!mbar_wait_warp(sm.afull + 8 * s, ph, p.limit_ns, abort_flag, ready)) {
                 set_abort(abort_flag, p.status, SITE_GEMM_WAIT_FULL, (int)sm.pair, -1 - kb);
                 return;
             }
-            fence_proxy_async_smem();
-            if (sm.rank == 0) mbar_arrive(sm.full + 8 * s);
-            else bulk_signal_remote(sink_leader, sm.sink, full_leader + 8 * s);
+            if (elect_one()) {
+                fence_proxy_async_smem();
+                if (sm.rank == 0) mbar_arrive(sm.full + 8 * s);
+                else bulk_signal_remote(sink_leader, sm.sink, full_leader + 8 * s);
+            }
+            __syncwarp();
             if (++s == sm.nstages) {
                 s = 0;
                 ph ^= 1u;
             }
+            ready = mbar_test(sm.afull + 8 * s, ph);
         }
     }
 }
 
 // ------------------------------------------------------------------- MMA
 
-// Leader CTA, warp 8, lane 0.
-template <bool TRAIN>
+// Leader CTA, warp 8, all lanes in step; one elected lane issues.
+template <bool TRAIN, bool ONE>
 __device__ void mma_issuer(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64_t n_work,
                            volatile int* abort_flag) {
     // K-major operands: k-slice +32 B; MN-major operands: next 64-element atom LBO 8192,
@@ -552,15 +565,15 @@ __device__ void mma_issuer(const GemmArgs& p, const Smem& sm, uint32_t tmem, int
     int s = 0;
     uint32_t ph = 0;
     int it = 0;
-    bool issued = false;
-    TileLd nl{};   // next item's table entry, loaded one item ahead, checked when it starts
-    if (sm.pair < n_work) nl = tile_load(p, sm.pair);
+    bool issued = false, ready = false;
+    if (sm.pair >= n_work) return;
+    TileLd nl = tile_load(p, sm.pair);   // loaded one item ahead, checked when the item starts
     for (int64_t w = sm.pair; w < n_work; w += sm.npairs, ++it) {
         const Tile t = tile_finish(p, nl);
-        if (w + sm.npairs < n_work) nl = tile_load(p, w + sm.npairs);
+        nl = tile_load(p, w + sm.npairs < n_work ? w + sm.npairs : w);
         const int acc = it & 1;
         const uint32_t aph = (uint32_t)(it >> 1) & 1u;
-        if (!mbar_wait(sm.tempty + 8 * acc, aph ^ 1u, p.limit_ns, abort_flag)) {
+        if (!mbar_wait_warp<ONE>(sm.tempty + 8 * acc, aph ^ 1u, p.limit_ns, abort_flag)) {
             set_abort(abort_flag, p.status, SITE_GEMM_WAIT_TEMPTY, (int)sm.pair, it);
             break;
         }
@@ -571,7 +584,7 @@ __device__ void mma_issuer(const GemmArgs& p, const Smem& sm, uint32_t tmem, int
             // Operands in shared memory are ordered by the barrier alone (TMA bytes, or
             // gathered rows fenced to the async proxy before they were published); the
             // tcgen05 thread-sync fence is needed only where TMEM changes hands.
-            if (!mbar_wait(sm.full + 8 * s, ph, p.limit_ns, abort_flag)) {
+            if (!mbar_wait_warp<ONE>(sm.full + 8 * s, ph, p.limit_ns, abort_flag, ready)) {
                 set_abort(abort_flag, p.status, SITE_GEMM_WAIT_FULL, (int)sm.pair, kb);
                 ok = false;
                 break;
@@ -580,24 +593,30 @@ __device__ void mma_issuer(const GemmArgs& p, const Smem& sm, uint32_t tmem, int
             // (bits 0-13, address >> 4; shared addresses stay below 256 KB, no carry).
             const uint64_t ad = adesc0 + (uint64_t)((s * GM_A_BYTES) >> 4);
             const uint64_t bd = bdesc0 + (uint64_t)((s * GM_B_BYTES) >> 4);
-            tc_mma_bf16_pair(d_tmem, ad, bd, idesc, kb != t.kb0 ? 1u : 0u);
-            tc_mma_bf16_pair(d_tmem, ad + a_step, bd + b_step, idesc, 1u);
-            tc_mma_bf16_pair(d_tmem, ad + 2 * a_step, bd + 2 * b_step, idesc, 1u);
-            tc_mma_bf16_pair(d_tmem, ad + 3 * a_step, bd + 3 * b_step, idesc, 1u);
+            if (elect_one()) {
+                tc_mma_bf16_pair(d_tmem, ad, bd, idesc, kb != t.kb0 ? 1u : 0u);
+                tc_mma_bf16_pair(d_tmem, ad + a_step, bd + b_step, idesc, 1u);
+                tc_mma_bf16_pair(d_tmem, ad + 2 * a_step, bd + 2 * b_step, idesc, 1u);
+                tc_mma_bf16_pair(d_tmem, ad + 3 * a_step, bd + 3 * b_step, idesc, 1u);
+                tc_commit_pair(sm.empty + 8 * s);
+            }
+            __syncwarp();
             issued = true;
-            tc_commit_pair(sm.empty + 8 * s);
             if (++s == sm.nstages) {
                 s = 0;
                 ph ^= 1u;
             }
+            ready = mbar_test(sm.full + 8 * s, ph);
         }
         if (!ok) break;
-        tc_commit_pair(sm.tfull + 8 * acc);
+        if (elect_one()) tc_commit_pair(sm.tfull + 8 * acc);
+        __syncwarp();
     }
     // Every tcgen05.mma must be complete before TMEM is released.
     if (issued) {
-        tc_commit_pair(sm.drain);
-        if (!mbar_wait(sm.drain, 0, p.limit_ns, nullptr))
+        if (elect_one()) tc_commit_pair(sm.drain);
+        __syncwarp();
+        if (!mbar_wait_warp<ONE>(sm.drain, 0, p.limit_ns, nullptr))
             report(p.status, MOEVIE_ERR_TIMEOUT, SITE_GEMM_DRAIN, (int)sm.pair, 0);
     }
 }
@@ -660,8 +679,11 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
     const uint64_t stream_pol = l2_policy_evict_first();
     const uint32_t tempty_leader = peer_addr(sm.tempty, 0);
     int it = 0;
+    if (sm.pair >= n_work) return;
+    TileLd nl = tile_load(p, sm.pair);   // one item ahead
     for (int64_t w = sm.pair; w < n_work; w += sm.npairs, ++it) {
-        const Tile t = decode_tile(p, w);
+        const Tile t = tile_finish(p, nl);
+        nl = tile_load(p, w + sm.npairs < n_work ? w + sm.npairs : w);
         const int acc = it & 1;
         const uint32_t aph = (uint32_t)(it >> 1) & 1u;
         const int myrow = quad * 32 + lane;
@@ -945,8 +967,12 @@ __global__ void __launch_bounds__(GM_THREADS, 1) grouped_gemm_kernel(const __gri
     sm.pair = blockIdx.x >> 1;
     sm.npairs = gridDim.x >> 1;
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);   // warp-uniform
     constexpr bool gather = GATHER;   // A rows gathered by the gather warps (else TMA)
+    // TMA producer warps: with contiguous A the forwarder, idle there, joins GM_WARP_LOAD (not
+    // beside the router GEMM's side jobs, where it cost 5 %)
+    constexpr int NPROD = GATHER || ECLS == ECLS_F32 ? 1 : 2;
+    const int prod_id = warp == GM_WARP_LOAD ? 0 : NPROD > 1 && warp == GM_WARP_FWD ? 1 : -1;
     if (threadIdx.x == 0) {
         for (int s = 0; s < nst; ++s) {
             // leader's expect_tx arrival (+ the leader's forwarder; the peer's signals
@@ -988,15 +1014,13 @@ __global__ void __launch_bounds__(GM_THREADS, 1) grouped_gemm_kernel(const __gri
     if (warp < GM_EPI_WARPS) {
         epilogue<STG_ROWS, GATHER, ECLS, TRAIN>(p, sm, tmem, n_work, abort_flag);
     } else if (warp == GM_WARP_MMA) {
-        if ((threadIdx.x & 31) == 0 && sm.rank == 0) mma_issuer<TRAIN>(p, sm, tmem, n_work, abort_flag);
-    } else if (warp == GM_WARP_LOAD) {
-        if ((threadIdx.x & 31) == 0) producer_tma<GATHER, TRAIN>(p, sm, n_work, abort_flag);
-    } else if (warp == GM_WARP_FWD) {
-        if constexpr (GATHER) {
-            if ((threadIdx.x & 31) == 0) gather_forwarder(p, sm, n_work, abort_flag);
-        }
-    } else if constexpr (GATHER) {
-        producer_gather(p, sm, n_work, abort_flag);
+        if (sm.rank == 0) mma_issuer<TRAIN, ECLS == ECLS_F32>(p, sm, tmem, n_work, abort_flag);
+    } else if (prod_id >= 0) {
+        producer_tma<GATHER, TRAIN, ECLS == ECLS_F32>(p, sm, n_work, prod_id, NPROD, abort_flag);
+    } else if (GATHER && warp == GM_WARP_FWD) {
+        if constexpr (GATHER) gather_forwarder(p, sm, n_work, abort_flag);
+    } else if (GATHER && warp >= GM_WARP_GATHER && warp < GM_WARP_FWD) {
+        if constexpr (GATHER) producer_gather(p, sm, n_work, abort_flag);
     } else if (!GATHER && ECLS == ECLS_F32 && (p.zero || p.nrm_out || p.wn_out) &&
                warp >= GM_WARP_GATHER && warp < GM_WARP_FWD) {
         // Side jobs for the gather warps of a dense-A GEMM, while the MMAs run.
