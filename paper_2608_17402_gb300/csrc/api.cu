@@ -252,9 +252,20 @@ moevie_status run_gemm(const GemmSpec& g, DevStatus* st, cudaStream_t s) {
     const int64_t n_ld = g.N_ld > 0 ? g.N_ld : g.N;
     if (n_ld < g.N || n_ld % 8 != 0) return MOEVIE_ERR_UNSUPPORTED;
     const bool swiglu = g.epi == EPI_SWIGLU_BF16;
+    // Rows reduced into their tokens' rows: the transposed product (256 output columns a tile,
+    // N = the tile's rows), unless the items are band-ordered.  Measured, down-projection with
+    // staged 16-byte reductions -> transposed: T = 8192, d = 1024, E = 64 100 -> 95 us;
+    // T = 1024, d = 1536, E = 64 (one partial tile an expert) 47 -> 41 us; band-ordered,
+    // where DRAM traffic bounds the launch: T = 32768, E = 128 397 -> 393 us, T = 65536,
+    // E = 256 925 -> 1010 us.
+    a.trans = g.epi == EPI_ADD_F32 && !g.item_table ? 1 : 0;
+    if (a.trans && (g.ksplit > 1 || g.o_div > 1 || g.a_rows || g.a_ident || g.ldy >= (int64_t(1) << 31) ||
+                    (g.b_kmajor ? g.row_scale != nullptr : !g.o_rows || !g.row_scale)))
+        return MOEVIE_ERR_UNSUPPORTED;
     if (g.b_kmajor) {   // box: the CTA's half of an n-tile's columns
         int bn = 0, nnt = 0;
         choose_bn(g.N, &bn, &nnt);
+        if (a.trans) bn = GM_BM;
         if (swiglu || g.W2nd || g.b_k_ld % 8 != 0 || g.b_g_ld % 8 != 0 || g.b_k_ld < g.K)
             return MOEVIE_ERR_UNSUPPORTED;
         if (!make_kmajor_tmap(&a.tmB, g.W, g.K, g.N, g.G, g.b_k_ld, g.b_g_ld, bn / 2)) return MOEVIE_ERR_CUDA;
@@ -281,7 +292,8 @@ moevie_status run_gemm(const GemmSpec& g, DevStatus* st, cudaStream_t s) {
         if (g.a_rows || g.lda % 8 != 0 || g.item_table != 2) return MOEVIE_ERR_UNSUPPORTED;
         if (!make_weight_tmap_strided(&a.tmA, g.A, g.a_cols, g.a_nrows, 1, g.lda, g.lda * g.a_nrows))
             return MOEVIE_ERR_CUDA;
-    } else if (!g.a_rows && !make_rows_tmap(&a.tmA, g.A, g.a_cols > 0 ? g.a_cols : g.K, g.a_nrows, g.lda)) {
+    } else if (!g.a_rows && !make_rows_tmap(&a.tmA, g.A, g.a_cols > 0 ? g.a_cols : g.K, g.a_nrows, g.lda,
+                                            a.trans ? GM_ROW_BOX : GM_HALF)) {
         return MOEVIE_ERR_CUDA;
     }
     a.b_kmajor = g.b_kmajor ? 1 : 0;
@@ -307,9 +319,6 @@ moevie_status run_gemm(const GemmSpec& g, DevStatus* st, cudaStream_t s) {
     a.max_mtiles = g.tiles ? max_mtiles(g.m_total, g.G) : (g.m_total + GM_BM - 1) / GM_BM;
     a.item_table = g.item_table;
     a.a_ident = (g.a_ident && !g.a_rows) ? 1 : 0;
-    // reduction staging: a full-warp buffer (5 stages) unless the work is band-ordered
-    // (accumulator beyond L2, DRAM-bound: the sixth stage pays more)
-    a.stg_rows = g.item_table ? 16 : 32;
     if (g.zero && (g.a_rows || g.zero_n % 4 != 0 || !a16(g.zero))) return MOEVIE_ERR_UNSUPPORTED;
     a.zero = reinterpret_cast<float4*>(g.zero);
     a.zero_n = g.zero ? g.zero_n / 4 : 0;
@@ -342,6 +351,7 @@ moevie_status run_gemm(const GemmSpec& g, DevStatus* st, cudaStream_t s) {
     a.K = g.K;
     a.N = g.N;
     choose_bn(g.N, &a.BN, &a.n_ntiles);
+    if (a.trans) a.BN = GM_BM;   // as many n-tiles as choose_bn's: ceil(N / 256)
     a.n_step = a.BN;
     if (a.swiglu) {
         a.BN = GM_MAXBN;

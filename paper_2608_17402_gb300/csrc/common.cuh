@@ -236,6 +236,15 @@ __device__ __forceinline__ void st_global_v4_hint(void* p, const uint4& v, uint6
                  "r"(v.y), "r"(v.z), "r"(v.w), "l"(pol)
                  : "memory");
 }
+// *p += v as a relaxed reduction when sel >= 0 (predicated, no branch).  No memory clobber:
+// loads may move across it (nothing in the kernels that use it reads what it adds to).
+__device__ __forceinline__ void red_add_f32_if(float* p, float v, int sel) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\t"
+        "setp.ge.s32 q, %2, 0;\n\t"
+        "@q red.relaxed.gpu.global.add.f32 [%0], %1;\n\t}" ::"l"(p),
+        "f"(v), "r"(sel));
+}
 __device__ __forceinline__ void cp_async_commit() {
     asm volatile("cp.async.commit_group;" ::: "memory");
 }

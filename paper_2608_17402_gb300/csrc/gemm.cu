@@ -166,8 +166,12 @@ struct TileLd {
 __device__ __forceinline__ TileLd tile_load(const GemmArgs& p, int64_t w64) {
     TileLd l;
     const int w = (int)w64;
-    l.q = w / p.ksplit;   // split of K fastest
-    l.ks = w - l.q * p.ksplit;
+    l.q = w;
+    l.ks = 0;
+    if (p.ksplit > 1) {   // split of K fastest
+        l.q = w / p.ksplit;
+        l.ks = w - l.q * p.ksplit;
+    }
     if (p.item_table) l.d = __ldg(p.tiles + l.q);
     else if (p.tiles) l.d = __ldg(p.tiles + l.q / p.n_ntiles);
     else l.d = make_int4(0, 0, 0, 0);
@@ -300,7 +304,8 @@ struct Smem {
     uint32_t drain;
     uint32_t sink;            // 16 bytes: target / source of the peer's stage signals
     int nstages;              // operand ring depth of this launch
-    float* stg;               // reduction staging: STG_ROWS rows of GM_STG_LD floats per warp
+    float* stg;               // ECLS_ADD: GM_STG_ROWS staged rows of GM_STG_LD floats per warp;
+                              // ECLS_ADDT: 32 {token, scale} pairs per warp
     uint32_t rank;            // rank of this CTA in its pair
     int64_t pair, npairs;     // pair index and count
 };
@@ -317,6 +322,9 @@ __device__ __forceinline__ int rows_half(const Tile& t, uint32_t rank) {
     return r < 0 ? 0 : (r > GM_HALF ? GM_HALF : r);
 }
 
+// N of a transposed tile's MMAs: its rows rounded up to 64 (32 per CTA's half of B).
+__device__ __forceinline__ int trans_n(const Tile& t) { return t.nrows > 64 ? (t.nrows + 63) / 64 * 64 : 64; }
+
 // --------------------------------------------------------------- producers
 
 // TMA producers (all lanes of a warp in step, one elected lane issues): the CTA's half of
@@ -325,7 +333,7 @@ __device__ __forceinline__ int rows_half(const Tile& t, uint32_t rank) {
 // of about 725 cycles in one warp (clock sums in the kernel), longer than the 512 cycles of
 // the stage's MMAs: two producers took the down-projection at T = 8192, d = 1280, h = 854
 // from 141 to 137 us.  With gathered A, where the gather paces the ring, one is enough.  The leader posts the byte count of both CTAs on its full barrier.
-template <bool GATHER, bool TRAIN, bool ONE>
+template <bool GATHER, bool TRAIN, bool ONE, bool TRANS>
 __device__ void producer_tma(const GemmArgs& p, const Smem& sm, int64_t n_work, int pid, int np,
                              volatile int* abort_flag) {
     tma_prefetch_desc(&p.tmB);
@@ -363,14 +371,31 @@ __device__ void producer_tma(const GemmArgs& p, const Smem& sm, int64_t n_work, 
         if (p.swiglu)
             tmb = sm.rank == 1 ? (tail ? &p.tmB4 : &p.tmB2) : (tail ? &p.tmB3 : &p.tmB);
         const int gb = (TRAIN && p.item_table == 2) ? 0 : (tail ? t.g - p.g_split : t.g);
-        const int ncol0 = p.swiglu ? t.n0 : t.n0 + (int)(sm.rank * half_n);
+        const int ncol0 = p.swiglu ? t.n0 : t.n0 + (int)(sm.rank * (TRANS ? (uint32_t)GM_HALF : half_n));
+        const int rhalf = TRANS ? trans_n(t) / 2 : 0;   // rows of the CTA's half of the transposed B
         for (int kb = t.kb0; kb < t.kb1; ++kb) {
             if (turn == pid) {
                 if (!mbar_wait_warp<ONE>(sm.empty + 8 * s, ph ^ 1u, p.limit_ns, abort_flag, ready)) {
                     set_abort(abort_flag, p.status, SITE_GEMM_WAIT_EMPTY, (int)sm.pair, 1);
                     return;
                 }
-                if (elect_one()) {
+                if (TRANS && elect_one()) {
+                    const uint32_t bar = full_leader + 8 * s;
+                    if (sm.rank == 0)
+                        mbar_arrive_expect_tx(sm.full + 8 * s, 2u * (uint32_t)(GM_A_BYTES + rhalf * 128));
+                    const int kk = kb * GM_BK;
+                    const uint32_t a_dst = sm.a0 + s * GM_A_BYTES, b_dst = sm.b0 + s * GM_B_BYTES;
+                    if (TRAIN && p.b_kmajor) {   // 128 output columns' rows of 64 K values
+                        tma_load_3d_pair(a_dst, tmb, bar, kk, ncol0, gb);
+                    } else {                     // two boxes of 64 columns x 64 K rows
+                        tma_load_3d_pair(a_dst, tmb, bar, ncol0, kk, gb);
+                        tma_load_3d_pair(a_dst + GM_BK * 128, tmb, bar, ncol0 + 64, kk, gb);
+                    }
+                    const int row = t.row0 + (int)sm.rank * rhalf;
+                    for (int j = 0; j < rhalf; j += GM_ROW_BOX)
+                        tma_load_2d_pair(b_dst + j * 128, &p.tmA, bar, kk, row + j);
+                }
+                if (!TRANS && elect_one()) {
                     const uint32_t bar = full_leader + 8 * s;
                     if (sm.rank == 0) mbar_arrive_expect_tx(sm.full + 8 * s, stage_tx);
                     const uint32_t b_dst = sm.b0 + s * GM_B_BYTES;
@@ -550,13 +575,15 @@ __device__ void gather_forwarder(const GemmArgs& p, const Smem& sm, int64_t n_wo
 // ------------------------------------------------------------------- MMA
 
 // Leader CTA, warp 8, all lanes in step; one elected lane issues.
-template <bool TRAIN, bool ONE>
+template <bool TRAIN, bool ONE, bool TRANS>
 __device__ void mma_issuer(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64_t n_work,
                            volatile int* abort_flag) {
     // K-major operands: k-slice +32 B; MN-major operands: next 64-element atom LBO 8192,
-    // k-slice +2048 B (16 K rows of 128 bytes).  The forward's A is K-major, its B MN-major.
-    const bool a_mn = TRAIN && p.a_mn, b_km = TRAIN && p.b_kmajor;
-    const uint32_t idesc = idesc_bf16_f32(2 * GM_HALF, p.BN, a_mn, !b_km);
+    // k-slice +2048 B (16 K rows of 128 bytes).  The forward's A is K-major, its B MN-major;
+    // transposed, the weights are the MMA's A and the rows its K-major B.
+    const bool a_mn = TRANS ? !(TRAIN && p.b_kmajor) : TRAIN && p.a_mn;
+    const bool b_km = TRANS || (TRAIN && p.b_kmajor);
+    uint32_t idesc = idesc_bf16_f32(2 * GM_HALF, p.BN, a_mn, !b_km);
     const uint64_t adesc0 = a_mn ? smem_desc_sw128(sm.a0, 8192, 1024) : smem_desc_sw128(sm.a0, 16, 1024);
     const uint64_t bdesc0 = b_km ? smem_desc_sw128(sm.b0, 16, 1024) : smem_desc_sw128(sm.b0, 8192, 1024);
     const uint32_t a_step = a_mn ? (2048 >> 4) : (32 >> 4);
@@ -579,6 +606,7 @@ __device__ void mma_issuer(const GemmArgs& p, const Smem& sm, uint32_t tmem, int
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem + (uint32_t)acc * GM_MAXBN;
+        if (TRANS) idesc = idesc_bf16_f32(2 * GM_HALF, trans_n(t), a_mn, false);
         bool ok = true;
         for (int kb = t.kb0; kb < t.kb1; ++kb) {
             // Operands in shared memory are ordered by the barrier alone (TMA bytes, or
@@ -623,15 +651,15 @@ __device__ void mma_issuer(const GemmArgs& p, const Smem& sm, uint32_t tmem, int
 
 // -------------------------------------------------------------- epilogue
 
-// One 32-column chunk of the y-accumulator reductions of one warp: each lane holds
-// its row's 32 values; ROWS rows at a time (all 32, or 16 when the staging buffer is
-// halved) go to the warp's staging buffer, scaled and with the row's y offset; then
+// One 32-column chunk of the staged reductions (band-ordered rows, weight gradients) of one
+// warp: each lane holds its row's 32 values; GM_STG_ROWS rows at a time go to the warp's staging
+// buffer, scaled and with the row's offset; then
 // every lane reduces 4 columns of one of 4 rows per instruction, so 8 lanes cover a
 // row's 128 contiguous bytes (a whole L2 line).
-template <int ROWS>
 __device__ __forceinline__ void reduce_chunk(const GemmArgs& p, float* stg_all, int warp, int lane,
                                              const uint32_t (&v)[32], float sc, int64_t my_yoff,
                                              int n, bool store) {
+    constexpr int ROWS = GM_STG_ROWS;
     float* stg = stg_all + warp * (ROWS * GM_STG_LD);
     const int col = n + 4 * (lane & 7);
 #pragma unroll
@@ -661,6 +689,119 @@ __device__ __forceinline__ void reduce_chunk(const GemmArgs& p, float* stg_all, 
     }
 }
 
+// Epilogue of the transposed product (EPI_ADD_F32 of rows): the accumulator holds D^T, so
+// TMEM lane l of the CTA is output column n0 + 128 rank + l and TMEM column j is row j of
+// the tile.  A warp takes 32 columns and every fourth chunk of 32 rows; register i of all
+// its lanes is row i, so one scalar reduction instruction covers 128 contiguous bytes of one
+// token's row of y: whole L2 lines straight from registers.  (The product the other way
+// round holds a row per lane: its reductions needed a transposition through shared memory.)
+// Scalar 128-byte reductions run at 6.6 TB/s into an L2-resident buffer, as fast as 16-byte
+// vector ones.  The reductions bound the tile (1024 per CTA and full tile, 6 cycles each at
+// that rate, against 4096 cycles of MMAs at K = 512), so the gather warps, idle here, join
+// the eight epilogue warps: while some load their tables and accumulators the others keep
+// the reductions going.  The rows' tokens and scales are loaded one tile ahead and reach all
+// lanes through 256 bytes of shared memory per warp (two rows per 16-byte broadcast).
+template <bool TRAIN>
+__device__ void epilogue_addt(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64_t n_work, int warp,
+                              volatile int* abort_flag) {
+    const int lane = threadIdx.x & 31;
+    const int quad = warp & 3;   // the TMEM lanes a warp may read
+    const int part = warp < GM_EPI_WARPS ? warp >> 2 : 2 + ((warp - GM_WARP_GATHER) >> 2);
+    constexpr int NCH = GM_BM / 32 / GM_ADDT_PARTS;   // chunks of a warp in a full tile
+    const uint32_t tempty_leader = peer_addr(sm.tempty, 0);
+    int2* info = reinterpret_cast<int2*>(sm.stg) + (part * 4 + quad) * 32;
+    const int4* info2 = reinterpret_cast<const int4*>(info);
+    if (sm.pair >= n_work) return;
+    // token and scale of this lane's row of each of the warp's chunks (past the tile row 0's,
+    // unused); the forward has both tables
+    auto rows_load = [&](const Tile& t, int (&tok)[NCH], float (&sc)[NCH]) {
+#pragma unroll
+        for (int i = 0; i < NCH; ++i) {
+            const int r = (part + GM_ADDT_PARTS * i) * 32 + lane;
+            const int gr = r < t.nrows ? t.row0 + r : 0;
+            tok[i] = !TRAIN || p.o_rows ? __ldg(p.o_rows + gr) : gr;
+            sc[i] = !TRAIN ? __ldg(p.row_scale + gr) : p.scale;
+        }
+    };
+    int64_t w = sm.pair;
+    const int64_t w1 = w + sm.npairs < n_work ? w + sm.npairs : w;
+    const TileLd l0 = tile_load(p, w);
+    TileLd nl = tile_load(p, w1);
+    Tile t = tile_finish(p, l0);
+    int tok[NCH], ntok[NCH];
+    float sc[NCH], nsc[NCH];
+    rows_load(t, tok, sc);
+    const int ld = (int)p.ldy;
+    int it = 0;
+    for (; w < n_work; w += sm.npairs, ++it) {
+        // the next tile's entry (loaded a tile ago) and rows, the entry after it
+        const Tile tn = tile_finish(p, nl);
+        rows_load(tn, ntok, nsc);
+        const int64_t w2 = w + 2 * sm.npairs;
+        nl = tile_load(p, w2 < n_work ? w2 : w);
+        const int acc = it & 1;
+        const int nch = trans_n(t) / 32;
+        const int col = t.n0 + (int)sm.rank * GM_HALF + quad * 32 + lane;
+        const bool col_ok = col < p.N;
+        float* yb = p.yacc + col;
+        if (!mbar_wait(sm.tfull + 8 * acc, (uint32_t)(it >> 1) & 1u, p.limit_ns, abort_flag)) {
+            set_abort(abort_flag, p.status, SITE_GEMM_WAIT_TFULL, (int)sm.pair, it);
+            return;
+        }
+        tc_fence_after();
+        const uint32_t tbase = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)acc * GM_MAXBN;
+        if (part >= nch) {   // no rows for this warp in this tile
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_remote(tempty_leader + 8 * acc);
+        }
+#pragma unroll
+        for (int i = 0; i < NCH; ++i) {
+            const int ch = part + GM_ADDT_PARTS * i;
+            if (ch >= nch) break;
+            uint32_t v[32];
+            tmem_ld_32x32b_x32(tbase + ch * 32, v);
+            int tk = tok[i];
+            if (ch * 32 + lane >= t.nrows) tk = -1;
+            else if (tk < 0 || tk >= p.o_nrows) {
+                if (!(p.o_neg_skip && tk < 0))   // a padding row writes nothing
+                    report(p.status, MOEVIE_ERR_DEVICE, SITE_GEMM_OUT_ROW, t.row0 + ch * 32 + lane, tk);
+                tk = -1;
+            }
+            info[lane] = make_int2(tk, __float_as_int(sc[i]));
+            __syncwarp();
+            tmem_wait_ld();
+            if (ch + GM_ADDT_PARTS >= nch) {   // this warp's last read of the accumulator
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_remote(tempty_leader + 8 * acc);
+            }
+            if (col_ok) {
+#pragma unroll
+                for (int r0 = 0; r0 < 32; r0 += 8) {
+                    int4 q[4];   // four broadcasts in flight before the eight reductions
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) q[j] = info2[r0 / 2 + j];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int r = r0 + 2 * j;
+                        red_add_f32_if(yb + (int64_t)q[j].x * ld, __int_as_float(q[j].y) * __uint_as_float(v[r]), q[j].x);
+                        red_add_f32_if(yb + (int64_t)q[j].z * ld, __int_as_float(q[j].w) * __uint_as_float(v[r + 1]),
+                                       q[j].z);
+                    }
+                }
+            }
+            __syncwarp();
+        }
+        t = tn;
+#pragma unroll
+        for (int i = 0; i < NCH; ++i) {
+            tok[i] = ntok[i];
+            sc[i] = nsc[i];
+        }
+    }
+}
+
 // Warp w reads TMEM lanes 32 (w % 4) .. +31 (its rows) and the 32-column chunks
 // c = w / 4, w / 4 + 2, ... of each tile.  bf16 outputs and fp32 stores: each thread
 // takes its own row (32x32b loads) and writes it straight from registers with
@@ -668,7 +809,7 @@ __device__ __forceinline__ void reduce_chunk(const GemmArgs& p, float* stg_all, 
 // per-warp staging buffer so that each 16-byte vector reduction instruction of a
 // warp covers four rows x 128 contiguous bytes, i.e. whole L2 lines.  When a warp has read
 // its last chunk of the accumulator it arrives (once) on the leader's tempty barrier.
-template <int STG_ROWS, bool GATHER, int ECLS, bool TRAIN>
+template <bool GATHER, int ECLS, bool TRAIN>
 __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64_t n_work,
                          volatile int* abort_flag) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -806,7 +947,7 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
         float dg_acc = 0.f;   // EPI_DGELU_BF16: this thread's share of its row's dot
         for (int ch = half; ch < nchunk; ch += 2) {
             const int c0 = ch * 32;
-            if constexpr (ECLS == ECLS_ADD) {   // the y-accumulator reductions
+            if constexpr (ECLS == ECLS_ADD) {   // staged reductions
                 uint32_t v[32];
                 tmem_ld_32x32b_x32(tbase + c0, v);
                 tmem_wait_ld();
@@ -817,7 +958,7 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
                 }
                 const int n = t.n0 + c0;
                 const int64_t my_yoff = ok_row ? t.ks * p.y_split_stride + tok * p.ldy : -1;
-                reduce_chunk<STG_ROWS>(p, sm.stg, warp, lane, v, sc, my_yoff, n, TRAIN && t.store);
+                reduce_chunk(p, sm.stg, warp, lane, v, sc, my_yoff, n, TRAIN && t.store);
                 continue;
             }
             uint32_t v[32];
@@ -935,18 +1076,16 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
     }
 }
 
-// STG_ROWS: rows per warp of the reduction staging buffer (EPI_ADD_F32), one kernel
-// instance each so that the epilogue loops have constant trip counts.
-template <int STG_ROWS, bool GATHER, int ECLS, bool TRAIN>
+template <bool GATHER, int ECLS, bool TRAIN>
 __global__ void __launch_bounds__(GM_THREADS, 1) grouped_gemm_kernel(const __grid_constant__ GemmArgs p) {
     extern __shared__ uint8_t gm_smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(gm_smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint8_t* sA = smem;
-    const int nst = gm_stages(ECLS == ECLS_ADD ? EPI_ADD_F32 : p.epi, STG_ROWS);
+    constexpr int nst = gm_stages(ECLS);
     uint8_t* sB = smem + nst * GM_A_BYTES;
-    uint8_t* sStg = sB + nst * GM_B_BYTES;                       // reduction staging (EPI_ADD_F32)
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sStg + gm_stg_bytes(ECLS == ECLS_ADD ? EPI_ADD_F32 : p.epi, STG_ROWS));
+    uint8_t* sStg = sB + nst * GM_B_BYTES;                       // epilogue staging
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sStg + gm_stg_bytes(ECLS));
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * GM_STAGES_MAX + 5);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     uint8_t* sink = reinterpret_cast<uint8_t*>(bars) + 256;   // 16-byte aligned, after the barriers
@@ -983,7 +1122,8 @@ __global__ void __launch_bounds__(GM_THREADS, 1) grouped_gemm_kernel(const __gri
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(sm.tfull + 8 * a, 1);         // multicast tcgen05.commit
-            mbar_init(sm.tempty + 8 * a, 2 * GM_EPI_WARPS);   // every epilogue warp of the pair
+            // every epilogue warp of the pair
+            mbar_init(sm.tempty + 8 * a, 2 * (ECLS == ECLS_ADDT ? 4 * GM_ADDT_PARTS : GM_EPI_WARPS));
         }
         mbar_init(sm.drain, 1);
         *abort_flag = 0;
@@ -1011,12 +1151,13 @@ __global__ void __launch_bounds__(GM_THREADS, 1) grouped_gemm_kernel(const __gri
     }
     const int64_t n_work = p.item_table ? n_mtiles * p.ksplit : n_mtiles * p.n_ntiles * p.ksplit;
 
-    if (warp < GM_EPI_WARPS) {
-        epilogue<STG_ROWS, GATHER, ECLS, TRAIN>(p, sm, tmem, n_work, abort_flag);
+    if (warp < GM_EPI_WARPS || (ECLS == ECLS_ADDT && warp >= GM_WARP_GATHER && warp < GM_WARP_FWD)) {
+        if constexpr (ECLS == ECLS_ADDT) epilogue_addt<TRAIN>(p, sm, tmem, n_work, warp, abort_flag);
+        else epilogue<GATHER, ECLS, TRAIN>(p, sm, tmem, n_work, abort_flag);
     } else if (warp == GM_WARP_MMA) {
-        if (sm.rank == 0) mma_issuer<TRAIN, ECLS == ECLS_F32>(p, sm, tmem, n_work, abort_flag);
+        if (sm.rank == 0) mma_issuer<TRAIN, ECLS == ECLS_F32, ECLS == ECLS_ADDT>(p, sm, tmem, n_work, abort_flag);
     } else if (prod_id >= 0) {
-        producer_tma<GATHER, TRAIN, ECLS == ECLS_F32>(p, sm, n_work, prod_id, NPROD, abort_flag);
+        producer_tma<GATHER, TRAIN, ECLS == ECLS_F32, ECLS == ECLS_ADDT>(p, sm, n_work, prod_id, NPROD, abort_flag);
     } else if (GATHER && warp == GM_WARP_FWD) {
         if constexpr (GATHER) gather_forwarder(p, sm, n_work, abort_flag);
     } else if (GATHER && warp >= GM_WARP_GATHER && warp < GM_WARP_FWD) {
@@ -1135,12 +1276,13 @@ bool make_kmajor_tmap(CUtensorMap* tm, const void* base, int64_t K, int64_t N, i
     return r == CUDA_SUCCESS;
 }
 
-bool make_rows_tmap(CUtensorMap* tm, const void* base, int64_t cols, int64_t rows, int64_t ld) {
+bool make_rows_tmap(CUtensorMap* tm, const void* base, int64_t cols, int64_t rows, int64_t ld,
+                    int box_rows) {
     PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode_fn();
-    if (!enc) return false;
+    if (!enc || box_rows < 8 || box_rows > 256) return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    cuuint32_t box[2] = {64, (cuuint32_t)GM_HALF};
+    cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides,
                      box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -1157,18 +1299,24 @@ void choose_bn(int N, int* BN, int* n_ntiles) {
 }
 
 cudaError_t launch_grouped_gemm(const GemmArgs& a, int grid, cudaStream_t s) {
-    if (a.stg_rows != 32 && a.stg_rows != 16) return cudaErrorInvalidValue;
-    // one instance per (staging rows, A path, epilogue class, training-path layouts): each
-    // holds only the code its launches run (constant trip counts, no other epilogue or
-    // operand layout to crowd its registers)
+    // one instance per (A path, epilogue class, training-path layouts): each holds only the
+    // code its launches run (constant trip counts, no other epilogue or operand layout to
+    // crowd its registers)
     using Kern = void (*)(GemmArgs);
-    static const Kern kerns[8] = {
-        grouped_gemm_kernel<32, false, ECLS_ADD, false>, grouped_gemm_kernel<16, false, ECLS_ADD, false>,
-        grouped_gemm_kernel<32, false, ECLS_F32, false>, grouped_gemm_kernel<32, false, ECLS_BF16, false>,
-        grouped_gemm_kernel<32, true, ECLS_BF16, false>,
-        // the training path: K-major B, M-major A, weight-gradient items, backward epilogues
-        grouped_gemm_kernel<32, true, ECLS_BF16, true>, grouped_gemm_kernel<32, false, ECLS_ADD, true>,
-        grouped_gemm_kernel<16, false, ECLS_ADD, true>};
+    struct Inst {
+        Kern kern;
+        int ecls;
+    };
+    static const Inst insts[8] = {
+        {grouped_gemm_kernel<false, ECLS_ADDT, false>, ECLS_ADDT},
+        {grouped_gemm_kernel<false, ECLS_F32, false>, ECLS_F32},
+        {grouped_gemm_kernel<false, ECLS_BF16, false>, ECLS_BF16},
+        {grouped_gemm_kernel<true, ECLS_BF16, false>, ECLS_BF16},
+        // the training path: K-major weights, M-major A, weight-gradient items, backward epilogues
+        {grouped_gemm_kernel<true, ECLS_BF16, true>, ECLS_BF16},
+        {grouped_gemm_kernel<false, ECLS_ADDT, true>, ECLS_ADDT},
+        {grouped_gemm_kernel<false, ECLS_ADD, true>, ECLS_ADD},
+        {grouped_gemm_kernel<false, ECLS_ADD, false>, ECLS_ADD}};
     const bool gathered = a.a_rows || a.a_ident;   // A rows through the gather warps
     const bool train = a.b_kmajor || a.a_mn || a.item_table == 2 || a.epi == EPI_GELU2_BF16 ||
                        a.epi == EPI_DGELU_BF16 || a.epi == EPI_DSWIGLU_BF16 || a.out2 != nullptr;
@@ -1176,22 +1324,21 @@ cudaError_t launch_grouped_gemm(const GemmArgs& a, int grid, cudaStream_t s) {
                           a.epi == EPI_GELU2_BF16 || a.epi == EPI_DGELU_BF16 || a.epi == EPI_DSWIGLU_BF16;
     if (gathered && !bf16_out) return cudaErrorInvalidValue;
     if (!gathered && a.epi == EPI_SWIGLU_BF16) return cudaErrorInvalidValue;
-    Kern kern;
-    if (train) {
-        if (gathered) kern = kerns[5];
-        else if (a.epi == EPI_ADD_F32) kern = a.stg_rows == 32 ? kerns[6] : kerns[7];
-        else return cudaErrorInvalidValue;
-    } else if (gathered) kern = kerns[4];
-    else if (a.epi == EPI_ADD_F32) kern = a.stg_rows == 32 ? kerns[0] : kerns[1];
-    else if (a.epi == EPI_STORE_F32 || a.epi == EPI_SUM2_F32) kern = kerns[2];
-    else kern = kerns[3];
+    if (a.trans && (a.epi != EPI_ADD_F32 || a.item_table)) return cudaErrorInvalidValue;
+    int which;
+    if (a.trans) which = train ? 5 : 0;
+    else if (train && gathered) which = 4;
+    else if (a.epi == EPI_ADD_F32) which = train ? 6 : 7;
+    else if (train) return cudaErrorInvalidValue;
+    else if (gathered) which = 3;
+    else which = a.epi == EPI_STORE_F32 || a.epi == EPI_SUM2_F32 ? 1 : 2;
     static bool attr_set[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
-        for (Kern k : kerns) {
-            cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 GM_SMEM_BYTES_MAX);
+        for (const Inst& k : insts) {
+            cudaError_t e = cudaFuncSetAttribute(k.kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 gm_smem_bytes(k.ecls));
             if (e != cudaSuccess) return e;
         }
         attr_set[dev] = true;
@@ -1199,7 +1346,7 @@ cudaError_t launch_grouped_gemm(const GemmArgs& a, int grid, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((grid + 1) & ~1));   // whole pairs
     cfg.blockDim = dim3(GM_THREADS);
-    cfg.dynamicSmemBytes = gm_smem_bytes(a.epi, a.stg_rows);
+    cfg.dynamicSmemBytes = gm_smem_bytes(insts[which].ecls);
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1210,7 +1357,7 @@ cudaError_t launch_grouped_gemm(const GemmArgs& a, int grid, cudaStream_t s) {
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, insts[which].kern, a);
     count_launches(1);
     return e != cudaSuccess ? e : cudaGetLastError();
 }

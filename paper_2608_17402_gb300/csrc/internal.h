@@ -170,34 +170,44 @@ constexpr int GM_GATHER_RSTEP = GM_GATHER_WARPS * 32 / 8;
 constexpr int GM_GATHER_ROWS = 128 / GM_GATHER_RSTEP;
 constexpr int GM_A_BYTES = GM_HALF * GM_BK * 2;           // one CTA's A rows per stage
 constexpr int GM_B_BYTES = GM_BK * (GM_MAXBN / 2) * 2;    // one CTA's half of B per stage
-constexpr int GM_STG_ROWS = 32;    // rows per warp in the reduction staging buffer (at most)
+constexpr int GM_STG_ROWS = 16;    // ECLS_ADD: rows per warp in the reduction staging buffer
 constexpr int GM_STG_LD = 36;      // floats per staged row: 32 values, the row's y offset, pad
 constexpr int GM_OVERHEAD_BYTES = 1024 + 512;   // alignment, barriers / TMEM slot / flags / sink
-// The y-accumulator epilogue (epi 2, EPI_ADD_F32) stages stg_rows (32 or 16) rows per warp
-// and gives up operand stages for them: 32 rows -> 5 stages, 16 rows -> 6.  Other
-// epilogues run 7 stages.
-__host__ __device__ constexpr int gm_stg_bytes(int epi, int stg_rows) {
-    return epi == 2 ? GM_EPI_WARPS * stg_rows * GM_STG_LD * 4 : 0;
+// Epilogue classes of the grouped GEMM's kernel instances: bf16 outputs (GELU, SwiGLU,
+// plain), fp32 stores (plain, two-group sums), staged fp32 reductions (weight-gradient
+// tiles, which also store, and band-ordered rows), and fp32 reductions of rows into their
+// tokens' rows by the transposed product.
+enum { ECLS_BF16 = 0, ECLS_F32 = 1, ECLS_ADD = 2, ECLS_ADDT = 3 };
+// Epilogue warps per TMEM lane quadrant of ECLS_ADDT: two epilogue warps and two of the
+// (idle) gather warps, each taking every fourth chunk of 32 rows.
+constexpr int GM_ADDT_PARTS = 4;
+static_assert(4 * GM_ADDT_PARTS == GM_EPI_WARPS + GM_GATHER_WARPS, "the gather warps join the epilogue");
+// Shared memory beside the operand ring: ECLS_ADD stages 16 rows per warp, ECLS_ADDT keeps
+// the {token, scale} pairs of 32 rows per warp; both give up one of the 7 stages.
+__host__ __device__ constexpr int gm_stg_bytes(int ecls) {
+    return ecls == ECLS_ADD ? GM_EPI_WARPS * GM_STG_ROWS * GM_STG_LD * 4
+           : ecls == ECLS_ADDT ? 4 * GM_ADDT_PARTS * 32 * 8 : 0;
 }
-__host__ __device__ constexpr int gm_stages(int epi, int stg_rows) {
-    return epi == 2 ? (stg_rows > 16 ? 5 : 6) : 7;
+__host__ __device__ constexpr int gm_stages(int ecls) {
+    return ecls == ECLS_ADD || ecls == ECLS_ADDT ? 6 : 7;
 }
-__host__ __device__ constexpr int gm_smem_bytes(int epi, int stg_rows) {
-    return gm_stages(epi, stg_rows) * (GM_A_BYTES + GM_B_BYTES) + gm_stg_bytes(epi, stg_rows) +
-           GM_OVERHEAD_BYTES;
+__host__ __device__ constexpr int gm_smem_bytes(int ecls) {
+    return gm_stages(ecls) * (GM_A_BYTES + GM_B_BYTES) + gm_stg_bytes(ecls) + GM_OVERHEAD_BYTES;
 }
-constexpr int GM_SMEM_BYTES_MAX = GM_STAGES_MAX * (GM_A_BYTES + GM_B_BYTES) + GM_OVERHEAD_BYTES;
-static_assert(GM_SMEM_BYTES_MAX <= 232448 && gm_smem_bytes(2, 32) <= 232448 &&
-                  gm_smem_bytes(2, 16) <= 232448,
+static_assert(gm_smem_bytes(ECLS_BF16) <= 232448 && gm_smem_bytes(ECLS_ADD) <= 232448 &&
+                  gm_smem_bytes(ECLS_ADDT) <= 232448,
               "shared memory of one CTA");
 static_assert(3 * GM_STAGES_MAX + 5 <= 32, "barriers fit before the signal sink at +256 bytes");
+// The transposed product reads the GEMM rows through boxes of 32 rows, as many as its
+// N (the tile's rows rounded up to 64, half of them per CTA) needs.
+constexpr int GM_ROW_BOX = 32;
 
 inline int64_t max_mtiles(int64_t rows, int64_t groups) { return (rows + GM_BM - 1) / GM_BM + groups; }
 
 enum Epilogue : int {
     EPI_GELU_BF16 = 0,   // out[r, n] = bf16(GELU(acc))
     EPI_STORE_BF16 = 1,  // out[r, n] = bf16(acc)
-    EPI_ADD_F32 = 2,     // yacc[tok(r), n] += scale(r) * acc   (vector atomics)
+    EPI_ADD_F32 = 2,     // yacc[tok(r), n] += scale(r) * acc   (reductions)
     EPI_STORE_F32 = 3,   // yacc[tok(r), n]  = scale(r) * acc
     EPI_SWIGLU_BF16 = 5, // out[r, n] = bf16(SiLU(acc[gate n]) * acc[up n]): accumulator columns
                          //   0..127 from W1 (gate, the pair's first CTA's B half), 128..255 from
@@ -210,18 +220,16 @@ enum Epilogue : int {
     EPI_DSWIGLU_BF16 = 8,// SwiGLU a = SiLU(u) v: out = du = bf16(scale acc v SiLU'(u)), out2 = dv =
                          //   bf16(scale acc SiLU(u)), and the row dot sum_n acc a as for EPI_DGELU_BF16
 };
-static_assert(EPI_ADD_F32 == 2, "gm_stages / gm_smem_bytes test the reduction epilogue by value");
-// Epilogue classes of the grouped GEMM's kernel instances: bf16 outputs (GELU, SwiGLU,
-// plain), fp32 stores (plain, two-group sums), fp32 reductions into the accumulator.
-enum { ECLS_BF16 = 0, ECLS_F32 = 1, ECLS_ADD = 2 };
-
 struct GemmArgs {
     CUtensorMap tmB;            // B = weights [G][K][N] bf16 (N contiguous), 3-D map {N, K, G}
     CUtensorMap tmB2;           // groups g >= g_split: B from this map, group g - g_split
     CUtensorMap tmB3;           // swiglu with groups g >= g_split: their gate (CTA rank 0) and
     CUtensorMap tmB4;           //   up (rank 1) weights, group g - g_split
     CUtensorMap tmA;            // A = rows [a_nrows][K_A] bf16, 2-D map {K_A, a_nrows}, box
-                                // {64, 128}; used when A rows are contiguous (a_rows == nullptr)
+                                // {64, 128} ({64, 32} with trans); used when A rows are
+                                // contiguous (a_rows == nullptr)
+    int trans;                  // EPI_ADD_F32 of rows without an item table: D^T = B^T A^T, output
+                                //   columns along the MMA's M, rows along its N (epilogue_addt)
     const __nv_bfloat16* A;     // A rows, for the token gather
     int64_t lda;
     const int32_t* a_rows;      // A row of GEMM row r: a_rows ? a_rows[r] / a_div : r (gather)
@@ -233,7 +241,6 @@ struct GemmArgs {
                                 // with item_table: work items {g, row0, nrows, n0}
     int item_table;             // tiles lists (m-tile, n-tile) items; *n_tiles_dev counts items
     int a_ident;                // gathered path with A row r = r (contiguous rows through cp.async)
-    int stg_rows;               // EPI_ADD_F32: rows staged per warp and phase (32 or 16)
     const int32_t* n_tiles_dev; // number of entries of `tiles`
     int64_t max_mtiles;         // host bound on *n_tiles_dev
     int G, K, N, BN, n_ntiles, num_kb, nbox;
@@ -265,8 +272,8 @@ struct GemmArgs {
     float* wn_out;              //   (the router's |W_r[:, e]| and |lo_e| from per-CTA partial sums)
     // Operand layouts and work items of the training path (all 0 on the forward):
     int b_kmajor;               // B stored K-major, W[G][N][K] (K contiguous): tmB is the 3-D map
-                                //   {K, N, G} with box {64, BN/2, 1}; the shared tile holds BN/2
-                                //   rows of 128 bytes like A's
+                                //   {K, N, G} with box {64, BN/2, 1} (trans: {64, 128, 1}); the
+                                //   shared tile holds those rows of 128 bytes like A's
     int a_mn;                   // A stored M-major, A[K][M] (M contiguous): tmA is the 3-D map
                                 //   {M, K, 1} with box {64, 64, 1}, two boxes per CTA and stage
     int wg_M;                   // item_table == 2: weight-gradient items {g, m0 | n0 << 16, kb0,
@@ -292,8 +299,9 @@ bool make_weight_tmap(CUtensorMap* tm, const void* base, int64_t N, int64_t K, i
 bool make_weight_tmap_strided(CUtensorMap* tm, const void* base, int64_t N, int64_t K, int64_t G,
                               int64_t k_ld, int64_t g_ld);
 // Encodes the 2-D row tensor map {cols, rows} of A[rows][cols] bf16 (row stride ld
-// elements), box {64, GM_HALF}.
-bool make_rows_tmap(CUtensorMap* tm, const void* base, int64_t cols, int64_t rows, int64_t ld);
+// elements), box {64, box_rows}.
+bool make_rows_tmap(CUtensorMap* tm, const void* base, int64_t cols, int64_t rows, int64_t ld,
+                    int box_rows = GM_HALF);
 // The 3-D map {K, N, G} of a K-major operand W[G][N][K] bf16 (row stride k_ld, group
 // stride g_ld elements, multiples of 8), box {64, box_n, 1}.
 bool make_kmajor_tmap(CUtensorMap* tm, const void* base, int64_t K, int64_t N, int64_t G, int64_t k_ld,
