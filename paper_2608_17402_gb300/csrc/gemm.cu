@@ -944,7 +944,6 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
             __syncwarp();
             if (lane == 0) mbar_arrive_remote(tempty_leader + 8 * acc);
         }
-        float dg_acc = 0.f;   // EPI_DGELU_BF16: this thread's share of its row's dot
         for (int ch = half; ch < nchunk; ch += 2) {
             const int c0 = ch * 32;
             if constexpr (ECLS == ECLS_ADD) {   // staged reductions
@@ -973,67 +972,6 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
             const int n = t.n0 + c0;
             if constexpr (!to_f32) {
                 __nv_bfloat16* orow = p.out + (int64_t)gr * p.ldo + n;
-                if (TRAIN && p.epi == EPI_DSWIGLU_BF16) {   // SwiGLU: du, dv and the dot acc . a
-                    const __nv_bfloat16* urow = p.epi_u + (int64_t)gr * p.ldo + n;
-                    const __nv_bfloat16* vrow = p.epi_v + (int64_t)gr * p.ldo + n;
-                    const __nv_bfloat16* arow = p.epi_a + (int64_t)gr * p.ldo + n;
-#pragma unroll
-                    for (int g8 = 0; g8 < 4; ++g8) {
-                        if (n + 8 * g8 >= p.N) break;
-                        float uf[8], vf[8], af[8], fu[8], fv[8];
-                        unpack_bf16x8(*reinterpret_cast<const uint4*>(urow + 8 * g8), uf);
-                        unpack_bf16x8(*reinterpret_cast<const uint4*>(vrow + 8 * g8), vf);
-                        unpack_bf16x8(*reinterpret_cast<const uint4*>(arow + 8 * g8), af);
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const float a = __uint_as_float(v[8 * g8 + i]);
-                            const bool in = n + 8 * g8 + i < p.N;   // columns past N: padding
-                            dg_acc += in ? a * af[i] : 0.f;
-                            const float sg = __fdividef(1.0f, 1.0f + __expf(-uf[i]));   // SiLU(u) = u sg
-                            fu[i] = in ? sc * a * vf[i] * sg * (1.0f + uf[i] * (1.0f - sg)) : 0.f;
-                            fv[i] = in ? sc * a * uf[i] * sg : 0.f;
-                        }
-                        uint4 u, w;
-                        u.x = pack_bf16x2(fu[0], fu[1]);
-                        u.y = pack_bf16x2(fu[2], fu[3]);
-                        u.z = pack_bf16x2(fu[4], fu[5]);
-                        u.w = pack_bf16x2(fu[6], fu[7]);
-                        w.x = pack_bf16x2(fv[0], fv[1]);
-                        w.y = pack_bf16x2(fv[2], fv[3]);
-                        w.z = pack_bf16x2(fv[4], fv[5]);
-                        w.w = pack_bf16x2(fv[6], fv[7]);
-                        *reinterpret_cast<uint4*>(orow + 8 * g8) = u;
-                        *reinterpret_cast<uint4*>(p.out2 + (int64_t)gr * p.ldo + n + 8 * g8) = w;
-                    }
-                    continue;
-                }
-                if (TRAIN && p.epi == EPI_DGELU_BF16) {   // training path: du = scale acc GELU'(u), dot acc . a
-                    const __nv_bfloat16* urow = p.epi_u + (int64_t)gr * p.ldo + n;
-                    const __nv_bfloat16* arow = p.epi_a + (int64_t)gr * p.ldo + n;
-#pragma unroll
-                    for (int g8 = 0; g8 < 4; ++g8) {
-                        if (n + 8 * g8 >= p.N) break;
-                        float uf[8], af[8], f[8];
-                        unpack_bf16x8(*reinterpret_cast<const uint4*>(urow + 8 * g8), uf);
-                        unpack_bf16x8(*reinterpret_cast<const uint4*>(arow + 8 * g8), af);
-#pragma unroll
-                        for (int i = 0; i < 8; i += 2) gelu_grad2(uf[i], uf[i + 1]);   // GELU'(u)
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const float a = __uint_as_float(v[8 * g8 + i]);
-                            const bool in = n + 8 * g8 + i < p.N;   // columns past N: padding
-                            dg_acc += in ? a * af[i] : 0.f;
-                            f[i] = in ? sc * a * uf[i] : 0.f;
-                        }
-                        uint4 u;
-                        u.x = pack_bf16x2(f[0], f[1]);
-                        u.y = pack_bf16x2(f[2], f[3]);
-                        u.z = pack_bf16x2(f[4], f[5]);
-                        u.w = pack_bf16x2(f[6], f[7]);
-                        *reinterpret_cast<uint4*>(orow + 8 * g8) = u;
-                    }
-                    continue;
-                }
 #pragma unroll
                 for (int g8 = 0; g8 < 4; ++g8) {
                     if (n + 8 * g8 >= p.N) break;
@@ -1070,10 +1008,144 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
                 }
             }
         }
-        if (TRAIN && !to_f32 && (p.epi == EPI_DGELU_BF16 || p.epi == EPI_DSWIGLU_BF16) && ok_row &&
-            p.dg_part)   // row dot (the gates' gradient; none for the shared expert)
-            p.dg_part[(int64_t)(2 * (t.n0 / p.n_step) + half) * p.m_total + gr] = dg_acc;
     }
+}
+
+// Epilogue of the activation derivatives (EPI_DGELU_BF16, EPI_DSWIGLU_BF16): each thread takes
+// its own row, 16 columns at a time: du = scale acc GELU'(u) (SwiGLU: du = scale acc v
+// SiLU'(u), dv = scale acc SiLU(u)) and the row dot acc . a.  What bounds it is the latency of
+// the u, v and a rows (64 KB a tile each), so they come through a double buffer in shared
+// memory, whole 32-byte sectors by cp.async one 16-column step ahead, also across tiles.
+// At T = 8192, d = 1024, E = 31, k = 3, h = 684 (SwiGLU) the launch took 236 us with each
+// thread loading its row's 16-byte pieces as it needed them, 156 us with the pieces one step
+// ahead in registers (which spilled), and 75 us this way.
+template <bool SWIGLU>
+__device__ void epilogue_dact(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64_t n_work,
+                              volatile int* abort_flag) {
+    constexpr int NARR = SWIGLU ? 3 : 2;   // u, a (, v)
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int quad = warp & 3, half = warp >> 2;
+    const int nchunk = p.BN / 32;
+    const int nsub = half < nchunk ? (nchunk - half + 1) / 2 * 2 : 0;   // 16-column steps of this warp
+    const uint32_t tempty_leader = peer_addr(sm.tempty, 0);
+    // this warp's buffer: 2 slots x NARR arrays x 32 rows x 32 bytes; 16-byte piece q of row r
+    // at r * 32 + 16 (q ^ (r / 4 & 1)), so that eight consecutive rows' pieces hit all banks
+    uint8_t* buf = reinterpret_cast<uint8_t*>(sm.stg) + warp * (2 * NARR * 1024);
+    const uint32_t buf_a = smem_u32(buf);
+    if (sm.pair >= n_work) return;
+    auto col_of = [&](int k) { return (half + 2 * (k >> 1)) * 32 + (k & 1) * 16; };
+    // step k of tile tt into slot `slot`: lane l copies piece l & 1 of rows l / 2 and l / 2 + 16
+    auto fetch = [&](const Tile& tt, int k, int slot) {
+        const int q = lane & 1;
+        const int n = tt.n0 + col_of(k) + 8 * q;
+        const int nh = rows_half(tt, sm.rank);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int r = (lane >> 1) + 16 * i;
+            const bool ok = quad * 32 + r < nh && n < p.N;
+            const int64_t off = ok ? (int64_t)(tt.row0 + (int)sm.rank * GM_HALF + quad * 32 + r) * p.ldo + n : 0;
+            const uint32_t dst = buf_a + slot * (NARR * 1024) + r * 32 + 16 * (q ^ ((r >> 2) & 1));
+            cp_async16(dst, p.epi_u + off, ok ? 16u : 0u);
+            cp_async16(dst + 1024, p.epi_a + off, ok ? 16u : 0u);
+            if (SWIGLU) cp_async16(dst + 2048, p.epi_v + off, ok ? 16u : 0u);
+        }
+    };
+    const TileLd l0 = tile_load(p, sm.pair);
+    TileLd nl = tile_load(p, sm.pair + sm.npairs < n_work ? sm.pair + sm.npairs : sm.pair);
+    Tile t = tile_finish(p, l0);
+    if (nsub > 0) fetch(t, 0, 0);
+    cp_async_commit();
+    int it = 0;
+    for (int64_t w = sm.pair; w < n_work; w += sm.npairs, ++it) {
+        const Tile tn = tile_finish(p, nl);   // (past the last item: the last one again)
+        const int64_t w2 = w + 2 * sm.npairs;
+        nl = tile_load(p, w2 < n_work ? w2 : w);
+        const int acc = it & 1;
+        const int myrow = quad * 32 + lane;
+        const int gr = t.row0 + (int)sm.rank * GM_HALF + myrow;
+        const bool ok_row = myrow < rows_half(t, sm.rank);
+        const float sc = p.row_scale ? __ldg(p.row_scale + (ok_row ? gr : 0)) : p.scale;
+        const int64_t row = (int64_t)(ok_row ? gr : 0) * p.ldo;
+        if (!mbar_wait(sm.tfull + 8 * acc, (uint32_t)(it >> 1) & 1u, p.limit_ns, abort_flag)) {
+            set_abort(abort_flag, p.status, SITE_GEMM_WAIT_TFULL, (int)sm.pair, it);
+            cp_async_wait_all();
+            return;
+        }
+        tc_fence_after();
+        const uint32_t tbase = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)acc * GM_MAXBN;
+        if (nsub == 0) {   // no columns for this warp in this tile
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_remote(tempty_leader + 8 * acc);
+        }
+        float dg_acc = 0.f;   // this thread's share of its row's dot
+        for (int k = 0; k < nsub; ++k) {   // nsub is even: step k of every tile uses slot k & 1
+            __syncwarp();   // every lane has read the slot that is filled next
+            if (k + 1 < nsub) fetch(t, k + 1, (k + 1) & 1);
+            else fetch(tn, 0, 0);
+            cp_async_commit();
+            uint32_t x[16];
+            tmem_ld_32x32b_x16(tbase + col_of(k), x);
+            cp_async_wait<1>();
+            tmem_wait_ld();
+            __syncwarp();   // step k's pieces, copied by all lanes
+            if (k + 1 == nsub) {   // this warp's last read of the accumulator
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_remote(tempty_leader + 8 * acc);
+            }
+            if (!ok_row) continue;
+            const int n = t.n0 + col_of(k);
+            const uint8_t* in = buf + (k & 1) * (NARR * 1024) + lane * 32;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if (n + 8 * q >= p.N) break;
+                const uint8_t* piece = in + 16 * (q ^ ((lane >> 2) & 1));
+                float uf[8], af[8], fu[8];
+                unpack_bf16x8(*reinterpret_cast<const uint4*>(piece), uf);
+                unpack_bf16x8(*reinterpret_cast<const uint4*>(piece + 1024), af);
+                if constexpr (SWIGLU) {
+                    float vf[8], fv[8];
+                    unpack_bf16x8(*reinterpret_cast<const uint4*>(piece + 2048), vf);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float a = __uint_as_float(x[8 * q + i]);
+                        const bool ok = n + 8 * q + i < p.N;   // columns past N: padding
+                        dg_acc += ok ? a * af[i] : 0.f;
+                        const float sg = __fdividef(1.0f, 1.0f + __expf(-uf[i]));   // SiLU(u) = u sg
+                        fu[i] = ok ? sc * a * vf[i] * sg * (1.0f + uf[i] * (1.0f - sg)) : 0.f;
+                        fv[i] = ok ? sc * a * uf[i] * sg : 0.f;
+                    }
+                    uint4 o;
+                    o.x = pack_bf16x2(fv[0], fv[1]);
+                    o.y = pack_bf16x2(fv[2], fv[3]);
+                    o.z = pack_bf16x2(fv[4], fv[5]);
+                    o.w = pack_bf16x2(fv[6], fv[7]);
+                    *reinterpret_cast<uint4*>(p.out2 + row + n + 8 * q) = o;
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; i += 2) gelu_grad2(uf[i], uf[i + 1]);   // GELU'(u)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const float a = __uint_as_float(x[8 * q + i]);
+                        const bool ok = n + 8 * q + i < p.N;   // columns past N: padding
+                        dg_acc += ok ? a * af[i] : 0.f;
+                        fu[i] = ok ? sc * a * uf[i] : 0.f;
+                    }
+                }
+                uint4 o;
+                o.x = pack_bf16x2(fu[0], fu[1]);
+                o.y = pack_bf16x2(fu[2], fu[3]);
+                o.z = pack_bf16x2(fu[4], fu[5]);
+                o.w = pack_bf16x2(fu[6], fu[7]);
+                *reinterpret_cast<uint4*>(p.out + row + n + 8 * q) = o;
+            }
+        }
+        if (ok_row && p.dg_part)   // row dot (the gates' gradient; none for the shared expert)
+            p.dg_part[(int64_t)(2 * (t.n0 / p.n_step) + half) * p.m_total + gr] = dg_acc;
+        t = tn;
+    }
+    cp_async_wait_all();
 }
 
 template <bool GATHER, int ECLS, bool TRAIN>
@@ -1153,6 +1225,8 @@ __global__ void __launch_bounds__(GM_THREADS, 1) grouped_gemm_kernel(const __gri
 
     if (warp < GM_EPI_WARPS || (ECLS == ECLS_ADDT && warp >= GM_WARP_GATHER && warp < GM_WARP_FWD)) {
         if constexpr (ECLS == ECLS_ADDT) epilogue_addt<TRAIN>(p, sm, tmem, n_work, warp, abort_flag);
+        else if constexpr (ECLS == ECLS_DGELU) epilogue_dact<false>(p, sm, tmem, n_work, abort_flag);
+        else if constexpr (ECLS == ECLS_DSWIGLU) epilogue_dact<true>(p, sm, tmem, n_work, abort_flag);
         else epilogue<GATHER, ECLS, TRAIN>(p, sm, tmem, n_work, abort_flag);
     } else if (warp == GM_WARP_MMA) {
         if (sm.rank == 0) mma_issuer<TRAIN, ECLS == ECLS_F32, ECLS == ECLS_ADDT>(p, sm, tmem, n_work, abort_flag);
@@ -1307,7 +1381,7 @@ cudaError_t launch_grouped_gemm(const GemmArgs& a, int grid, cudaStream_t s) {
         Kern kern;
         int ecls;
     };
-    static const Inst insts[8] = {
+    static const Inst insts[10] = {
         {grouped_gemm_kernel<false, ECLS_ADDT, false>, ECLS_ADDT},
         {grouped_gemm_kernel<false, ECLS_F32, false>, ECLS_F32},
         {grouped_gemm_kernel<false, ECLS_BF16, false>, ECLS_BF16},
@@ -1316,7 +1390,9 @@ cudaError_t launch_grouped_gemm(const GemmArgs& a, int grid, cudaStream_t s) {
         {grouped_gemm_kernel<true, ECLS_BF16, true>, ECLS_BF16},
         {grouped_gemm_kernel<false, ECLS_ADDT, true>, ECLS_ADDT},
         {grouped_gemm_kernel<false, ECLS_ADD, true>, ECLS_ADD},
-        {grouped_gemm_kernel<false, ECLS_ADD, false>, ECLS_ADD}};
+        {grouped_gemm_kernel<false, ECLS_ADD, false>, ECLS_ADD},
+        {grouped_gemm_kernel<true, ECLS_DGELU, true>, ECLS_DGELU},
+        {grouped_gemm_kernel<true, ECLS_DSWIGLU, true>, ECLS_DSWIGLU}};
     const bool gathered = a.a_rows || a.a_ident;   // A rows through the gather warps
     const bool train = a.b_kmajor || a.a_mn || a.item_table == 2 || a.epi == EPI_GELU2_BF16 ||
                        a.epi == EPI_DGELU_BF16 || a.epi == EPI_DSWIGLU_BF16 || a.out2 != nullptr;
@@ -1327,7 +1403,7 @@ cudaError_t launch_grouped_gemm(const GemmArgs& a, int grid, cudaStream_t s) {
     if (a.trans && (a.epi != EPI_ADD_F32 || a.item_table)) return cudaErrorInvalidValue;
     int which;
     if (a.trans) which = train ? 5 : 0;
-    else if (train && gathered) which = 4;
+    else if (train && gathered) which = a.epi == EPI_DGELU_BF16 ? 8 : a.epi == EPI_DSWIGLU_BF16 ? 9 : 4;
     else if (a.epi == EPI_ADD_F32) which = train ? 6 : 7;
     else if (train) return cudaErrorInvalidValue;
     else if (gathered) which = 3;

@@ -176,26 +176,31 @@ constexpr int GM_OVERHEAD_BYTES = 1024 + 512;   // alignment, barriers / TMEM sl
 // Epilogue classes of the grouped GEMM's kernel instances: bf16 outputs (GELU, SwiGLU,
 // plain), fp32 stores (plain, two-group sums), staged fp32 reductions (weight-gradient
 // tiles, which also store, and band-ordered rows), and fp32 reductions of rows into their
-// tokens' rows by the transposed product.
-enum { ECLS_BF16 = 0, ECLS_F32 = 1, ECLS_ADD = 2, ECLS_ADDT = 3 };
+// tokens' rows by the transposed product, and the activation derivatives of the training
+// path.
+enum { ECLS_BF16 = 0, ECLS_F32 = 1, ECLS_ADD = 2, ECLS_ADDT = 3, ECLS_DGELU = 4, ECLS_DSWIGLU = 5 };
 // Epilogue warps per TMEM lane quadrant of ECLS_ADDT: two epilogue warps and two of the
 // (idle) gather warps, each taking every fourth chunk of 32 rows.
 constexpr int GM_ADDT_PARTS = 4;
 static_assert(4 * GM_ADDT_PARTS == GM_EPI_WARPS + GM_GATHER_WARPS, "the gather warps join the epilogue");
 // Shared memory beside the operand ring: ECLS_ADD stages 16 rows per warp, ECLS_ADDT keeps
-// the {token, scale} pairs of 32 rows per warp; both give up one of the 7 stages.
+// the {token, scale} pairs of 32 rows per warp; both give up one of the 7 stages.  The
+// activation derivatives buffer two 16-column steps of u, a (and v) per warp, two stages.
 __host__ __device__ constexpr int gm_stg_bytes(int ecls) {
     return ecls == ECLS_ADD ? GM_EPI_WARPS * GM_STG_ROWS * GM_STG_LD * 4
-           : ecls == ECLS_ADDT ? 4 * GM_ADDT_PARTS * 32 * 8 : 0;
+           : ecls == ECLS_ADDT ? 4 * GM_ADDT_PARTS * 32 * 8
+           : ecls == ECLS_DGELU ? GM_EPI_WARPS * 2 * 2 * 1024
+           : ecls == ECLS_DSWIGLU ? GM_EPI_WARPS * 2 * 3 * 1024 : 0;
 }
 __host__ __device__ constexpr int gm_stages(int ecls) {
-    return ecls == ECLS_ADD || ecls == ECLS_ADDT ? 6 : 7;
+    return ecls == ECLS_DGELU || ecls == ECLS_DSWIGLU ? 5 : ecls == ECLS_ADD || ecls == ECLS_ADDT ? 6 : 7;
 }
 __host__ __device__ constexpr int gm_smem_bytes(int ecls) {
     return gm_stages(ecls) * (GM_A_BYTES + GM_B_BYTES) + gm_stg_bytes(ecls) + GM_OVERHEAD_BYTES;
 }
 static_assert(gm_smem_bytes(ECLS_BF16) <= 232448 && gm_smem_bytes(ECLS_ADD) <= 232448 &&
-                  gm_smem_bytes(ECLS_ADDT) <= 232448,
+                  gm_smem_bytes(ECLS_ADDT) <= 232448 && gm_smem_bytes(ECLS_DGELU) <= 232448 &&
+                  gm_smem_bytes(ECLS_DSWIGLU) <= 232448,
               "shared memory of one CTA");
 static_assert(3 * GM_STAGES_MAX + 5 <= 32, "barriers fit before the signal sink at +256 bytes");
 // The transposed product reads the GEMM rows through boxes of 32 rows, as many as its
