@@ -802,22 +802,19 @@ __device__ void epilogue_addt(const GemmArgs& p, const Smem& sm, uint32_t tmem, 
     }
 }
 
-// Warp w reads TMEM lanes 32 (w % 4) .. +31 (its rows) and the 32-column chunks
-// c = w / 4, w / 4 + 2, ... of each tile.  bf16 outputs and fp32 stores: each thread
+// Epilogue of the fp32 outputs.  Warp w reads TMEM lanes 32 (w % 4) .. +31 (its rows) and
+// the 32-column chunks c = w / 4, w / 4 + 2, ... of each tile.  fp32 stores: each thread
 // takes its own row (32x32b loads) and writes it straight from registers with
-// 16-byte stores.  fp32 reductions (the y accumulator): the rows pass a small
+// 16-byte stores.  fp32 reductions: the rows pass a small
 // per-warp staging buffer so that each 16-byte vector reduction instruction of a
 // warp covers four rows x 128 contiguous bytes, i.e. whole L2 lines.  When a warp has read
 // its last chunk of the accumulator it arrives (once) on the leader's tempty barrier.
-template <bool GATHER, int ECLS, bool TRAIN>
+template <int ECLS, bool TRAIN>
 __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64_t n_work,
                          volatile int* abort_flag) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int quad = warp & 3, half = warp >> 2;
-    constexpr bool to_f32 = ECLS != ECLS_BF16;
     const int nchunk = p.BN / 32;
-    // bf16 results are written once and read back later: let them leave L2 first
-    const uint64_t stream_pol = l2_policy_evict_first();
     const uint32_t tempty_leader = peer_addr(sm.tempty, 0);
     int it = 0;
     if (sm.pair >= n_work) return;
@@ -835,7 +832,7 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
         if (ok_row) {
             if (p.o_rows) tok = __ldg(p.o_rows + gr) / p.o_div;
             if (p.row_scale) sc = __ldg(p.row_scale + gr);
-            if (to_f32 && (tok < 0 || tok >= p.o_nrows)) {
+            if (tok < 0 || tok >= p.o_nrows) {
                 if (!(p.o_neg_skip && tok < 0))   // a padding row writes nothing
                     report(p.status, MOEVIE_ERR_DEVICE, SITE_GEMM_OUT_ROW, gr, (int)tok);
                 ok_row = false;
@@ -881,64 +878,6 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
             }
             continue;
         }
-        if (GATHER && ECLS == ECLS_BF16 && p.epi == EPI_SWIGLU_BF16) {   // (gathered A only)
-            // output chunk ch (32 columns): gate = accumulator chunk ch, up = chunk ch + nout
-            const int nout = nchunk / 2;
-            if (half >= nout) {
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_remote(tempty_leader + 8 * acc);
-            }
-            for (int ch = half; ch < nout; ch += 2) {
-                uint32_t v[32];
-                float gt[32];
-                tmem_ld_32x32b_x32(tbase + ch * 32, v);
-                tmem_wait_ld();
-#pragma unroll
-                for (int i = 0; i < 32; ++i) gt[i] = __uint_as_float(v[i]);
-                tmem_ld_32x32b_x32(tbase + (ch + nout) * 32, v);
-                tmem_wait_ld();
-                if (ch + 2 >= nout) {   // this warp's last read of the accumulator
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive_remote(tempty_leader + 8 * acc);
-                }
-                if (!ok_row) continue;
-                const int n = t.n0 + ch * 32;
-                __nv_bfloat16* orow = p.out + (int64_t)gr * p.ldo + n;
-#pragma unroll
-                for (int g8 = 0; g8 < 4; ++g8) {
-                    if (n + 8 * g8 >= p.N) break;
-                    float f[8];
-                    if (TRAIN && p.out2) {   // the training path keeps u and v as well
-                        uint4 uu, vv;
-                        uu.x = pack_bf16x2(gt[8 * g8 + 0], gt[8 * g8 + 1]);
-                        uu.y = pack_bf16x2(gt[8 * g8 + 2], gt[8 * g8 + 3]);
-                        uu.z = pack_bf16x2(gt[8 * g8 + 4], gt[8 * g8 + 5]);
-                        uu.w = pack_bf16x2(gt[8 * g8 + 6], gt[8 * g8 + 7]);
-                        vv.x = pack_bf16x2(__uint_as_float(v[8 * g8 + 0]), __uint_as_float(v[8 * g8 + 1]));
-                        vv.y = pack_bf16x2(__uint_as_float(v[8 * g8 + 2]), __uint_as_float(v[8 * g8 + 3]));
-                        vv.z = pack_bf16x2(__uint_as_float(v[8 * g8 + 4]), __uint_as_float(v[8 * g8 + 5]));
-                        vv.w = pack_bf16x2(__uint_as_float(v[8 * g8 + 6]), __uint_as_float(v[8 * g8 + 7]));
-                        *reinterpret_cast<uint4*>(p.out2 + (int64_t)gr * p.ldo + n + 8 * g8) = uu;
-                        *reinterpret_cast<uint4*>(p.out3 + (int64_t)gr * p.ldo + n + 8 * g8) = vv;
-                    }
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        // SiLU(g) u = g u / (1 + e^-g); e^-g = inf for g far below 0 gives 0
-                        const float g = gt[8 * g8 + i];
-                        f[i] = __fdividef(g, 1.0f + __expf(-g)) * __uint_as_float(v[8 * g8 + i]);
-                    }
-                    uint4 u;
-                    u.x = pack_bf16x2(f[0], f[1]);
-                    u.y = pack_bf16x2(f[2], f[3]);
-                    u.z = pack_bf16x2(f[4], f[5]);
-                    u.w = pack_bf16x2(f[6], f[7]);
-                    st_global_v4_hint(orow + 8 * g8, u, stream_pol);
-                }
-            }
-            continue;
-        }
         if (half >= nchunk) {   // no columns for this warp in this tile
             tc_fence_before();
             __syncwarp();
@@ -970,34 +909,7 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
             }
             if (!ok_row) continue;
             const int n = t.n0 + c0;
-            if constexpr (!to_f32) {
-                __nv_bfloat16* orow = p.out + (int64_t)gr * p.ldo + n;
-#pragma unroll
-                for (int g8 = 0; g8 < 4; ++g8) {
-                    if (n + 8 * g8 >= p.N) break;
-                    float f[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(v[8 * g8 + i]);
-                    if (TRAIN && p.epi == EPI_GELU2_BF16) {   // the pre-activation as well
-                        uint4 u;
-                        u.x = pack_bf16x2(f[0], f[1]);
-                        u.y = pack_bf16x2(f[2], f[3]);
-                        u.z = pack_bf16x2(f[4], f[5]);
-                        u.w = pack_bf16x2(f[6], f[7]);
-                        *reinterpret_cast<uint4*>(p.out2 + (int64_t)gr * p.ldo + n + 8 * g8) = u;
-                    }
-                    if (p.epi == EPI_GELU_BF16 || (TRAIN && p.epi == EPI_GELU2_BF16)) {
-#pragma unroll
-                        for (int i = 0; i < 8; i += 2) gelu_erf2(f[i], f[i + 1]);
-                    }
-                    uint4 u;
-                    u.x = pack_bf16x2(f[0], f[1]);
-                    u.y = pack_bf16x2(f[2], f[3]);
-                    u.z = pack_bf16x2(f[4], f[5]);
-                    u.w = pack_bf16x2(f[6], f[7]);
-                    st_global_v4_hint(orow + 8 * g8, u, stream_pol);
-                }
-            } else {
+            {
                 float* yrow = p.yacc + t.ks * p.y_split_stride + tok * p.ldy + n;
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
@@ -1006,6 +918,118 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
                         make_float4(sc * __uint_as_float(v[4 * q]), sc * __uint_as_float(v[4 * q + 1]),
                                     sc * __uint_as_float(v[4 * q + 2]), sc * __uint_as_float(v[4 * q + 3]));
                 }
+            }
+        }
+    }
+}
+
+// Epilogue of the bf16 outputs (GELU, SwiGLU, plain; the training path's also keep the
+// pre-activations).  Warp w reads TMEM lanes 32 (w % 4) .. +31 (its rows); each thread forms
+// 32 (training path 16) columns of its own row at a time, and the warp's 32 rows pass a buffer in shared
+// memory, from which whole sectors are stored, 64 (training path 32) bytes of a row by
+// neighbouring lanes.  Stored by each thread straight from its registers they left as
+// 16-byte pieces of 32 different lines an instruction; staged, for one stage of the operand
+// ring: up-projection T = 65536, d = 1664, E = 256 612 -> 593 us, T = 32768, E = 128 287 -> 268,
+// T = 8192, d = 1280, h = 854 (SwiGLU) 208 -> 203, T = 8192, d = 1024, E = 64 unchanged (84).
+template <bool TRAIN>
+__device__ void epilogue_bf16(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64_t n_work,
+                              volatile int* abort_flag) {
+    constexpr int COLS = TRAIN ? 16 : 32, NP = COLS / 8;   // columns a step, 16-byte pieces of a row
+    constexpr int ARR = 32 * COLS * 2;                     // bytes of one array's step
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int quad = warp & 3, half = warp >> 2;
+    const int nchunk = p.swiglu ? p.BN / 64 : p.BN / 32;   // 32-column chunks of the output
+    const int up0 = p.swiglu ? p.BN / 2 : 0;               // SwiGLU: first accumulator column of the up projection
+    // bf16 results are written once and read back later: let them leave L2 first
+    const uint64_t stream_pol = l2_policy_evict_first();
+    const uint32_t tempty_leader = peer_addr(sm.tempty, 0);
+    uint8_t* buf = reinterpret_cast<uint8_t*>(sm.stg) + warp * gm_bf16_warp_bytes(TRAIN);
+    // piece q of row r at r * 2 COLS + 16 (q ^ swizzle(r)): eight consecutive rows' pieces (the
+    // threads' writes) and eight consecutive pieces (the copies out) hit all banks
+    auto place = [](int r, int q) { return r * (2 * COLS) + 16 * (q ^ (NP == 4 ? (r >> 1) & 3 : (r >> 2) & 1)); };
+    if (sm.pair >= n_work) return;
+    TileLd nl = tile_load(p, sm.pair);   // one item ahead
+    int it = 0;
+    for (int64_t w = sm.pair; w < n_work; w += sm.npairs, ++it) {
+        const Tile t = tile_finish(p, nl);
+        nl = tile_load(p, w + sm.npairs < n_work ? w + sm.npairs : w);
+        const int acc = it & 1;
+        const int nrow = rows_half(t, sm.rank) - quad * 32;   // rows of this warp (may be < 1 or > 32)
+        const int64_t row0 = t.row0 + (int64_t)sm.rank * GM_HALF + quad * 32;
+        if (!mbar_wait(sm.tfull + 8 * acc, (uint32_t)(it >> 1) & 1u, p.limit_ns, abort_flag)) {
+            set_abort(abort_flag, p.status, SITE_GEMM_WAIT_TFULL, (int)sm.pair, it);
+            return;
+        }
+        tc_fence_after();
+        const uint32_t tbase = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)acc * GM_MAXBN;
+        if (half >= nchunk) {   // no columns for this warp in this tile
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_remote(tempty_leader + 8 * acc);
+        }
+        for (int ch = half; ch < nchunk; ch += 2) {
+#pragma unroll
+            for (int c0 = 0; c0 < 32; c0 += COLS) {
+                const int c = ch * 32 + c0;
+#pragma unroll
+                for (int s0 = 0; s0 < COLS; s0 += 16) {
+                    uint32_t x[16], y[16];
+                    tmem_ld_32x32b_x16(tbase + c + s0, x);
+                    if (p.swiglu) tmem_ld_32x32b_x16(tbase + up0 + c + s0, y);
+                    tmem_wait_ld();
+                    if (ch + 2 >= nchunk && c0 + s0 + 16 == 32) {   // this warp's last read of the accumulator
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive_remote(tempty_leader + 8 * acc);
+                    }
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        float f[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(x[8 * q + i]);
+                        const int at = place(lane, s0 / 8 + q);
+                        auto put = [&](int arr, const float (&o)[8]) {
+                            uint4 u;
+                            u.x = pack_bf16x2(o[0], o[1]);
+                            u.y = pack_bf16x2(o[2], o[3]);
+                            u.z = pack_bf16x2(o[4], o[5]);
+                            u.w = pack_bf16x2(o[6], o[7]);
+                            *reinterpret_cast<uint4*>(buf + arr * ARR + at) = u;
+                        };
+                        if (TRAIN && p.out2) put(1, f);   // the pre-activation (SwiGLU: the gate's) as well
+                        if (p.swiglu) {
+                            float g[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) g[i] = __uint_as_float(y[8 * q + i]);
+                            if (TRAIN && p.out2) put(2, g);
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                // SiLU(u) v = u v / (1 + e^-u); e^-u = inf for u far below 0 gives 0
+                                f[i] = __fdividef(f[i], 1.0f + __expf(-f[i])) * g[i];
+                        } else if (p.epi == EPI_GELU_BF16 || (TRAIN && p.epi == EPI_GELU2_BF16)) {
+#pragma unroll
+                            for (int i = 0; i < 8; i += 2) gelu_erf2(f[i], f[i + 1]);
+                        }
+                        put(0, f);
+                    }
+                }
+                __syncwarp();   // the step's rows, written by all lanes
+                const int n = t.n0 + c;
+#pragma unroll
+                for (int i = 0; i < NP; ++i) {
+                    const int r = (lane + 32 * i) / NP, q = (lane + 32 * i) % NP;
+                    if (r < nrow && n + 8 * q < p.N) {
+                        const int64_t off = (row0 + r) * p.ldo + n + 8 * q;
+                        const uint8_t* from = buf + place(r, q);
+                        st_global_v4_hint(p.out + off, *reinterpret_cast<const uint4*>(from), stream_pol);
+                        if (TRAIN && p.out2) {
+                            *reinterpret_cast<uint4*>(p.out2 + off) = *reinterpret_cast<const uint4*>(from + ARR);
+                            if (p.swiglu)
+                                *reinterpret_cast<uint4*>(p.out3 + off) = *reinterpret_cast<const uint4*>(from + 2 * ARR);
+                        }
+                    }
+                }
+                __syncwarp();   // copied out before the next step overwrites it
             }
         }
     }
@@ -1154,10 +1178,10 @@ __global__ void __launch_bounds__(GM_THREADS, 1) grouped_gemm_kernel(const __gri
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(gm_smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint8_t* sA = smem;
-    constexpr int nst = gm_stages(ECLS);
+    constexpr int nst = gm_stages(ECLS, TRAIN);
     uint8_t* sB = smem + nst * GM_A_BYTES;
     uint8_t* sStg = sB + nst * GM_B_BYTES;                       // epilogue staging
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sStg + gm_stg_bytes(ECLS));
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sStg + gm_stg_bytes(ECLS, TRAIN));
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * GM_STAGES_MAX + 5);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     uint8_t* sink = reinterpret_cast<uint8_t*>(bars) + 256;   // 16-byte aligned, after the barriers
@@ -1227,7 +1251,8 @@ __global__ void __launch_bounds__(GM_THREADS, 1) grouped_gemm_kernel(const __gri
         if constexpr (ECLS == ECLS_ADDT) epilogue_addt<TRAIN>(p, sm, tmem, n_work, warp, abort_flag);
         else if constexpr (ECLS == ECLS_DGELU) epilogue_dact<false>(p, sm, tmem, n_work, abort_flag);
         else if constexpr (ECLS == ECLS_DSWIGLU) epilogue_dact<true>(p, sm, tmem, n_work, abort_flag);
-        else epilogue<GATHER, ECLS, TRAIN>(p, sm, tmem, n_work, abort_flag);
+        else if constexpr (ECLS == ECLS_BF16) epilogue_bf16<TRAIN>(p, sm, tmem, n_work, abort_flag);
+        else epilogue<ECLS, TRAIN>(p, sm, tmem, n_work, abort_flag);
     } else if (warp == GM_WARP_MMA) {
         if (sm.rank == 0) mma_issuer<TRAIN, ECLS == ECLS_F32, ECLS == ECLS_ADDT>(p, sm, tmem, n_work, abort_flag);
     } else if (prod_id >= 0) {
@@ -1380,6 +1405,7 @@ cudaError_t launch_grouped_gemm(const GemmArgs& a, int grid, cudaStream_t s) {
     struct Inst {
         Kern kern;
         int ecls;
+        bool train = false;
     };
     static const Inst insts[10] = {
         {grouped_gemm_kernel<false, ECLS_ADDT, false>, ECLS_ADDT},
@@ -1387,12 +1413,12 @@ cudaError_t launch_grouped_gemm(const GemmArgs& a, int grid, cudaStream_t s) {
         {grouped_gemm_kernel<false, ECLS_BF16, false>, ECLS_BF16},
         {grouped_gemm_kernel<true, ECLS_BF16, false>, ECLS_BF16},
         // the training path: K-major weights, M-major A, weight-gradient items, backward epilogues
-        {grouped_gemm_kernel<true, ECLS_BF16, true>, ECLS_BF16},
-        {grouped_gemm_kernel<false, ECLS_ADDT, true>, ECLS_ADDT},
-        {grouped_gemm_kernel<false, ECLS_ADD, true>, ECLS_ADD},
+        {grouped_gemm_kernel<true, ECLS_BF16, true>, ECLS_BF16, true},
+        {grouped_gemm_kernel<false, ECLS_ADDT, true>, ECLS_ADDT, true},
+        {grouped_gemm_kernel<false, ECLS_ADD, true>, ECLS_ADD, true},
         {grouped_gemm_kernel<false, ECLS_ADD, false>, ECLS_ADD},
-        {grouped_gemm_kernel<true, ECLS_DGELU, true>, ECLS_DGELU},
-        {grouped_gemm_kernel<true, ECLS_DSWIGLU, true>, ECLS_DSWIGLU}};
+        {grouped_gemm_kernel<true, ECLS_DGELU, true>, ECLS_DGELU, true},
+        {grouped_gemm_kernel<true, ECLS_DSWIGLU, true>, ECLS_DSWIGLU, true}};
     const bool gathered = a.a_rows || a.a_ident;   // A rows through the gather warps
     const bool train = a.b_kmajor || a.a_mn || a.item_table == 2 || a.epi == EPI_GELU2_BF16 ||
                        a.epi == EPI_DGELU_BF16 || a.epi == EPI_DSWIGLU_BF16 || a.out2 != nullptr;
@@ -1414,7 +1440,7 @@ cudaError_t launch_grouped_gemm(const GemmArgs& a, int grid, cudaStream_t s) {
     if (dev >= 0 && dev < 64 && !attr_set[dev]) {
         for (const Inst& k : insts) {
             cudaError_t e = cudaFuncSetAttribute(k.kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 gm_smem_bytes(k.ecls));
+                                                 gm_smem_bytes(k.ecls, k.train));
             if (e != cudaSuccess) return e;
         }
         attr_set[dev] = true;
@@ -1422,7 +1448,7 @@ cudaError_t launch_grouped_gemm(const GemmArgs& a, int grid, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((grid + 1) & ~1));   // whole pairs
     cfg.blockDim = dim3(GM_THREADS);
-    cfg.dynamicSmemBytes = gm_smem_bytes(insts[which].ecls);
+    cfg.dynamicSmemBytes = gm_smem_bytes(insts[which].ecls, insts[which].train);
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;

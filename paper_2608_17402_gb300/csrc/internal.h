@@ -183,24 +183,28 @@ enum { ECLS_BF16 = 0, ECLS_F32 = 1, ECLS_ADD = 2, ECLS_ADDT = 3, ECLS_DGELU = 4,
 // (idle) gather warps, each taking every fourth chunk of 32 rows.
 constexpr int GM_ADDT_PARTS = 4;
 static_assert(4 * GM_ADDT_PARTS == GM_EPI_WARPS + GM_GATHER_WARPS, "the gather warps join the epilogue");
-// Shared memory beside the operand ring: ECLS_ADD stages 16 rows per warp, ECLS_ADDT keeps
-// the {token, scale} pairs of 32 rows per warp; both give up one of the 7 stages.  The
+// Shared memory beside the operand ring: the bf16 outputs pass 32 columns (training path: 16
+// of up to three arrays) of 32 rows per warp, ECLS_ADD stages 16 rows per warp, ECLS_ADDT keeps
+// the {token, scale} pairs of 32 rows per warp; each gives up one of the 7 stages.  The
 // activation derivatives buffer two 16-column steps of u, a (and v) per warp, two stages.
-__host__ __device__ constexpr int gm_stg_bytes(int ecls) {
-    return ecls == ECLS_ADD ? GM_EPI_WARPS * GM_STG_ROWS * GM_STG_LD * 4
+__host__ __device__ constexpr int gm_bf16_warp_bytes(bool train) { return train ? 3 * 32 * 32 : 32 * 64; }
+__host__ __device__ constexpr int gm_stg_bytes(int ecls, bool train) {
+    return ecls == ECLS_BF16 ? GM_EPI_WARPS * gm_bf16_warp_bytes(train)
+           : ecls == ECLS_ADD ? GM_EPI_WARPS * GM_STG_ROWS * GM_STG_LD * 4
            : ecls == ECLS_ADDT ? 4 * GM_ADDT_PARTS * 32 * 8
            : ecls == ECLS_DGELU ? GM_EPI_WARPS * 2 * 2 * 1024
            : ecls == ECLS_DSWIGLU ? GM_EPI_WARPS * 2 * 3 * 1024 : 0;
 }
-__host__ __device__ constexpr int gm_stages(int ecls) {
-    return ecls == ECLS_DGELU || ecls == ECLS_DSWIGLU ? 5 : ecls == ECLS_ADD || ecls == ECLS_ADDT ? 6 : 7;
+__host__ __device__ constexpr int gm_stages(int ecls, bool) {
+    return ecls == ECLS_DGELU || ecls == ECLS_DSWIGLU ? 5 : ecls == ECLS_F32 ? 7 : 6;
 }
-__host__ __device__ constexpr int gm_smem_bytes(int ecls) {
-    return gm_stages(ecls) * (GM_A_BYTES + GM_B_BYTES) + gm_stg_bytes(ecls) + GM_OVERHEAD_BYTES;
+__host__ __device__ constexpr int gm_smem_bytes(int ecls, bool train) {
+    return gm_stages(ecls, train) * (GM_A_BYTES + GM_B_BYTES) + gm_stg_bytes(ecls, train) + GM_OVERHEAD_BYTES;
 }
-static_assert(gm_smem_bytes(ECLS_BF16) <= 232448 && gm_smem_bytes(ECLS_ADD) <= 232448 &&
-                  gm_smem_bytes(ECLS_ADDT) <= 232448 && gm_smem_bytes(ECLS_DGELU) <= 232448 &&
-                  gm_smem_bytes(ECLS_DSWIGLU) <= 232448,
+static_assert(gm_smem_bytes(ECLS_BF16, true) <= 232448 && gm_smem_bytes(ECLS_BF16, false) <= 232448 &&
+                  gm_smem_bytes(ECLS_F32, false) <= 232448 && gm_smem_bytes(ECLS_ADD, true) <= 232448 &&
+                  gm_smem_bytes(ECLS_ADDT, true) <= 232448 && gm_smem_bytes(ECLS_DGELU, true) <= 232448 &&
+                  gm_smem_bytes(ECLS_DSWIGLU, true) <= 232448,
               "shared memory of one CTA");
 static_assert(3 * GM_STAGES_MAX + 5 <= 32, "barriers fit before the signal sink at +256 bytes");
 // The transposed product reads the GEMM rows through boxes of 32 rows, as many as its
