@@ -399,6 +399,9 @@ moevie_status route_impl(const void* x, const float* W_r, const float* b, int64_
                          void* ws, cudaStream_t s, bool logits_only = false,
                          float* logits_out = nullptr, float* zero_acc = nullptr) {
     DevStatus* st = at<DevStatus>(ws, L.status);
+    if (!logits_only && route_small(T, (int)d, (int)E))
+        return cuda_status(launch_route_small(static_cast<const __nv_bfloat16*>(x), W_r, b, (int)T, (int)d, (int)E,
+                                              (int)k, idx, gate, st, s, zero_acc, T * d));
     const int Ep = route_epad((int)E);
     __nv_bfloat16* wsplit = at<__nv_bfloat16>(ws, L.wsplit);
     float* wrt = at<float>(ws, L.wrt);

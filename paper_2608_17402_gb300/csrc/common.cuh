@@ -24,7 +24,9 @@ struct DevStatus {
     int fb_count;    // router: tokens re-decided with exact logits in the last call
     int bar_count;   // grid barrier of a cooperative launch: arrivals so far (0 between barriers)
     int bar_gen;     //   and the barrier's generation (bumped by the last arrival)
-    int pad[57];
+    int route_sum;    // one-launch router: tokens re-decided so far in the running call,
+    int route_ticket; //   and its CTAs done (both 0 between calls)
+    int pad[55];
 };
 static_assert(sizeof(DevStatus) == 256, "status block is 256 bytes");
 

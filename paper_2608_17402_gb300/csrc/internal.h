@@ -97,6 +97,13 @@ int route_ksplit(int64_t T, int d, int E);
 // monotone in T (ROUTE_MAX_KSPLIT T, and (ROUTE_SPLIT_TARGET + m-tiles x n-tiles) x 256).
 int64_t route_logits_rows(int64_t T, int d, int E);
 
+// The one-launch router of small problems (route_small_kernel): whether these sizes take it,
+// and its launch (idx, gate, fb_count; it also clears zero[0, zero_n) as launch_route_select).
+bool route_small(int64_t T, int d, int E);
+cudaError_t launch_route_small(const __nv_bfloat16* x, const float* Wr, const float* b, int T, int d, int E, int k,
+                               int32_t* idx, float* gate, DevStatus* st, cudaStream_t s, float* zero = nullptr,
+                               int64_t zero_n = 0);
+
 // out = the sum over the nparts partial logit arrays (n floats each, part_stride apart).
 cudaError_t launch_route_sum_parts(const float* logits, int64_t part_stride, int nparts, int64_t n,
                                    float* out, cudaStream_t s);

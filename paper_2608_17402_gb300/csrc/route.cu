@@ -230,10 +230,89 @@ __device__ __forceinline__ double long_acc_value(unsigned __int128 u, int Q) {
     return neg ? -r : r;
 }
 
+// The k experts of largest key sigmoid(s) + b of one token (a warp; expert e sits in lane
+// e % 32, slot e / 32), ties to the lower id, and whether the logit error bounds ts certify
+// them.  Each of the k selection rounds takes the warp maximum of the keys' order codes
+// (redux.sync) and then the lowest id holding it (ballots in slot order).
+template <int NPL>
+__device__ __forceinline__ bool select_certified(const float (&sv)[NPL], const float (&ts)[NPL],
+                                                 const float* __restrict__ b, int E, int k, int lane,
+                                                 float (&sg)[NPL], uint32_t& taken) {
+    float key[NPL];
+    uint32_t code[NPL];
+#pragma unroll
+    for (int i = 0; i < NPL; ++i) {
+        const int e = lane + 32 * i;
+        if (e < E) {
+            sg[i] = sigmoid_fast(sv[i]);
+            key[i] = sg[i] + b[e];
+            code[i] = ord_f32(key[i]);
+        } else {
+            sg[i] = 0.f;
+            key[i] = -INFINITY;
+            code[i] = 0;
+        }
+    }
+    taken = 0;
+    for (int j = 0; j < k; ++j) {
+        uint32_t best = 0;
+#pragma unroll
+        for (int i = 0; i < NPL; ++i) {
+            const uint32_t c = ((taken >> i) & 1u) ? 0u : code[i];
+            best = c > best ? c : best;
+        }
+        best = __reduce_max_sync(0xffffffffu, best);
+#pragma unroll
+        for (int i = 0; i < NPL; ++i) {
+            const uint32_t m = __ballot_sync(0xffffffffu, !((taken >> i) & 1u) && code[i] == best);
+            if (m) {
+                if (lane == __ffs(m) - 1) taken |= 1u << i;
+                break;
+            }
+        }
+    }
+    bool certain = k >= E;
+    for (int pass = 0; pass < 2 && !certain; ++pass) {
+        float lo_in = INFINITY, hi_out = -INFINITY;
+#pragma unroll
+        for (int i = 0; i < NPL; ++i) {
+            const int e = lane + 32 * i;
+            if (e >= E) continue;
+            const float tk = pass == 0 ? 0.25f * ts[i] + ROUTE_KEY_SLACK
+                                       : key_tau_exact_slope(sv[i], ts[i]);
+            if ((taken >> i) & 1u) lo_in = fminf(lo_in, key[i] - tk);
+            else hi_out = fmaxf(hi_out, key[i] + tk);
+        }
+        certain = __reduce_min_sync(0xffffffffu, ord_f32(lo_in)) >
+                  __reduce_max_sync(0xffffffffu, ord_f32(hi_out));
+    }
+    return certain;
+}
+
+// Ascending ids of the selected experts and their gates sigmoid(s) / sum.
+template <int NPL>
+__device__ __forceinline__ void write_selection(uint32_t taken, const float (&sg)[NPL], int64_t t, int k, int lane,
+                                                int32_t* __restrict__ idx, float* __restrict__ gate) {
+    float ssum = 0.f;
+#pragma unroll
+    for (int i = 0; i < NPL; ++i) ssum += ((taken >> i) & 1u) ? sg[i] : 0.f;
+    ssum = warp_sum(ssum);
+    const uint32_t lt = (1u << lane) - 1u;
+    int base = 0;
+#pragma unroll
+    for (int i = 0; i < NPL; ++i) {
+        const uint32_t m = __ballot_sync(0xffffffffu, (taken >> i) & 1u);
+        if ((taken >> i) & 1u) {
+            const int pos = base + __popc(m & lt);
+            idx[t * k + pos] = lane + 32 * i;
+            gate[t * k + pos] = __fdividef(sg[i], ssum);
+        }
+        base += __popc(m);
+    }
+}
+
 // One warp per token.  NPL = experts per lane (expert e sits in lane e % 32, slot e / 32).
-// s holds nparts partial logit arrays, part p at s + p * part_stride.  Each of the k
-// selection rounds takes the warp maximum of the keys' order codes (redux.sync) and
-// then the lowest id holding it (ballots in slot order), so ties go to the lower id.
+// s holds nparts partial logit arrays, part p at s + p * part_stride.
 // A token the certificate cannot settle is listed for route_fallback_kernel.
 template <int NPL>
 __global__ void __launch_bounds__(256) route_topk_kernel(
@@ -270,56 +349,14 @@ __global__ void __launch_bounds__(256) route_topk_kernel(
         }
     }
     const float xn = xnorm[t];   // |x_t|, written by the router GEMM
-    float sg[NPL], key[NPL], ts[NPL];
-    uint32_t code[NPL];
+    float sg[NPL], ts[NPL];
 #pragma unroll
     for (int i = 0; i < NPL; ++i) {
         const int e = lane + 32 * i;
-        if (e < E) {
-            sg[i] = sigmoid_fast(sv[i]);
-            key[i] = sg[i] + b[e];
-            ts[i] = logit_tau(xn, wnorm[e], wnorm[E + e]);
-            code[i] = ord_f32(key[i]);
-        } else {
-            sg[i] = 0.f;
-            key[i] = -INFINITY;
-            ts[i] = 0.f;
-            code[i] = 0;
-        }
+        ts[i] = e < E ? logit_tau(xn, wnorm[e], wnorm[E + e]) : 0.f;
     }
-    uint32_t taken = 0;
-    for (int j = 0; j < k; ++j) {
-        uint32_t best = 0;
-#pragma unroll
-        for (int i = 0; i < NPL; ++i) {
-            const uint32_t c = ((taken >> i) & 1u) ? 0u : code[i];
-            best = c > best ? c : best;
-        }
-        best = __reduce_max_sync(0xffffffffu, best);
-#pragma unroll
-        for (int i = 0; i < NPL; ++i) {
-            const uint32_t m = __ballot_sync(0xffffffffu, !((taken >> i) & 1u) && code[i] == best);
-            if (m) {
-                if (lane == __ffs(m) - 1) taken |= 1u << i;
-                break;
-            }
-        }
-    }
-    bool certain = k >= E;
-    for (int pass = 0; pass < 2 && !certain; ++pass) {
-        float lo_in = INFINITY, hi_out = -INFINITY;
-#pragma unroll
-        for (int i = 0; i < NPL; ++i) {
-            const int e = lane + 32 * i;
-            if (e >= E) continue;
-            const float tk = pass == 0 ? 0.25f * ts[i] + ROUTE_KEY_SLACK
-                                       : key_tau_exact_slope(sv[i], ts[i]);
-            if ((taken >> i) & 1u) lo_in = fminf(lo_in, key[i] - tk);
-            else hi_out = fmaxf(hi_out, key[i] + tk);
-        }
-        certain = __reduce_min_sync(0xffffffffu, ord_f32(lo_in)) >
-                  __reduce_max_sync(0xffffffffu, ord_f32(hi_out));
-    }
+    uint32_t taken;
+    const bool certain = select_certified<NPL>(sv, ts, b, E, k, lane, sg, taken);
     if (!certain) {
         if (nparts > 1) {   // the re-decision reads the summed logits from part 0
 #pragma unroll
@@ -334,26 +371,11 @@ __global__ void __launch_bounds__(256) route_topk_kernel(
         }
         return;
     }
-    float ssum = 0.f;
-#pragma unroll
-    for (int i = 0; i < NPL; ++i) ssum += ((taken >> i) & 1u) ? sg[i] : 0.f;
-    ssum = warp_sum(ssum);
-    const uint32_t lt = (1u << lane) - 1u;
-    int base = 0;
-#pragma unroll
-    for (int i = 0; i < NPL; ++i) {
-        const uint32_t m = __ballot_sync(0xffffffffu, (taken >> i) & 1u);
-        if ((taken >> i) & 1u) {
-            const int pos = base + __popc(m & lt);
-            idx[(int64_t)t * k + pos] = lane + 32 * i;
-            gate[(int64_t)t * k + pos] = __fdividef(sg[i], ssum);
-        }
-        base += __popc(m);
-    }
+    write_selection<NPL>(taken, sg, t, k, lane, idx, gate);
 }
 
 
-// Exact re-decision of uncertified tokens, one CTA (8 warps) per token.  The CTA stages
+// Exact re-decision of one uncertified token by a CTA of 8 warps.  The CTA stages
 // the token's x row in shared memory (16-byte loads) and finds its largest exponent
 // field; warp 0 bounds the keys and lists the candidates; then the candidates' exact
 // logits are formed FB_BATCH at a time by all 256 threads (threads over the d terms,
@@ -373,6 +395,185 @@ constexpr int FB_X_SMEM = 16384;  // largest d whose x row is staged in shared m
 // that up to five tokens per SM are re-decided at once
 constexpr int FB_CTAS_PER_SM = 5;
 template <int NPL>
+struct FbShared {
+    int cand[32 * NPL];
+    double key[32 * NPL];
+    unsigned long long acc[8][FB_BATCH][2];
+    int q[FB_BATCH];
+    int ncand;
+    int qx;
+};
+
+// Token t: xg its x row, fb_x its staging buffer (staged), logits(sv, ts) this lane's fast
+// logits and their error bounds (called by warp 0; slots past E get anything), window(e) the
+// largest exponent field of W_r[:, e] (called by a warp), weight(e, i) = W_r[i, e].  The caller
+// synchronises the CTA before sh and fb_x are used again.
+template <int NPL, class Logits, class Window, class Weight>
+__device__ __forceinline__ void redecide_token(FbShared<NPL>& sh, const uint16_t* __restrict__ xg, uint16_t* fb_x,
+                                               bool staged, const float* __restrict__ b, int64_t t, int d, int E,
+                                               int k, int32_t* __restrict__ idx, float* __restrict__ gate,
+                                               DevStatus* st, Logits logits, Window window, Weight weight) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    if (threadIdx.x == 0) sh.qx = 1;
+    __syncthreads();
+    if (warp > 0 || !staged) {   // warps 1-7 stage x_t while warp 0 bounds the keys
+        int m = 1;
+        const int nthr = staged ? (int)blockDim.x - 32 : (int)blockDim.x;
+        const int tid = staged ? (int)threadIdx.x - 32 : (int)threadIdx.x;
+        for (int i = tid; i < d / 8; i += nthr) {   // d % 8 == 0, rows 16-byte aligned
+            const uint4 v = reinterpret_cast<const uint4*>(xg)[i];
+            if (staged) reinterpret_cast<uint4*>(fb_x)[i] = v;
+            const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                m = max(m, max((int)((w4[j] >> 7) & 0xffu), (int)((w4[j] >> 23) & 0xffu)));
+        }
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (lane == 0) atomicMax(&sh.qx, m);
+    }
+    float sv[NPL], ts[NPL];
+    uint32_t sure_in = 0, cand = 0;
+    int need = 0;
+    if (warp == 0) {
+        float up[NPL], lo[NPL];
+        logits(sv, ts);
+#pragma unroll
+        for (int i = 0; i < NPL; ++i) {
+            const int e = lane + 32 * i;
+            if (e < E) {
+                const float key = sigmoid_fast(sv[i]) + b[e];
+                const float tk = key_tau_exact_slope(sv[i], ts[i]);
+                up[i] = key + tk;
+                lo[i] = key - tk;
+            } else {
+                up[i] = lo[i] = -INFINITY;
+            }
+        }
+        // k-th / (k+1)-th largest upper ends and k-th largest lower end
+        float u_k, u_k1, l_k, l_k1;
+        warp_kth_values<NPL>(up, E, k, lane, u_k, u_k1);
+        warp_kth_values<NPL>(lo, E, k, lane, l_k, l_k1);
+#pragma unroll
+        for (int i = 0; i < NPL; ++i) {
+            const int e = lane + 32 * i;
+            if (e >= E) continue;
+            // k-th largest upper end among the others (u_k when e may sit at rank k: conservative)
+            const float thr = up[i] > u_k ? u_k1 : u_k;
+            if (k >= E || lo[i] > thr) sure_in |= 1u << i;
+            else if (!(up[i] < l_k)) cand |= 1u << i;
+        }
+        int n_in = 0, n_cand = 0;
+#pragma unroll
+        for (int i = 0; i < NPL; ++i) {
+            n_in += __popc(__ballot_sync(0xffffffffu, (sure_in >> i) & 1u));
+            const uint32_t m = __ballot_sync(0xffffffffu, (cand >> i) & 1u);
+            if ((cand >> i) & 1u) sh.cand[n_cand + __popc(m & lt)] = lane + 32 * i;
+            n_cand += __popc(m);
+        }
+        need = k - n_in;
+        const bool bad = need < 0 || need > n_cand;
+        if (lane == 0) {
+            if (bad) report(st, MOEVIE_ERR_DEVICE, SITE_ROUTE_FALLBACK, t, need);
+            sh.ncand = bad ? -1 : (need == 0 ? 0 : n_cand);
+        }
+    }
+    __syncthreads();
+    const int nc = sh.ncand;
+    const int qx = sh.qx;
+    const uint16_t* xs = staged ? fb_x : xg;
+    for (int c0 = 0; c0 < nc; c0 += FB_BATCH) {
+        const int cn = min(FB_BATCH, nc - c0);
+        if (warp < cn) {   // warp c: the window of candidate c0 + c
+            const int e = sh.cand[c0 + warp];
+            const int qw = window(e);
+            if (lane == 0) sh.q[warp] = (qx == 255 || qw == 255) ? -1 : qx + qw;   // -1: NaN
+        }
+        __syncthreads();
+        unsigned __int128 acc[FB_BATCH];
+        int Q[FB_BATCH];
+        int ec[FB_BATCH];
+#pragma unroll
+        for (int c = 0; c < FB_BATCH; ++c) {
+            acc[c] = 0;
+            Q[c] = c < cn ? sh.q[c] : -1;
+            ec[c] = sh.cand[c0 + (c < cn ? c : 0)];
+        }
+        for (int i = threadIdx.x; i < d; i += blockDim.x) {
+            const uint32_t hx = xs[i];
+            uint32_t uw[FB_BATCH];
+#pragma unroll
+            for (int c = 0; c < FB_BATCH; ++c) uw[c] = Q[c] > 0 ? __float_as_uint(weight(ec[c], i)) : 0u;
+#pragma unroll
+            for (int c = 0; c < FB_BATCH; ++c)
+                if (Q[c] > 0) long_acc_term(hx, uw[c], Q[c], acc[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < FB_BATCH; ++c) {
+            if (Q[c] <= 0) continue;   // uniform over the CTA
+            const unsigned __int128 a = warp_sum_u128(acc[c]);
+            if (lane == 0) {
+                sh.acc[warp][c][0] = (unsigned long long)(uint64_t)a;
+                sh.acc[warp][c][1] = (unsigned long long)(uint64_t)(a >> 64);
+            }
+        }
+        __syncthreads();
+        if (warp == 0 && lane < cn) {   // candidate c0 + lane: the sum over the 8 warps
+            const int q = sh.q[lane];
+            double v = __longlong_as_double(0x7ff8000000000000ll);
+            if (q > 0) {
+                unsigned __int128 u = 0;
+#pragma unroll
+                for (int w = 0; w < 8; ++w)
+                    u += ((unsigned __int128)sh.acc[w][lane][1] << 64) | sh.acc[w][lane][0];
+                v = long_acc_value(u, q);
+            }
+            sh.key[c0 + lane] = 1.0 / (1.0 + exp(-v)) + (double)b[sh.cand[c0 + lane]];
+        }
+        __syncthreads();
+    }
+    if (warp == 0 && nc >= 0) {
+        double exk[NPL];
+        int base = 0;
+#pragma unroll
+        for (int i = 0; i < NPL; ++i) {
+            const uint32_t m = __ballot_sync(0xffffffffu, (cand >> i) & 1u);
+            exk[i] = ((cand >> i) & 1u && nc > 0) ? sh.key[base + __popc(m & lt)] : -INFINITY;
+            base += __popc(m);
+        }
+        // choose `need` candidates by exact key, ties to the lower id
+        uint32_t chosen = sure_in;
+        for (int r = 0; r < need; ++r) {
+            double bv = -INFINITY;
+            int bi = 0x7fffffff;
+#pragma unroll
+            for (int i = 0; i < NPL; ++i) {
+                const int e = lane + 32 * i;
+                if (((cand >> i) & 1u) && !((chosen >> i) & 1u) &&
+                    (exk[i] > bv || bi == 0x7fffffff)) {
+                    bv = exk[i];
+                    bi = e;
+                }
+            }
+#pragma unroll
+            for (int o = 16; o; o >>= 1) {
+                const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+                if (ov > bv || (ov == bv && oi < bi)) {
+                    bv = ov;
+                    bi = oi;
+                }
+            }
+            if ((bi & 31) == lane) chosen |= 1u << (bi >> 5);
+        }
+        float sg[NPL];
+#pragma unroll
+        for (int i = 0; i < NPL; ++i) sg[i] = ((chosen >> i) & 1u) ? sigmoid_fast(sv[i]) : 0.f;
+        write_selection<NPL>(chosen, sg, t, k, lane, idx, gate);
+    }
+}
+
+template <int NPL>
 __global__ void __launch_bounds__(256, (NPL <= 8 ? FB_CTAS_PER_SM : 1)) route_fallback_kernel(
     const __nv_bfloat16* __restrict__ x, const float* __restrict__ wrt, int dp,
     const int32_t* __restrict__ wexp, int wexp_parts, int Ep,
@@ -382,195 +583,235 @@ __global__ void __launch_bounds__(256, (NPL <= 8 ? FB_CTAS_PER_SM : 1)) route_fa
     DevStatus* st) {
     pdl_wait();
     extern __shared__ __align__(16) uint16_t fb_x[];   // the token's x row when d <= FB_X_SMEM
-    __shared__ int s_cand[32 * NPL];
-    __shared__ double s_key[32 * NPL];
-    __shared__ unsigned long long s_acc[8][FB_BATCH][2];
-    __shared__ int s_q[FB_BATCH];
-    __shared__ int s_ncand;
-    __shared__ int s_qx;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t lt = (1u << lane) - 1u;
+    __shared__ FbShared<NPL> sh;
+    const int lane = threadIdx.x & 31;
     const int nfb = st->fb_count;
     const bool staged = d <= FB_X_SMEM;
     for (int f = blockIdx.x; f < nfb; f += gridDim.x) {
         const int t = fb_tokens[f];
-        const uint16_t* xg = reinterpret_cast<const uint16_t*>(x) + (int64_t)t * d;
-        if (threadIdx.x == 0) s_qx = 1;
-        __syncthreads();
-        if (warp > 0 || !staged) {   // warps 1-7 stage x_t while warp 0 bounds the keys
-            int m = 1;
-            const int nthr = staged ? (int)blockDim.x - 32 : (int)blockDim.x;
-            const int tid = staged ? (int)threadIdx.x - 32 : (int)threadIdx.x;
-            for (int i = tid; i < d / 8; i += nthr) {   // d % 8 == 0, rows 16-byte aligned
-                const uint4 v = reinterpret_cast<const uint4*>(xg)[i];
-                if (staged) reinterpret_cast<uint4*>(fb_x)[i] = v;
-                const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    m = max(m, max((int)((w4[j] >> 7) & 0xffu), (int)((w4[j] >> 23) & 0xffu)));
-            }
-            m = __reduce_max_sync(0xffffffffu, m);
-            if (lane == 0) atomicMax(&s_qx, m);
-        }
-        float sv[NPL];
-        uint32_t sure_in = 0, cand = 0;
-        int need = 0;
-        if (warp == 0) {
-            const float xn = xnorm[t];
-            float up[NPL], lo[NPL];
-#pragma unroll
-            for (int i = 0; i < NPL; ++i) {
-                const int e = lane + 32 * i;
-                if (e < E) {
-                    sv[i] = s[(int64_t)t * ld + e];
-                    const float key = sigmoid_fast(sv[i]) + b[e];
-                    const float tk = key_tau_exact_slope(sv[i], logit_tau(xn, wnorm[e], wnorm[E + e]));
-                    up[i] = key + tk;
-                    lo[i] = key - tk;
-                } else {
-                    sv[i] = 0.f;
-                    up[i] = lo[i] = -INFINITY;
-                }
-            }
-            // k-th / (k+1)-th largest upper ends and k-th largest lower end
-            float u_k, u_k1, l_k, l_k1;
-            warp_kth_values<NPL>(up, E, k, lane, u_k, u_k1);
-            warp_kth_values<NPL>(lo, E, k, lane, l_k, l_k1);
-#pragma unroll
-            for (int i = 0; i < NPL; ++i) {
-                const int e = lane + 32 * i;
-                if (e >= E) continue;
-                // k-th largest upper end among the others (u_k when e may sit at rank k: conservative)
-                const float thr = up[i] > u_k ? u_k1 : u_k;
-                if (k >= E || lo[i] > thr) sure_in |= 1u << i;
-                else if (!(up[i] < l_k)) cand |= 1u << i;
-            }
-            int n_in = 0, n_cand = 0;
-#pragma unroll
-            for (int i = 0; i < NPL; ++i) {
-                n_in += __popc(__ballot_sync(0xffffffffu, (sure_in >> i) & 1u));
-                const uint32_t m = __ballot_sync(0xffffffffu, (cand >> i) & 1u);
-                if ((cand >> i) & 1u) s_cand[n_cand + __popc(m & lt)] = lane + 32 * i;
-                n_cand += __popc(m);
-            }
-            need = k - n_in;
-            const bool bad = need < 0 || need > n_cand;
-            if (lane == 0) {
-                if (bad) report(st, MOEVIE_ERR_DEVICE, SITE_ROUTE_FALLBACK, t, need);
-                s_ncand = bad ? -1 : (need == 0 ? 0 : n_cand);
-            }
-        }
-        __syncthreads();
-        const int nc = s_ncand;
-        const int qx = s_qx;
-        const uint16_t* xs = staged ? fb_x : xg;
-        for (int c0 = 0; c0 < nc; c0 += FB_BATCH) {
-            const int cn = min(FB_BATCH, nc - c0);
-            if (warp < cn) {   // warp c: the window of candidate c0 + c
-                const int e = s_cand[c0 + warp];
-                int qw = 1;
-                for (int pp = lane; pp < wexp_parts; pp += 32) qw = max(qw, __ldg(wexp + (int64_t)pp * Ep + e));
-                qw = __reduce_max_sync(0xffffffffu, qw);
-                if (lane == 0) s_q[warp] = (qx == 255 || qw == 255) ? -1 : qx + qw;   // -1: NaN
-            }
-            __syncthreads();
-            unsigned __int128 acc[FB_BATCH];
-            int Q[FB_BATCH];
-            const float* wc[FB_BATCH];
-#pragma unroll
-            for (int c = 0; c < FB_BATCH; ++c) {
-                acc[c] = 0;
-                Q[c] = c < cn ? s_q[c] : -1;
-                wc[c] = wrt + (int64_t)s_cand[c0 + (c < cn ? c : 0)] * dp;
-            }
-            for (int i = threadIdx.x; i < d; i += blockDim.x) {
-                const uint32_t hx = xs[i];
-                uint32_t uw[FB_BATCH];
-#pragma unroll
-                for (int c = 0; c < FB_BATCH; ++c) uw[c] = Q[c] > 0 ? __float_as_uint(__ldg(wc[c] + i)) : 0u;
-#pragma unroll
-                for (int c = 0; c < FB_BATCH; ++c)
-                    if (Q[c] > 0) long_acc_term(hx, uw[c], Q[c], acc[c]);
-            }
-#pragma unroll
-            for (int c = 0; c < FB_BATCH; ++c) {
-                if (Q[c] <= 0) continue;   // uniform over the CTA
-                const unsigned __int128 a = warp_sum_u128(acc[c]);
-                if (lane == 0) {
-                    s_acc[warp][c][0] = (unsigned long long)(uint64_t)a;
-                    s_acc[warp][c][1] = (unsigned long long)(uint64_t)(a >> 64);
-                }
-            }
-            __syncthreads();
-            if (warp == 0 && lane < cn) {   // candidate c0 + lane: the sum over the 8 warps
-                const int q = s_q[lane];
-                double v = __longlong_as_double(0x7ff8000000000000ll);
-                if (q > 0) {
-                    unsigned __int128 u = 0;
-#pragma unroll
-                    for (int w = 0; w < 8; ++w)
-                        u += ((unsigned __int128)s_acc[w][lane][1] << 64) | s_acc[w][lane][0];
-                    v = long_acc_value(u, q);
-                }
-                s_key[c0 + lane] = 1.0 / (1.0 + exp(-v)) + (double)b[s_cand[c0 + lane]];
-            }
-            __syncthreads();
-        }
-        if (warp == 0 && nc >= 0) {
-            double exk[NPL];
-            int base = 0;
-#pragma unroll
-            for (int i = 0; i < NPL; ++i) {
-                const uint32_t m = __ballot_sync(0xffffffffu, (cand >> i) & 1u);
-                exk[i] = ((cand >> i) & 1u && nc > 0) ? s_key[base + __popc(m & lt)] : -INFINITY;
-                base += __popc(m);
-            }
-            // choose `need` candidates by exact key, ties to the lower id
-            uint32_t chosen = sure_in;
-            for (int r = 0; r < need; ++r) {
-                double bv = -INFINITY;
-                int bi = 0x7fffffff;
+        redecide_token<NPL>(
+            sh, reinterpret_cast<const uint16_t*>(x) + (int64_t)t * d, fb_x, staged, b, t, d, E, k, idx, gate, st,
+            [&](float (&sv)[NPL], float (&ts)[NPL]) {
+                const float xn = xnorm[t];
 #pragma unroll
                 for (int i = 0; i < NPL; ++i) {
                     const int e = lane + 32 * i;
-                    if (((cand >> i) & 1u) && !((chosen >> i) & 1u) &&
-                        (exk[i] > bv || bi == 0x7fffffff)) {
-                        bv = exk[i];
-                        bi = e;
-                    }
+                    sv[i] = e < E ? s[(int64_t)t * ld + e] : 0.f;
+                    ts[i] = e < E ? logit_tau(xn, wnorm[e], wnorm[E + e]) : 0.f;
                 }
+            },
+            [&](int e) {
+                int qw = 1;
+                for (int pp = lane; pp < wexp_parts; pp += 32) qw = max(qw, __ldg(wexp + (int64_t)pp * Ep + e));
+                return (int)__reduce_max_sync(0xffffffffu, qw);
+            },
+            [&](int e, int i) { return __ldg(wrt + (int64_t)e * dp + i); });
+        __syncthreads();   // sh / fb_x are reused by the next token
+    }
+}
+
+// The whole router of a layer with few tokens x experts x d in one launch: fp32 logits on the
+// FMA pipes straight from W_r, the certified top-k, and the exact re-decision.  The
+// tensor-core route (split of W_r, GEMM, top-k, re-decision) is four dependent launches, 17.5
+// us at T = 512, d = 768, E = 16 and 18.0 at T = 256, E = 31 (back to back calls); this kernel
+// takes 10.5 (the rate of the calls) and 12.8.  A CTA of 8 warps takes 8 tokens, each warp an
+// eighth of d: chunks of CH rows of W_r and columns of x go through registers (one chunk
+// ahead) into the warp's shared memory as fp32, and each lane forms one token x 8 NE experts
+// with packed FMAs (lane = 4 token + expert group).  What bounds it is the L2 latency of the
+// chunks, about half a microsecond each: the rule that chooses it is route_small.  A product
+// of a bf16 and an fp32 value is rounded once with its sum (fma), `per` terms a warp, the
+// warps' sums added in order, so
+//   |s_fast - s| <= (per + 8) 2^-24 |x_t| |W_r[:, e]|
+// to first order (one more unit covers the rest): rigorous.  The loading lanes also form
+// |W_r[:, e]|, the columns' largest exponent fields and |x_t|.
+constexpr int RS_TB = 8, RS_NW = 8;   // tokens and warps per CTA
+template <int NE>
+constexpr size_t route_small_smem() {
+    constexpr size_t EP = 32 * NE, CH = 16 / NE;
+    return 4 * RS_NW * (CH * (RS_TB + EP) > RS_TB * EP ? CH * (RS_TB + EP) : RS_TB * EP);
+}
+// Units of 2^-24 |x_t| |W_r[:, e]| certified at least: twice the sum's own bound at d = 192.
+constexpr int ROUTE_SMALL_TAU_MIN = 64;
+template <int NE>
+__global__ void __launch_bounds__(256, 2) route_small_kernel(
+    const __nv_bfloat16* __restrict__ x, const float* __restrict__ Wr, const float* __restrict__ b, int T, int d,
+    int E, int k, int32_t* __restrict__ idx, float* __restrict__ gate, DevStatus* st, float4* __restrict__ zero,
+    int64_t zero_n4) {
+    pdl_wait();
+    if (zero) {   // side job: clear another buffer (the layer's fp32 y accumulator)
+        const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+        const uint64_t pol = l2_policy_evict_first();
+        for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < zero_n4;
+             i += (int64_t)gridDim.x * blockDim.x)
+            st_global_v4_hint(zero + i, z, pol);
+    }
+    constexpr int TB = RS_TB, EP = 32 * NE, NW = RS_NW, CH = 16 / NE;
+    constexpr int XPC = TB * CH / 8;          // 16-byte pieces of x a chunk: piece q of token tt is q * TB + tt
+    static_assert(XPC <= 32, "at most one piece of x a lane");
+    // per warp: x [CH][TB] and w [CH][EP]; afterwards the partial logits [NW][TB][EP]
+    constexpr int WBUF = CH * (TB + EP);
+    extern __shared__ __align__(16) float buf[];   // route_small_smem<NE>()
+    __shared__ float s_w2[NW][EP];      // partial sums of squares of W_r's columns, then |W_r[:, e]|
+    __shared__ uint32_t s_wmax[NW][EP]; // largest |w| bits, then exponent fields
+    __shared__ float s_x2[NW][TB];
+    __shared__ int s_list[TB], s_nlist;
+    __shared__ FbShared<NE> sh;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t t0 = (int64_t)blockIdx.x * TB;
+    if (threadIdx.x == 0) s_nlist = 0;
+    float* xs = buf + warp * WBUF;
+    float* ws = xs + CH * TB;
+    const int per = (d / 8 + NW - 1) / NW * 8;   // d % 8 == 0: slices of whole groups of 8
+    const int kbeg = warp * per, kend = min(d, kbeg + per);
+    const int xt = lane % TB, xk = 8 * (lane / TB);   // this lane's piece of x: its token, its first column
+    uint4 xr;
+    float wv[CH][NE];
+    auto load = [&](int k0) {   // chunk k0 .. k0 + CH - 1 into registers (zeros past kend, T and E)
+        const bool ok = lane < XPC && k0 + xk < kend && t0 + xt < T;
+        xr = ok ? *reinterpret_cast<const uint4*>(x + (t0 + xt) * d + k0 + xk) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-                for (int o = 16; o; o >>= 1) {
-                    const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-                    const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                    if (ov > bv || (ov == bv && oi < bi)) {
-                        bv = ov;
-                        bi = oi;
-                    }
-                }
-                if ((bi & 31) == lane) chosen |= 1u << (bi >> 5);
+        for (int u = 0; u < CH; ++u)
+#pragma unroll
+            for (int i = 0; i < NE; ++i) {
+                const int e = lane + 32 * i;
+                wv[u][i] = k0 + u < kend && e < E ? __ldg(Wr + (int64_t)(k0 + u) * E + e) : 0.f;
             }
-            float sg[NPL];
-            float ssum = 0.f;
+    };
+    uint64_t acc[4 * NE];   // token lane / 4, expert pairs 32 (p / 4) + 8 (lane % 4) + 2 (p % 4)
 #pragma unroll
-            for (int i = 0; i < NPL; ++i) {
-                sg[i] = ((chosen >> i) & 1u) ? sigmoid_fast(sv[i]) : 0.f;
-                ssum += sg[i];
-            }
-            ssum = warp_sum(ssum);
-            int pbase = 0;
+    for (int p = 0; p < 4 * NE; ++p) acc[p] = 0ull;
+    float w2[NE], x2 = 0.f;
+    uint32_t wm[NE];
 #pragma unroll
-            for (int i = 0; i < NPL; ++i) {
-                const uint32_t m = __ballot_sync(0xffffffffu, (chosen >> i) & 1u);
-                if ((chosen >> i) & 1u) {
-                    const int pos = pbase + __popc(m & lt);
-                    idx[(int64_t)t * k + pos] = lane + 32 * i;
-                    gate[(int64_t)t * k + pos] = __fdividef(sg[i], ssum);
-                }
-                pbase += __popc(m);
+    for (int i = 0; i < NE; ++i) {
+        w2[i] = 0.f;
+        wm[i] = 0u;
+    }
+    const int tg = lane >> 2, eg = lane & 3;
+    if (kbeg < kend) load(kbeg);
+    for (int k0 = kbeg; k0 < kend; k0 += CH) {
+        __syncwarp();   // the previous chunk has been read
+        if (lane < XPC) {
+            float f[8];
+            unpack_bf16x8(xr, f);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                xs[(xk + i) * TB + xt] = f[i];
+                x2 = fmaf(f[i], f[i], x2);
             }
         }
-        __syncthreads();   // s_cand / s_key / s_ncand / s_qx / fb_x are reused by the next token
+#pragma unroll
+        for (int u = 0; u < CH; ++u)
+#pragma unroll
+            for (int i = 0; i < NE; ++i) {
+                ws[u * EP + lane + 32 * i] = wv[u][i];
+                w2[i] = fmaf(wv[u][i], wv[u][i], w2[i]);
+                wm[i] = max(wm[i], __float_as_uint(wv[u][i]) & 0x7fffffffu);
+            }
+        __syncwarp();
+        if (k0 + CH < kend) load(k0 + CH);
+#pragma unroll
+        for (int u = 0; u < CH; ++u) {
+            uint64_t w[4 * NE];
+#pragma unroll
+            for (int i = 0; i < NE; ++i)
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(ws + u * EP + 32 * i + 8 * eg + 4 * p);
+                    w[4 * i + 2 * p] = v.x;
+                    w[4 * i + 2 * p + 1] = v.y;
+                }
+            const float xv = xs[u * TB + tg];
+            const uint64_t xx = f2_pack(xv, xv);
+#pragma unroll
+            for (int p = 0; p < 4 * NE; ++p) acc[p] = f2_fma(xx, w[p], acc[p]);
+        }
+    }
+    __syncthreads();   // the chunks are done with
+#pragma unroll
+    for (int p = 0; p < 4 * NE; ++p) {
+        float a0, a1;
+        f2_unpack(acc[p], a0, a1);
+        *reinterpret_cast<float2*>(buf + (warp * TB + tg) * EP + 32 * (p / 4) + 8 * eg + 2 * (p % 4)) =
+            make_float2(a0, a1);
+    }
+#pragma unroll
+    for (int i = 0; i < NE; ++i) {
+        s_w2[warp][lane + 32 * i] = w2[i];
+        s_wmax[warp][lane + 32 * i] = wm[i];
+    }
+#pragma unroll
+    for (int o = TB; o < 32; o <<= 1) x2 += __shfl_xor_sync(0xffffffffu, x2, o);   // a token's pieces: lanes TB apart
+    if (lane < TB) s_x2[warp][lane] = x2;
+    __syncthreads();
+    for (int e = threadIdx.x; e < EP; e += blockDim.x) {
+        float v = 0.f;
+        uint32_t m = 0u;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {
+            v += s_w2[q][e];
+            m = max(m, s_wmax[q][e]);
+        }
+        s_w2[0][e] = sqrtf(v);
+        s_wmax[0][e] = max(1u, m >> 23);   // exponent field (subnormals and zero count as 1)
+    }
+    __syncthreads();
+    const float tau = (float)max(per + NW + 1, ROUTE_SMALL_TAU_MIN) * 5.9604645e-8f * 1.001f;
+    auto token_tau = [&](int tt, float (&ts)[NE]) {
+        float q2 = 0.f;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) q2 += s_x2[q][tt];
+        const float xn = sqrtf(q2);
+#pragma unroll
+        for (int i = 0; i < NE; ++i) ts[i] = tau * s_w2[0][lane + 32 * i] * xn;
+    };
+    static_assert(TB == NW, "a warp per token");
+    const int tt = warp;
+    if (t0 + tt < T) {
+        float sv[NE], ts[NE], sg[NE];
+#pragma unroll
+        for (int i = 0; i < NE; ++i) {
+            float v = 0.f;
+#pragma unroll
+            for (int q = 0; q < NW; ++q) v += buf[(q * TB + tt) * EP + lane + 32 * i];
+            sv[i] = v;
+        }
+        token_tau(tt, ts);
+        uint32_t taken;
+        if (select_certified<NE>(sv, ts, b, E, k, lane, sg, taken)) {
+            write_selection<NE>(taken, sg, t0 + tt, k, lane, idx, gate);
+        } else {   // listed; its logits stay in the first partial array
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < NE; ++i) buf[tt * EP + lane + 32 * i] = sv[i];
+            if (lane == 0) s_list[atomicAdd(&s_nlist, 1)] = tt;
+        }
+    }
+    __syncthreads();
+    const int nlist = s_nlist;
+    for (int f = 0; f < nlist; ++f) {
+        const int tt = s_list[f];
+        redecide_token<NE>(
+            sh, reinterpret_cast<const uint16_t*>(x) + (t0 + tt) * d, nullptr, false, b, t0 + tt, d, E, k, idx, gate,
+            st,
+            [&](float (&sv)[NE], float (&ts)[NE]) {
+#pragma unroll
+                for (int i = 0; i < NE; ++i) sv[i] = buf[tt * EP + lane + 32 * i];
+                token_tau(tt, ts);
+            },
+            [&](int e) { return (int)s_wmax[0][e]; },
+            [&](int e, int i) { return __ldg(Wr + (int64_t)i * E + e); });
+        __syncthreads();   // sh is reused
+    }
+    // tokens re-decided in this call: the last CTA publishes the sum and clears the counters
+    if (threadIdx.x == 0) {
+        if (nlist) atomicAdd(&st->route_sum, nlist);
+        __threadfence();
+        if (atomicAdd(&st->route_ticket, 1) == (int)gridDim.x - 1) {
+            __threadfence();
+            st->fb_count = atomicExch(&st->route_sum, 0);
+            st->route_ticket = 0;
+        }
     }
 }
 
@@ -628,6 +869,27 @@ cudaError_t launch_route_sum_parts(const float* logits, int64_t part_stride, int
                                    float* out, cudaStream_t s) {
     const cudaError_t e = launch_pdl(route_sum_parts_kernel, dim3((unsigned)((n + 255) / 256)),
                                      dim3(256), 0, s, logits, part_stride, nparts, n, out);
+    count_launches(1);
+    return e;
+}
+
+// The one-launch router takes up to eight tokens for each SM (one wave of CTAs) and chunks
+// few enough: 32 ceil(E / 32) d <= 32768, so at most eight chunks a warp.  Measured against the
+// tensor-core route, back to back calls: T = 512, d = 768, E = 16 10.5 against 17.5 us, T = 256,
+// E = 31 12.8 against 18.0; past the line, T = 1024, d = 1536, E = 64 (24 chunks) 31 against 24.
+bool route_small(int64_t T, int d, int E) {
+    return T >= 1 && T <= 8 * 152 && E <= 64 && (int64_t)(E + 31) / 32 * 32 * d <= 32768;
+}
+
+cudaError_t launch_route_small(const __nv_bfloat16* x, const float* Wr, const float* b, int T, int d, int E, int k,
+                               int32_t* idx, float* gate, DevStatus* st, cudaStream_t s, float* zero,
+                               int64_t zero_n) {
+    if (!route_small(T, d, E)) return cudaErrorInvalidValue;
+    static_assert(route_small_smem<1>() <= 48 * 1024 && route_small_smem<2>() <= 48 * 1024, "no opt-in needed");
+    const auto kern = E <= 32 ? route_small_kernel<1> : route_small_kernel<2>;
+    const cudaError_t e = launch_pdl(kern, dim3((unsigned)((T + RS_TB - 1) / RS_TB)), dim3(256),
+                                     E <= 32 ? route_small_smem<1>() : route_small_smem<2>(), s, x, Wr, b, T, d, E, k,
+                                     idx, gate, st, reinterpret_cast<float4*>(zero), zero ? zero_n / 4 : (int64_t)0);
     count_launches(1);
     return e;
 }
