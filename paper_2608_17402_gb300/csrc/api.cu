@@ -1166,41 +1166,52 @@ moevie_status moevie_moe_backward(const moevie_layer* Lr, const void* x, const v
                           at<int32_t>(ws, L.hist), at<int32_t>(ws, L.counts), at<int32_t>(ws, L.offsets),
                           at<int4>(ws, L.tiles), at<int32_t>(ws, L.n_tiles), at<int32_t>(ws, L.perm),
                           at<int32_t>(ws, L.inv), nullptr, nullptr, st, s));
-    // 2. segments padded to 64 rows: row maps, m-tiles, weight-gradient items
-    MV_TRY(launch_bwd_pad(at<int32_t>(ws, L.counts), (int)E, poff, s));
+    // 2. segments padded to 64 rows: offsets, m-tiles, weight-gradient items; row maps
+    int bn_s = 0, nt_s = 0;
+    const int64_t hsp = shared ? row_ld(hs) : 0;
+    BwdPlan plan{};
+    plan.counts = at<int32_t>(ws, L.counts);
+    plan.E = (int)E;
+    plan.poff = poff;
+    plan.tiles = at<int4>(ws, L.ptiles);
+    plan.n_tiles = at<int32_t>(ws, L.n_ptiles);
+    plan.st = st;
+    auto item_set = [&](int64_t dense_rows, int64_t M, int64_t N, int bn, int64_t max_items, size_t items,
+                        size_t n_items, size_t gclear) {
+        plan.sets[plan.nsets++] = {(int)M, (int)N, bn, (int)max_items, dense_rows, at<int4>(ws, items),
+                                   at<int32_t>(ws, n_items), at<int32_t>(ws, gclear)};
+    };
+    item_set(0, h, d, bn_d, L.max_it2, L.it2, L.n_it2, L.gc2);
+    item_set(0, d, h, bn_h, L.max_it1, L.it1, L.n_it1, L.gc1);
+    item_set(T, d, Ep, bn_e, L.max_itr, L.itr, L.n_itr, L.gcr);
+    if (shared) {
+        choose_bn((int)hs, &bn_s, &nt_s);
+        item_set(T, hs, d, bn_d, L.max_its2, L.its2, L.n_its2, L.gcs2);
+        item_set(T, d, hs, bn_s, L.max_its1, L.its1, L.n_its1, L.gcs1);
+    }
+    MV_TRY(launch_bwd_plan(plan, s));
     MV_TRY(launch_bwd_rows(idx, at<int32_t>(ws, L.inv), at<int32_t>(ws, L.counts), at<int32_t>(ws, L.offsets),
                            poff, at<float>(ws, L.gate), n, (int)k, (int)E, ptok, pgate,
                            at<int32_t>(ws, L.slot_prow), s));
-    MV_TRY(launch_tile_table(poff, (int)E, GM_BM, at<int4>(ws, L.ptiles), at<int32_t>(ws, L.n_ptiles), s));
-    MV_TRY(launch_bwd_items(poff, (int)E, 0, (int)h, (int)d, bn_d, (int)L.max_it2, at<int4>(ws, L.it2),
-                            at<int32_t>(ws, L.n_it2), at<int32_t>(ws, L.gc2), st, s));
-    MV_TRY(launch_bwd_items(poff, (int)E, 0, (int)d, (int)h, bn_h, (int)L.max_it1, at<int4>(ws, L.it1),
-                            at<int32_t>(ws, L.n_it1), at<int32_t>(ws, L.gc1), st, s));
-    MV_TRY(launch_bwd_items(nullptr, 1, T, (int)d, (int)Ep, bn_e, (int)L.max_itr, at<int4>(ws, L.itr),
-                            at<int32_t>(ws, L.n_itr), at<int32_t>(ws, L.gcr), st, s));
-    int bn_s = 0, nt_s = 0;
-    const int64_t hsp = shared ? row_ld(hs) : 0;
-    if (shared) {
-        choose_bn((int)hs, &bn_s, &nt_s);
-        MV_TRY(launch_bwd_items(nullptr, 1, T, (int)hs, (int)d, bn_d, (int)L.max_its2, at<int4>(ws, L.its2),
-                                at<int32_t>(ws, L.n_its2), at<int32_t>(ws, L.gcs2), st, s));
-        MV_TRY(launch_bwd_items(nullptr, 1, T, (int)d, (int)hs, bn_s, (int)L.max_its1, at<int4>(ws, L.its1),
-                                at<int32_t>(ws, L.n_its1), at<int32_t>(ws, L.gcs1), st, s));
-    }
     // 3. accumulators cleared (of the weight gradients only what their items will add
     //    into, or not write at all); gathered copies of x and g dy
     const int sms = num_sms();
-    MV_TRY(launch_zero_f32(dx, T * d, s));
-    MV_TRY(launch_bwd_zero(at<int32_t>(ws, L.gc1), (int)E, (int)d, (int)h, hp, dW1, sms, s));
-    MV_TRY(launch_bwd_zero(at<int32_t>(ws, L.gc2), (int)E, (int)h, (int)d, d, dW2, sms, s));
-    if (swiglu) MV_TRY(launch_bwd_zero(at<int32_t>(ws, L.gc1), (int)E, (int)d, (int)h, hp, dW3, sms, s));
+    BwdZero zero{};
+    auto clear = [&](const int32_t* gclear, int64_t G, int64_t M, int64_t N, int64_t ld, float* out) {
+        zero.jobs[zero.njobs++] = {gclear, (int)G, (int)M, (int)N, ld, out};
+    };
+    clear(nullptr, 1, T, d, d, dx);
+    clear(nullptr, 1, T, Ep / 2, Ep / 2, reinterpret_cast<float*>(DS));   // bf16 [T][Ep]
+    clear(at<int32_t>(ws, L.gcr), 1, d, Ep, Ep, dwr);
+    clear(at<int32_t>(ws, L.gc1), E, d, h, hp, dW1);
+    clear(at<int32_t>(ws, L.gc2), E, h, d, d, dW2);
+    if (swiglu) clear(at<int32_t>(ws, L.gc1), E, d, h, hp, dW3);
     if (shared) {
-        MV_TRY(launch_bwd_zero(at<int32_t>(ws, L.gcs1), 1, (int)d, (int)hs, hsp, dWs1, sms, s));
-        MV_TRY(launch_bwd_zero(at<int32_t>(ws, L.gcs2), 1, (int)hs, (int)d, d, dWs2, sms, s));
-        if (swiglu) MV_TRY(launch_bwd_zero(at<int32_t>(ws, L.gcs1), 1, (int)d, (int)hs, hsp, dWs3, sms, s));
+        clear(at<int32_t>(ws, L.gcs1), 1, d, hs, hsp, dWs1);
+        clear(at<int32_t>(ws, L.gcs2), 1, hs, d, d, dWs2);
+        if (swiglu) clear(at<int32_t>(ws, L.gcs1), 1, d, hs, hsp, dWs3);
     }
-    MV_TRY(launch_bwd_zero(at<int32_t>(ws, L.gcr), 1, (int)d, (int)Ep, Ep, dwr, sms, s));
-    MV_TRY(launch_zero_f32(reinterpret_cast<float*>(DS), T * Ep / 2, s));
+    MV_TRY(launch_bwd_zero(zero, sms, s));
     MV_TRY(launch_bwd_gather(xb, static_cast<const __nv_bfloat16*>(dy), ptok, pgate, poff, (int)E, (int)d,
                              L.rows_max, static_cast<__nv_bfloat16*>(Xp), static_cast<__nv_bfloat16*>(Gm), s));
     // 4. up-projection again: u = x W1[e] and a = GELU(u), both kept (bf16; SwiGLU: u, v and a)

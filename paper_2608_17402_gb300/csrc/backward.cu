@@ -6,15 +6,13 @@
 // around them, all memory- or latency-bound:
 //   bwd_gates_kernel   per token, the fp32 logits of its k selected experts (W_r's
 //                      transposed copy), sigma, their sum S and the gates g = sigma / S
-//   bwd_pad_kernel     expert segments padded to multiples of 64 rows (the K blocks of
-//                      the weight-gradient GEMMs never straddle two experts)
+//   bwd_plan_kernel    expert segments padded to multiples of 64 rows (the K blocks of
+//                      the weight-gradient GEMMs never straddle two experts), their m-tiles,
+//                      and every weight-gradient item table, a CTA per table
 //   bwd_rows_kernel    per padded row its token (-1 for padding) and gate (0), and per
 //                      routing slot its padded row
-//   bwd_items_kernel   the weight-gradient work items {g, m0 | n0 << 16, kb0, kb1}: per
-//                      group, output tiles x chunks of at most BWD_KCH k-blocks (a group of
-//                      one chunk stores its gradient instead of adding into it)
-//   bwd_zero_kernel    clears what the items will add into or not write: the gradients of
-//                      groups with no rows or several chunks, and pad columns
+//   bwd_zero_kernel    clears dx, ds and, of every weight gradient, what its items will add
+//                      into or not write: groups with no rows or several chunks, pad columns
 //   bwd_gather_kernel  the padded rows of x and of g dy (bf16; zero rows for padding)
 //   bwd_router_kernel  per token: dg_j = dy . E_j(x) from the partial row dots, the gate
 //                      derivative ds (Eqs. 4-5), dx += ds W_r^T, and ds into a dense
@@ -36,7 +34,8 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 }
 
 // One warp per token: s_j = x_t . W_r[:, e_j] for its k experts (fp32, lanes over d; the
-// k dot products advance together, so each lane has k loads in flight per step),
+// k dot products advance together, four steps' loads ahead of their sums: with one step's
+// loads in flight the chain of d / 32 load latencies took 30 us at T = 8192, d = 1024),
 // sigma_j = 1 / (1 + e^-s_j), S = sum_j sigma_j, g_j = sigma_j / S.  KB >= k.
 template <int KB>
 __global__ void __launch_bounds__(256) bwd_gates_kernel(const __nv_bfloat16* __restrict__ x,
@@ -49,27 +48,43 @@ __global__ void __launch_bounds__(256) bwd_gates_kernel(const __nv_bfloat16* __r
     const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (t >= T) return;
     const __nv_bfloat16* xr = x + t * d;
-    const float* w[KB];
+    const float* w[KB];   // past k and for bad ids: any row, unused
     float acc[KB];
+    uint32_t okm = 0;
 #pragma unroll
     for (int j = 0; j < KB; ++j) {
         acc[j] = 0.f;
         const int e = j < k ? idx[t * k + j] : 0;
         const bool ok = e >= 0 && e < E;
         if (j < k && !ok && lane == 0) report(st, MOEVIE_ERR_DEVICE, SITE_PERMUTE_ID, (int)(t * k + j), e);
-        w[j] = (j < k && ok) ? wrt + (int64_t)e * dp : nullptr;
+        if (j < k && ok) okm |= 1u << j;
+        w[j] = wrt + (int64_t)(ok ? e : 0) * dp;
     }
-    for (int i = lane; i < d; i += 32) {
+    constexpr int U = KB <= 8 ? 4 : 1;
+    int i = lane;
+    for (; i + 32 * (U - 1) < d; i += 32 * U) {
+        float xi[U], wv[U][KB];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            xi[u] = __bfloat162float(xr[i + 32 * u]);
+#pragma unroll
+            for (int j = 0; j < KB; ++j) wv[u][j] = __ldg(w[j] + i + 32 * u);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int j = 0; j < KB; ++j) acc[j] = fmaf(xi[u], wv[u][j], acc[j]);
+    }
+    for (; i < d; i += 32) {
         const float xi = __bfloat162float(xr[i]);
 #pragma unroll
-        for (int j = 0; j < KB; ++j)
-            if (w[j]) acc[j] = fmaf(xi, __ldg(w[j] + i), acc[j]);
+        for (int j = 0; j < KB; ++j) acc[j] = fmaf(xi, __ldg(w[j] + i), acc[j]);
     }
     float ssum = 0.f, mine = 0.f;   // lane j keeps sigma_j
 #pragma unroll
     for (int j = 0; j < KB; ++j) {
         if (j >= k) break;
-        const float sgm = 1.0f / (1.0f + expf(-warp_sum_f(acc[j])));
+        const float sgm = 1.0f / (1.0f + expf(-warp_sum_f((okm >> j) & 1u ? acc[j] : 0.f)));
         if (lane == j) mine = sgm;
         ssum += sgm;
     }
@@ -79,36 +94,90 @@ __global__ void __launch_bounds__(256) bwd_gates_kernel(const __nv_bfloat16* __r
     }
 }
 
-// One CTA of 1024 threads (E <= 1024): poff[e] = sum over e' < e of counts rounded up to
-// 64 rows, poff[E] the padded total.
-__global__ void __launch_bounds__(1024) bwd_pad_kernel(const int32_t* __restrict__ counts, int E,
-                                                       int32_t* __restrict__ poff) {
-    pdl_wait();
-    __shared__ int wsum[32];
-    const int e = threadIdx.x, lane = e & 31, warp = e >> 5;
-    const int v = e < E ? (counts[e] + 63) / 64 * 64 : 0;
+// Exclusive scan of one int per thread over a CTA of 1024; *total = the sum (s_w: 33 ints).
+__device__ __forceinline__ int block_scan_1024(int v, int* s_w, int* total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int inc = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int u = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += u;
     }
-    if (lane == 31) wsum[warp] = inc;
+    if (lane == 31) s_w[warp] = inc;
     __syncthreads();
     if (warp == 0) {
-        const int w = wsum[lane];
+        const int w = s_w[lane];
         int wi = w;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int u = __shfl_up_sync(0xffffffffu, wi, o);
             if (lane >= o) wi += u;
         }
-        wsum[lane] = wi - w;
+        s_w[lane] = wi - w;
+        if (lane == 31) s_w[32] = wi;
     }
     __syncthreads();
-    const int ex = wsum[warp] + inc - v;
-    if (e < E) poff[e] = ex;
-    if (e == E - 1) poff[E] = ex + v;
+    const int ex = s_w[warp] + inc - v;
+    *total = s_w[32];
+    __syncthreads();   // s_w may be reused
+    return ex;
+}
+
+// The plan of the backward in one launch, CTAs of 1024 threads, one thread per expert (E <=
+// 1024): every CTA forms the padded offsets (counts rounded up to 64 rows) itself.  CTA 0
+// writes poff[E + 1] and the m-tile table of the padded rows; CTA q > 0 the item table of set
+// q - 1 (BwdItemSet): group g (an expert, or the one dense group) has the k-blocks of its
+// padded rows, cut into chunks of at most BWD_KCH; its items are every (m-tile of 256 of M
+// rows, n-tile of BN of N columns, chunk).  items[i] = {g, m0 | n0 << 16, kb0, kb1}; *n_items =
+// their number (at most max_items; more is a device error and none are listed).  A group
+// of one chunk writes each of its gradient's elements once: its items carry BWD_STORE_BIT in
+// kb1 (the GEMM stores instead of adding) and gclear[g] = 0; a group with no rows or several
+// chunks has gclear[g] = 1 (its gradient is cleared first).  (Seven to nine launches of one
+// CTA each before, 3 - 4 us apiece.)
+__global__ void __launch_bounds__(1024) bwd_plan_kernel(const __grid_constant__ BwdPlan p) {
+    pdl_wait();
+    __shared__ int s_w[33];
+    const int e = threadIdx.x;
+    int total;
+    const int v = e < p.E ? (p.counts[e] + 63) / 64 * 64 : 0;
+    const int off = block_scan_1024(v, s_w, &total);
+    if (blockIdx.x == 0) {
+        if (e < p.E) p.poff[e] = off;
+        if (e == 0) p.poff[p.E] = total;
+        const int nt = (v + GM_BM - 1) / GM_BM;
+        int ntiles;
+        const int toff = block_scan_1024(nt, s_w, &ntiles);
+        for (int m = 0; m < nt; ++m) p.tiles[toff + m] = make_int4(e, off + m * GM_BM, min(GM_BM, v - m * GM_BM), 0);
+        if (e == 0) *p.n_tiles = ntiles;
+        return;
+    }
+    const BwdItemSet& q = p.sets[blockIdx.x - 1];
+    const int G = q.dense_rows > 0 ? 1 : p.E;
+    const int mt = (q.M + GM_BM - 1) / GM_BM, nt = (q.N + q.BN - 1) / q.BN;
+    int kb0 = 0, kb1 = 0;
+    if (e < G) {
+        kb0 = q.dense_rows > 0 ? 0 : off / GM_BK;
+        kb1 = q.dense_rows > 0 ? (int)((q.dense_rows + GM_BK - 1) / GM_BK) : (off + v) / GM_BK;
+    }
+    const int chunks = (kb1 - kb0 + (int)BWD_KCH - 1) / (int)BWD_KCH;
+    int n;
+    int pos = block_scan_1024(chunks * mt * nt, s_w, &n);
+    if (n > q.max_items) {
+        if (e == 0) {
+            report(p.st, MOEVIE_ERR_DEVICE, SITE_GEMM_TILES, n, q.max_items);
+            *q.n_items = 0;
+        }
+        return;
+    }
+    const int store = chunks == 1 ? BWD_STORE_BIT : 0;
+    for (int c = 0; c < chunks; ++c) {
+        const int a = kb0 + c * (int)BWD_KCH, b = min(kb1, a + (int)BWD_KCH);
+        for (int m = 0; m < mt; ++m)
+            for (int j = 0; j < nt; ++j)
+                q.items[pos++] = make_int4(e, (m * GM_BM) | ((j * q.BN) << 16), a, b | store);
+    }
+    if (e < G) q.gclear[e] = chunks == 1 ? 0 : 1;
+    if (e == 0) *q.n_items = n;
 }
 
 // Threads over routing slots (t, j) and over (expert, padding row < 64): the padded row of
@@ -143,91 +212,23 @@ __global__ void bwd_rows_kernel(const int32_t* __restrict__ idx, const int32_t* 
     }
 }
 
-// One CTA of 1024 threads, one thread per group (G <= 1024): group g has the k-blocks
-// [koff[g] / 64, koff[g + 1] / 64) (koff == nullptr: one group of ceil(K_rows / 64)
-// k-blocks), cut into chunks of at most kch; its items are every (m-tile of 256 of M rows,
-// n-tile of BN of N columns, chunk).  items[i] = {g, m0 | n0 << 16, kb0, kb1}; *n_items =
-// their number (at most max_items; more is a device error and none are listed).  A group
-// of one chunk writes each of its gradient's elements once: its items carry
-// BWD_STORE_BIT in kb1 (the GEMM stores instead of adding) and gclear[g] = 0; a group
-// with no rows or several chunks has gclear[g] = 1 (its gradient is cleared first).
-__global__ void __launch_bounds__(1024) bwd_items_kernel(const int32_t* __restrict__ koff, int G,
-                                                         int64_t K_rows, int M, int N, int BN, int kch,
-                                                         int max_items, int4* __restrict__ items,
-                                                         int32_t* __restrict__ n_items,
-                                                         int32_t* __restrict__ gclear, DevStatus* st) {
+// Clears in one launch, blockIdx.y the buffer: of out [G][M][ld] (fp32) every row of a group
+// with gclear[g] set (or all rows, gclear == nullptr), and the pad columns [N, ld) of the
+// other groups' rows (what a weight gradient's items will not write).  One warp per row,
+// grid-strided; ld % 4 == 0.
+__global__ void __launch_bounds__(256) bwd_zero_kernel(const __grid_constant__ BwdZero z) {
     pdl_wait();
-    __shared__ int wsum[32];
-    __shared__ int s_total;
-    const int g = threadIdx.x, lane = g & 31, warp = g >> 5;
-    const int mt = (M + GM_BM - 1) / GM_BM, nt = (N + BN - 1) / BN;
-    int kb0 = 0, kb1 = 0;
-    if (g < G) {
-        if (koff) {
-            kb0 = koff[g] / GM_BK;
-            kb1 = koff[g + 1] / GM_BK;
-        } else {
-            kb1 = (int)((K_rows + GM_BK - 1) / GM_BK);
-        }
-    }
-    const int chunks = kb1 > kb0 ? (kb1 - kb0 + kch - 1) / kch : 0;
-    const int v = chunks * mt * nt;
-    int inc = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += u;
-    }
-    if (lane == 31) wsum[warp] = inc;
-    __syncthreads();
-    if (warp == 0) {
-        const int w = wsum[lane];
-        int wi = w;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += u;
-        }
-        wsum[lane] = wi - w;
-        if (lane == 31) s_total = wi;
-    }
-    __syncthreads();
-    const int total = s_total;
-    if (total > max_items) {
-        if (g == 0) {
-            report(st, MOEVIE_ERR_DEVICE, SITE_GEMM_TILES, total, max_items);
-            *n_items = 0;
-        }
-        return;
-    }
-    int pos = wsum[warp] + inc - v;
-    const int store = chunks == 1 ? BWD_STORE_BIT : 0;
-    for (int c = 0; c < chunks; ++c) {
-        const int a = kb0 + c * kch, b = min(kb1, a + kch);
-        for (int m = 0; m < mt; ++m)
-            for (int n = 0; n < nt; ++n)
-                items[pos++] = make_int4(g, (m * GM_BM) | ((n * BN) << 16), a, b | store);
-    }
-    if (g < G) gclear[g] = chunks == 1 ? 0 : 1;
-    if (g == 0) *n_items = total;
-}
-
-// The part of a weight gradient out [G][M][ld] (fp32) that the GEMM's items will not
-// write: every row of a group with gclear[g] set, and the pad columns [N, ld) of the
-// other groups' rows.  One warp per row, grid-strided; ld % 4 == 0.
-__global__ void __launch_bounds__(256) bwd_zero_kernel(const int32_t* __restrict__ gclear, int G, int M,
-                                                       int N, int64_t ld, float* __restrict__ out) {
-    pdl_wait();
+    const BwdZeroJob& j = z.jobs[blockIdx.y];
     const int lane = threadIdx.x & 31;
-    const int64_t rows = (int64_t)G * M;
+    const int64_t rows = (int64_t)j.G * j.M;
     for (int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < rows;
          q += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        float* row = out + q * ld;
-        if (gclear[q / M]) {
+        float* row = j.out + q * j.ld;
+        if (!j.gclear || j.gclear[q / j.M]) {
             float4* r4 = reinterpret_cast<float4*>(row);
-            for (int64_t c = lane; c < ld / 4; c += 32) r4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int64_t c = lane; c < j.ld / 4; c += 32) r4[c] = make_float4(0.f, 0.f, 0.f, 0.f);
         } else {
-            for (int64_t c = N + lane; c < ld; c += 32) row[c] = 0.f;
+            for (int64_t c = j.N + lane; c < j.ld; c += 32) row[c] = 0.f;
         }
     }
 }
@@ -264,8 +265,10 @@ __global__ void bwd_gather_kernel(const __nv_bfloat16* __restrict__ x, const __n
 
 // One warp per token (Eqs. 4-5 backward): dg_j = sum of the nparts partial row dots of
 // its padded row, gdg = sum_j g_j dg_j, ds_j = sigma_j (1 - sigma_j) (dg_j - gdg) / S;
-// dx_t += sum_j ds_j W_r[:, e_j] (after the grouped dx GEMM, same stream; the k columns
-// advance together), and ds_j into ds[t][e_j] (bf16, the rest of the row already zero).
+// dx_t += sum_j ds_j W_r[:, e_j] (after the grouped dx GEMM, same stream; four columns a
+// lane and the k experts' loads together, 16 bytes each: with scalar loads the chain of
+// d / 32 latencies took 42 us at T = 8192, d = 1024), and ds_j into ds[t][e_j] (bf16, the rest
+// of the row already zero).
 template <int KB>
 __global__ void __launch_bounds__(256) bwd_router_kernel(
     const int32_t* __restrict__ idx, const float* __restrict__ sig, const float* __restrict__ gate,
@@ -291,20 +294,31 @@ __global__ void __launch_bounds__(256) bwd_router_kernel(
     const float gdg = warp_sum_f(g * dg);
     const float ds = lane < k ? sg * (1.f - sg) * (dg - gdg) / S : 0.f;
     if (lane < k && e >= 0 && e < E) ds_out[t * Ep + e] = __float2bfloat16_rn(ds);
-    const float* w[KB];
+    const float* w[KB];   // past k and for bad ids: any row, with factor 0 and not added
     float dsj[KB];
+    uint32_t okm = 0;
 #pragma unroll
     for (int j = 0; j < KB; ++j) {
         dsj[j] = __shfl_sync(0xffffffffu, ds, j);
         const int ej = __shfl_sync(0xffffffffu, e, j);
-        w[j] = (j < k && ej >= 0 && ej < E) ? wrt + (int64_t)ej * dp : nullptr;
+        const bool ok = j < k && ej >= 0 && ej < E;
+        if (ok) okm |= 1u << j;
+        w[j] = wrt + (int64_t)(ok ? ej : 0) * dp;
     }
-    float* dxr = dx + t * d;
-    for (int i = lane; i < d; i += 32) {
-        float a = dxr[i];
+    float4* dxr = reinterpret_cast<float4*>(dx + t * d);   // d % 8 == 0, rows 16-byte aligned
+    for (int i = lane; i < d / 4; i += 32) {
+        float4 a = dxr[i];
+        float4 v[KB];
+#pragma unroll
+        for (int j = 0; j < KB; ++j) v[j] = __ldg(reinterpret_cast<const float4*>(w[j]) + i);
 #pragma unroll
         for (int j = 0; j < KB; ++j)
-            if (w[j]) a = fmaf(dsj[j], __ldg(w[j] + i), a);
+            if ((okm >> j) & 1u) {
+                a.x = fmaf(dsj[j], v[j].x, a.x);
+                a.y = fmaf(dsj[j], v[j].y, a.y);
+                a.z = fmaf(dsj[j], v[j].z, a.z);
+                a.w = fmaf(dsj[j], v[j].w, a.w);
+            }
         dxr[i] = a;
     }
 }
@@ -332,15 +346,17 @@ cudaError_t launch_bwd_gates(const __nv_bfloat16* x, const float* wrt, int dp, c
                              int d, int E, int k, float* sig, float* gate, DevStatus* st, cudaStream_t s) {
     const dim3 grid((unsigned)((T * 32 + 255) / 256));
     cudaError_t e;
-    if (k <= 8) e = launch_pdl(bwd_gates_kernel<8>, grid, dim3(256), 0, s, x, wrt, dp, idx, T, d, E, k, sig, gate, st);
+    if (k <= 4) e = launch_pdl(bwd_gates_kernel<4>, grid, dim3(256), 0, s, x, wrt, dp, idx, T, d, E, k, sig, gate, st);
+    else if (k <= 8) e = launch_pdl(bwd_gates_kernel<8>, grid, dim3(256), 0, s, x, wrt, dp, idx, T, d, E, k, sig, gate, st);
     else if (k <= 32) e = launch_pdl(bwd_gates_kernel<32>, grid, dim3(256), 0, s, x, wrt, dp, idx, T, d, E, k, sig, gate, st);
     else return cudaErrorInvalidValue;
     count_launches(1);
     return e;
 }
 
-cudaError_t launch_bwd_pad(const int32_t* counts, int E, int32_t* poff, cudaStream_t s) {
-    const cudaError_t e = launch_pdl(bwd_pad_kernel, dim3(1), dim3(1024), 0, s, counts, E, poff);
+cudaError_t launch_bwd_plan(const BwdPlan& p, cudaStream_t s) {
+    if (p.E > 1024 || p.nsets < 0 || p.nsets > BWD_MAX_SETS) return cudaErrorInvalidValue;
+    const cudaError_t e = launch_pdl(bwd_plan_kernel, dim3(1 + p.nsets), dim3(1024), 0, s, p);
     count_launches(1);
     return e;
 }
@@ -360,23 +376,15 @@ int64_t bwd_max_items(int64_t rows, int G, int M, int N, int BN) {
     return ((rows + GM_BK * BWD_KCH - 1) / (GM_BK * BWD_KCH) + G) * mt * nt;
 }
 
-cudaError_t launch_bwd_items(const int32_t* koff, int G, int64_t K_rows, int M, int N, int BN,
-                             int max_items, int4* items, int32_t* n_items, int32_t* gclear, DevStatus* st,
-                             cudaStream_t s) {
-    if (G > 1024) return cudaErrorInvalidValue;
-    const cudaError_t e = launch_pdl(bwd_items_kernel, dim3(1), dim3(1024), 0, s, koff, G, K_rows, M, N, BN,
-                                     (int)BWD_KCH, max_items, items, n_items, gclear, st);
-    count_launches(1);
-    return e;
-}
-
-cudaError_t launch_bwd_zero(const int32_t* gclear, int G, int M, int N, int64_t ld, float* out, int num_sms,
-                            cudaStream_t s) {
-    if (ld % 4 != 0 || N > ld) return cudaErrorInvalidValue;
-    const int64_t warps = (int64_t)G * M;
-    const int64_t blocks = std::min<int64_t>((warps + 7) / 8, (int64_t)num_sms * 8);
-    const cudaError_t e = launch_pdl(bwd_zero_kernel, dim3((unsigned)std::max<int64_t>(blocks, 1)), dim3(256), 0, s,
-                                     gclear, G, M, N, ld, out);
+cudaError_t launch_bwd_zero(const BwdZero& z, int num_sms, cudaStream_t s) {
+    int64_t rows = 1;
+    for (int j = 0; j < z.njobs; ++j) {
+        if (z.jobs[j].ld % 4 != 0 || z.jobs[j].N > z.jobs[j].ld) return cudaErrorInvalidValue;
+        rows = std::max<int64_t>(rows, (int64_t)z.jobs[j].G * z.jobs[j].M);
+    }
+    if (z.njobs < 1 || z.njobs > BWD_MAX_ZERO) return cudaErrorInvalidValue;
+    const int64_t blocks = std::min<int64_t>((rows + 7) / 8, (int64_t)num_sms * 8);
+    const cudaError_t e = launch_pdl(bwd_zero_kernel, dim3((unsigned)blocks, (unsigned)z.njobs), dim3(256), 0, s, z);
     count_launches(1);
     return e;
 }
@@ -396,7 +404,10 @@ cudaError_t launch_bwd_router(const int32_t* idx, const float* sig, const float*
                               cudaStream_t s) {
     const dim3 grid((unsigned)((T * 32 + 255) / 256));
     cudaError_t e;
-    if (k <= 8)
+    if (k <= 4)
+        e = launch_pdl(bwd_router_kernel<4>, grid, dim3(256), 0, s, idx, sig, gate, slot_prow, dg_part, nparts,
+                       part_stride, wrt, dp, T, d, E, k, Ep, dx, ds);
+    else if (k <= 8)
         e = launch_pdl(bwd_router_kernel<8>, grid, dim3(256), 0, s, idx, sig, gate, slot_prow, dg_part, nparts,
                        part_stride, wrt, dp, T, d, E, k, Ep, dx, ds);
     else if (k <= 32)

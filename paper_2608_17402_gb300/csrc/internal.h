@@ -337,24 +337,47 @@ constexpr int BWD_STORE_BIT = 1 << 30;
 // copy wrt [E][dp]) and gate = sig / sum_j sig (k <= 32).
 cudaError_t launch_bwd_gates(const __nv_bfloat16* x, const float* wrt, int dp, const int32_t* idx, int64_t T,
                              int d, int E, int k, float* sig, float* gate, DevStatus* st, cudaStream_t s);
-// poff[E + 1]: exclusive prefix of counts rounded up to multiples of 64 (E <= 1024).
-cudaError_t launch_bwd_pad(const int32_t* counts, int E, int32_t* poff, cudaStream_t s);
+// One weight-gradient item table of the plan (bwd_plan_kernel): the gradient [G][M][N] of
+// the experts' padded rows, or with dense_rows > 0 of one group of that many rows.
+constexpr int BWD_MAX_SETS = 5;
+struct BwdItemSet {
+    int M, N, BN, max_items;
+    int64_t dense_rows;
+    int4* items;
+    int32_t* n_items;
+    int32_t* gclear;   // per group: 1 = its gradient is cleared first
+};
+struct BwdPlan {
+    const int32_t* counts;   // rows per expert
+    int E, nsets;
+    int32_t* poff;           // [E + 1] exclusive prefix of counts rounded up to multiples of 64
+    int4* tiles;             // m-tile table of the padded rows
+    int32_t* n_tiles;
+    DevStatus* st;
+    BwdItemSet sets[BWD_MAX_SETS];
+};
+cudaError_t launch_bwd_plan(const BwdPlan& p, cudaStream_t s);
 // Padded rows: ptok / pgate of every padded row (-1 / 0 for padding) and the padded row
 // of every routing slot (from the stable expert-major rows inv and offsets).
 cudaError_t launch_bwd_rows(const int32_t* idx, const int32_t* inv, const int32_t* counts,
                             const int32_t* offsets, const int32_t* poff, const float* gate, int64_t n_slots,
                             int k, int E, int32_t* ptok, float* pgate, int32_t* slot_prow, cudaStream_t s);
-// Weight-gradient work items (see bwd_items_kernel) and a bound on their number for
-// groups holding `rows` rows in total.
+// A bound on the weight-gradient items of groups holding `rows` rows in total.
 int64_t bwd_max_items(int64_t rows, int G, int M, int N, int BN);
-cudaError_t launch_bwd_items(const int32_t* koff, int G, int64_t K_rows, int M, int N, int BN,
-                             int max_items, int4* items, int32_t* n_items, int32_t* gclear, DevStatus* st,
-                             cudaStream_t s);
-// Clears what the weight-gradient items will not write of out [G][M][ld] (fp32): the
-// groups with gclear[g] set (no rows, or several chunks adding up), and the pad columns
-// [N, ld) of the others.
-cudaError_t launch_bwd_zero(const int32_t* gclear, int G, int M, int N, int64_t ld, float* out, int num_sms,
-                            cudaStream_t s);
+// Buffers cleared by one launch of bwd_zero_kernel: of out [G][M][ld] (fp32) the groups with
+// gclear[g] set (all when gclear is null) and the pad columns [N, ld) of the others.
+constexpr int BWD_MAX_ZERO = 9;
+struct BwdZeroJob {
+    const int32_t* gclear;
+    int G, M, N;
+    int64_t ld;
+    float* out;
+};
+struct BwdZero {
+    int njobs;
+    BwdZeroJob jobs[BWD_MAX_ZERO];
+};
+cudaError_t launch_bwd_zero(const BwdZero& z, int num_sms, cudaStream_t s);
 // xp[r] = x[ptok[r]], gdy[r] = pgate[r] dy[ptok[r]] over the poff[E] padded rows.
 cudaError_t launch_bwd_gather(const __nv_bfloat16* x, const __nv_bfloat16* dy, const int32_t* ptok,
                               const float* pgate, const int32_t* poff, int E, int d, int64_t max_rows,
@@ -398,7 +421,6 @@ void* current_context();
 
 // ------------------------------------------------------------------- misc
 
-cudaError_t launch_zero_f32(float* p, int64_t n, cudaStream_t s);
 cudaError_t launch_f32_to_bf16(const float* src, __nv_bfloat16* dst, int64_t n, cudaStream_t s);
 // Loss-free bias update (Eq. 9 z-score, rule 0; Eq. 8 sign, rule 1) from counts[E], E <= 1024.
 cudaError_t launch_update_bias(const int32_t* counts, int E, float alpha, int rule, float* b,

@@ -1,5 +1,4 @@
 // misc.cu -- memory-bound helper kernels of the MoE-ViE layer, sm_103a.
-//   zero_f32_kernel      y accumulator := 0 (float4 stores)
 //   f32_to_bf16_kernel   y := bf16(y accumulator)  (32-byte loads, 16-byte stores)
 //   combine_kernel       Eq. (6) as a stand-alone gather-reduce over expert-major
 //                        rows: y[t] = sum_j gate[t, j] rows[inv[t*k + j]] + lambda * shared[t]
@@ -9,14 +8,6 @@
 namespace mv {
 
 namespace {
-
-__global__ void zero_f32_kernel(float4* __restrict__ p, int64_t n4) {
-    pdl_wait();
-    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n4;
-         i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = z;
-}
 
 // n8 groups of 8 values.
 __global__ void f32_to_bf16_kernel(const float4* __restrict__ src, uint4* __restrict__ dst,
@@ -192,15 +183,6 @@ int grid_for(int64_t n, int threads) {
 }
 
 }  // namespace
-
-cudaError_t launch_zero_f32(float* p, int64_t n, cudaStream_t s) {
-    const int64_t n4 = n / 4;   // callers pass multiples of 4
-    cudaError_t e = launch_pdl(zero_f32_kernel, dim3(grid_for(n4, 256)), dim3(256), 0, s,
-                               reinterpret_cast<float4*>(p), n4);
-    if (e != cudaSuccess) return e;
-    count_launches(1);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_f32_to_bf16(const float* src, __nv_bfloat16* dst, int64_t n, cudaStream_t s) {
     const int64_t n8 = n / 8;   // callers pass multiples of 8
