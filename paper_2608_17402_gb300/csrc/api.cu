@@ -748,8 +748,8 @@ static moevie_status forward_impl(const moevie_layer* Lr, const void* x, int64_t
     float* gate = r.gate ? r.gate : at<float>(ws, L.gate);
     int32_t* counts = r.counts ? r.counts : at<int32_t>(ws, L.counts);
     int32_t* offsets = r.offsets ? r.offsets : at<int32_t>(ws, L.offsets);
-    int32_t* perm = r.perm ? r.perm : at<int32_t>(ws, L.perm);
-    int32_t* inv = r.inv ? r.inv : at<int32_t>(ws, L.inv);
+    int32_t* perm = r.perm;   // by-products: written when asked for (the layer reads row_tok)
+    int32_t* inv = r.inv;
     if (!a16(idx)) return MOEVIE_ERR_INVALID_ARG;
     int4* tiles = at<int4>(ws, L.tiles);
     int32_t* n_tiles = at<int32_t>(ws, L.n_tiles);

@@ -49,6 +49,27 @@ cudaError_t launch_pdl_coop(void (*kern)(KArgs...), dim3 grid, dim3 block, size_
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
+// The same for clusters of `size` CTAs.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_cluster(void (*kern)(KArgs...), int size, dim3 grid, dim3 block, size_t smem,
+                               cudaStream_t s, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)size;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
 // ----------------------------------------------------------------- router
 
 // Error model of the fast logits used to decide when a token's selection must be
@@ -139,7 +160,8 @@ struct SharedRows {
 
 // Stable expert-major order; also writes the m-tile table of the grouped GEMMs
 // (tiles[i] = {expert, first row, rows, 0}, *n_tiles = their number), followed by the
-// tiles and rows of the always-on groups `sh` describes (none when sh is null).
+// tiles and rows of the always-on groups `sh` describes (none when sh is null).  perm and inv
+// may be null (not wanted).
 cudaError_t launch_permute(const int32_t* idx, int64_t n_slots, int k, int E, int bm, int chunk,
                            const float* gate_flat, int32_t* hist, int32_t* counts,
                            int32_t* offsets, int4* tiles, int32_t* n_tiles, int32_t* perm,
