@@ -296,6 +296,8 @@ moevie_status run_gemm(const GemmSpec& g, DevStatus* st, cudaStream_t s) {
                                             a.trans ? GM_ROW_BOX : GM_HALF)) {
         return MOEVIE_ERR_CUDA;
     }
+    if (a.trans && !make_rows_tmap(&a.tmA2, g.A, g.a_cols > 0 ? g.a_cols : g.K, g.a_nrows, g.lda, GM_HALF))
+        return MOEVIE_ERR_CUDA;
     a.b_kmajor = g.b_kmajor ? 1 : 0;
     a.a_mn = g.a_mn ? 1 : 0;
     a.wg_M = g.wg_M;

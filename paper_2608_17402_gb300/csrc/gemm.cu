@@ -38,7 +38,7 @@
 //   warp 18     lane 0: waits for afull, fences the stage to the async proxy and
 //               publishes it on the leader's full barrier (from the peer: a 16-byte
 //               bulk copy that completes transaction bytes there)
-// Shared memory: 7 stages (6 plus a reduction staging buffer for the y-accumulator
+// Shared memory: 6 stages and an epilogue buffer (5 for the activation-derivative
 // epilogue) x (A 128x64 + B 64x128) bf16; TMEM: two fp32 accumulators
 // of 256 columns, so the epilogue of one tile overlaps the main loop of the next.
 //
@@ -332,9 +332,11 @@ __device__ __forceinline__ int trans_n(const Tile& t) { return t.nrows > 64 ? (t
 // every np-th one.  The byte-count arrival, the copies and the wait of one stage are a chain
 // of about 725 cycles in one warp (clock sums in the kernel), longer than the 512 cycles of
 // the stage's MMAs: two producers took the down-projection at T = 8192, d = 1280, h = 854
-// from 141 to 137 us.  With gathered A, where the gather paces the ring, one is enough.  The leader posts the byte count of both CTAs on its full barrier.
-template <bool GATHER, bool TRAIN, bool ONE, bool TRANS>
-__device__ void producer_tma(const GemmArgs& p, const Smem& sm, int64_t n_work, int pid, int np,
+// from 141 to 137 us.  With gathered A a second producer slowed small launches; the one there
+// issues two stages at once when both are free (up-projection of that layer 203 -> 199 us).
+// The leader posts the byte count of both CTAs on its full barrier.
+template <bool GATHER, bool TRAIN, bool ONE, bool TRANS, int NP>
+__device__ void producer_tma(const GemmArgs& p, const Smem& sm, int64_t n_work, int pid,
                              volatile int* abort_flag) {
     tma_prefetch_desc(&p.tmB);
     if (p.g_split < p.G || p.swiglu) tma_prefetch_desc(&p.tmB2);
@@ -342,16 +344,16 @@ __device__ void producer_tma(const GemmArgs& p, const Smem& sm, int64_t n_work, 
         tma_prefetch_desc(&p.tmB3);
         tma_prefetch_desc(&p.tmB4);
     }
-    constexpr bool gather = GATHER;
-    if (!gather) tma_prefetch_desc(&p.tmA);
+    if (!GATHER) tma_prefetch_desc(&p.tmA);
+    if (TRANS) tma_prefetch_desc(&p.tmA2);
     const uint32_t half_n = (uint32_t)p.BN / 2;
     const uint32_t nboxh = (half_n + 63) / 64;
     // B per CTA and stage: nboxh boxes of 64 columns x 64 K rows (N-major), or half_n rows
     // of 64 K values (K-major)
     const uint32_t b_bytes = (TRAIN && p.b_kmajor) ? half_n * 128u : nboxh * GM_BK * 128;
-    const uint32_t cta_bytes = b_bytes + (gather ? 0u : (uint32_t)GM_A_BYTES);
+    const uint32_t cta_bytes = b_bytes + (GATHER ? 0u : (uint32_t)GM_A_BYTES);
     // gathering: plus the 16-byte signal with which the peer publishes its A half
-    const uint32_t stage_tx = 2 * cta_bytes + (gather ? 16u : 0u);
+    const uint32_t stage_tx = 2 * cta_bytes + (GATHER ? 16u : 0u);
     const uint32_t full_leader = peer_addr(sm.full, 0);
     int s = 0, turn = 0;
     uint32_t ph = 0;
@@ -373,59 +375,72 @@ __device__ void producer_tma(const GemmArgs& p, const Smem& sm, int64_t n_work, 
         const int gb = (TRAIN && p.item_table == 2) ? 0 : (tail ? t.g - p.g_split : t.g);
         const int ncol0 = p.swiglu ? t.n0 : t.n0 + (int)(sm.rank * (TRANS ? (uint32_t)GM_HALF : half_n));
         const int rhalf = TRANS ? trans_n(t) / 2 : 0;   // rows of the CTA's half of the transposed B
+        const int row = t.row0 + (int)sm.rank * (TRANS ? rhalf : GM_HALF);
+        auto issue = [&](int st, int kb) {   // one lane: the byte count and the copies of k-block kb into stage st
+            const uint32_t bar = full_leader + 8 * st;
+            const uint32_t a_dst = sm.a0 + st * GM_A_BYTES, b_dst = sm.b0 + st * GM_B_BYTES;
+            const int kk = kb * GM_BK;
+            if (TRANS) {
+                if (sm.rank == 0)
+                    mbar_arrive_expect_tx(sm.full + 8 * st, 2u * (uint32_t)(GM_A_BYTES + rhalf * 128));
+                if (TRAIN && p.b_kmajor) {   // 128 output columns' rows of 64 K values
+                    tma_load_3d_pair(a_dst, tmb, bar, kk, ncol0, gb);
+                } else {                     // two boxes of 64 columns x 64 K rows
+                    tma_load_3d_pair(a_dst, tmb, bar, ncol0, kk, gb);
+                    tma_load_3d_pair(a_dst + GM_BK * 128, tmb, bar, ncol0 + 64, kk, gb);
+                }
+                if (rhalf == GM_HALF) {
+                    tma_load_2d_pair(b_dst, &p.tmA2, bar, kk, row);
+                } else {
+                    for (int j = 0; j < rhalf; j += GM_ROW_BOX)
+                        tma_load_2d_pair(b_dst + j * 128, &p.tmA, bar, kk, row + j);
+                }
+                return;
+            }
+            if (sm.rank == 0) mbar_arrive_expect_tx(sm.full + 8 * st, stage_tx);
+            if (TRAIN && p.b_kmajor) {   // half_n rows of the CTA's columns, 64 K values each
+                tma_load_3d_pair(b_dst, tmb, bar, kk, ncol0, gb);
+            } else {
+                for (uint32_t j = 0; j < nboxh; ++j)
+                    tma_load_3d_pair(b_dst + j * (GM_BK * 128), tmb, bar, ncol0 + (int)(64 * j), kk, gb);
+            }
+            if (GATHER) return;
+            if (TRAIN && p.a_mn) {   // two 64-row halves of the CTA's 128 output rows, 64 K rows each
+                const int m = t.m0 + (int)sm.rank * GM_HALF;
+                tma_load_3d_pair(a_dst, &p.tmA, bar, m, kk, 0);
+                tma_load_3d_pair(a_dst + GM_BK * 128, &p.tmA, bar, m + 64, kk, 0);
+            } else {
+                const int col = p.a_kperiod ? kk % p.a_kperiod : kk;
+                tma_load_2d_pair(a_dst, &p.tmA, bar, col, row);
+            }
+        };
         for (int kb = t.kb0; kb < t.kb1; ++kb) {
-            if (turn == pid) {
+            if (NP == 1 || turn == pid) {
                 if (!mbar_wait_warp<ONE>(sm.empty + 8 * s, ph ^ 1u, p.limit_ns, abort_flag, ready)) {
                     set_abort(abort_flag, p.status, SITE_GEMM_WAIT_EMPTY, (int)sm.pair, 1);
                     return;
                 }
-                if (TRANS && elect_one()) {
-                    const uint32_t bar = full_leader + 8 * s;
-                    if (sm.rank == 0)
-                        mbar_arrive_expect_tx(sm.full + 8 * s, 2u * (uint32_t)(GM_A_BYTES + rhalf * 128));
-                    const int kk = kb * GM_BK;
-                    const uint32_t a_dst = sm.a0 + s * GM_A_BYTES, b_dst = sm.b0 + s * GM_B_BYTES;
-                    if (TRAIN && p.b_kmajor) {   // 128 output columns' rows of 64 K values
-                        tma_load_3d_pair(a_dst, tmb, bar, kk, ncol0, gb);
-                    } else {                     // two boxes of 64 columns x 64 K rows
-                        tma_load_3d_pair(a_dst, tmb, bar, ncol0, kk, gb);
-                        tma_load_3d_pair(a_dst + GM_BK * 128, tmb, bar, ncol0 + 64, kk, gb);
-                    }
-                    const int row = t.row0 + (int)sm.rank * rhalf;
-                    for (int j = 0; j < rhalf; j += GM_ROW_BOX)
-                        tma_load_2d_pair(b_dst + j * 128, &p.tmA, bar, kk, row + j);
-                }
-                if (!TRANS && elect_one()) {
-                    const uint32_t bar = full_leader + 8 * s;
-                    if (sm.rank == 0) mbar_arrive_expect_tx(sm.full + 8 * s, stage_tx);
-                    const uint32_t b_dst = sm.b0 + s * GM_B_BYTES;
-                    const int kk = kb * GM_BK;
-                    if (TRAIN && p.b_kmajor) {   // half_n rows of the CTA's columns, 64 K values each
-                        tma_load_3d_pair(b_dst, tmb, bar, kk, ncol0, gb);
-                    } else {
-                        for (uint32_t j = 0; j < nboxh; ++j)
-                            tma_load_3d_pair(b_dst + j * (GM_BK * 128), tmb, bar, ncol0 + (int)(64 * j), kk, gb);
-                    }
-                    if (!gather) {
-                        if (TRAIN && p.a_mn) {   // two 64-row halves of the CTA's 128 output rows, 64 K rows each
-                            const int m = t.m0 + (int)sm.rank * GM_HALF;
-                            tma_load_3d_pair(sm.a0 + s * GM_A_BYTES, &p.tmA, bar, m, kk, 0);
-                            tma_load_3d_pair(sm.a0 + s * GM_A_BYTES + GM_BK * 128, &p.tmA, bar, m + 64, kk, 0);
-                        } else {
-                            const int col = p.a_kperiod ? kk % p.a_kperiod : kk;
-                            tma_load_2d_pair(sm.a0 + s * GM_A_BYTES, &p.tmA, bar, col,
-                                             t.row0 + (int)sm.rank * GM_HALF);
-                        }
-                    }
+                // the next stage with this one when it is free already
+                const int s2 = s + 1 == sm.nstages ? 0 : s + 1;
+                const bool two = NP == 1 && !ONE && kb + 1 < t.kb1 &&
+                                 __all_sync(0xffffffffu, mbar_test(sm.empty + 8 * s2, (s2 ? ph : ph ^ 1u) ^ 1u));
+                if (elect_one()) {
+                    issue(s, kb);
+                    if (two) issue(s2, kb + 1);
                 }
                 __syncwarp();
+                if (two) {
+                    s = s2;
+                    if (s == 0) ph ^= 1u;
+                    ++kb;
+                }
             }
-            if (++turn == np) turn = 0;
+            if (++turn == NP) turn = 0;
             if (++s == sm.nstages) {
                 s = 0;
                 ph ^= 1u;
             }
-            ready = !ONE && turn == pid && mbar_test(sm.empty + 8 * s, ph ^ 1u);
+            ready = !ONE && (NP == 1 || turn == pid) && mbar_test(sm.empty + 8 * s, ph ^ 1u);
         }
         if (wn < n_work) t = tile_finish(p, nl);
     }
@@ -1256,7 +1271,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) grouped_gemm_kernel(const __gri
     } else if (warp == GM_WARP_MMA) {
         if (sm.rank == 0) mma_issuer<TRAIN, ECLS == ECLS_F32, ECLS == ECLS_ADDT>(p, sm, tmem, n_work, abort_flag);
     } else if (prod_id >= 0) {
-        producer_tma<GATHER, TRAIN, ECLS == ECLS_F32, ECLS == ECLS_ADDT>(p, sm, n_work, prod_id, NPROD, abort_flag);
+        producer_tma<GATHER, TRAIN, ECLS == ECLS_F32, ECLS == ECLS_ADDT, NPROD>(p, sm, n_work, prod_id, abort_flag);
     } else if (GATHER && warp == GM_WARP_FWD) {
         if constexpr (GATHER) gather_forwarder(p, sm, n_work, abort_flag);
     } else if (GATHER && warp >= GM_WARP_GATHER && warp < GM_WARP_FWD) {

@@ -266,6 +266,7 @@ struct GemmArgs {
     CUtensorMap tmA;            // A = rows [a_nrows][K_A] bf16, 2-D map {K_A, a_nrows}, box
                                 // {64, 128} ({64, 32} with trans); used when A rows are
                                 // contiguous (a_rows == nullptr)
+    CUtensorMap tmA2;           // trans: the same rows with box {64, 128}, for full tiles
     int trans;                  // EPI_ADD_F32 of rows without an item table: D^T = B^T A^T, output
                                 //   columns along the MMA's M, rows along its N (epilogue_addt)
     const __nv_bfloat16* A;     // A rows, for the token gather
