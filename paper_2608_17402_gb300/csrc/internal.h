@@ -184,7 +184,7 @@ cudaError_t launch_item_order(const int4* tiles, const int32_t* n_tiles, const i
 constexpr int GM_BM = 256;        // rows per m-tile: one CTA pair, 128 rows per CTA
 constexpr int GM_HALF = 128;      // rows per CTA (tcgen05 M = 256 across the pair)
 constexpr int GM_BK = 64;         // K per stage: 64 bf16 = one 128-byte swizzle row
-constexpr int GM_STAGES_MAX = 7;   // operand ring depth (6 when the reduction staging is needed)
+constexpr int GM_STAGES_MAX = 6;   // operand ring depth (5 beside the largest epilogue buffers)
 constexpr int GM_MAXBN = 256;     // largest N of one tcgen05.mma
 constexpr int GM_EPI_WARPS = 8;   // two warps per TMEM lane quadrant, alternate 32-column chunks
 constexpr int GM_WARP_MMA = GM_EPI_WARPS;        // TMEM allocation + tcgen05.mma issue
@@ -213,19 +213,21 @@ enum { ECLS_BF16 = 0, ECLS_F32 = 1, ECLS_ADD = 2, ECLS_ADDT = 3, ECLS_DGELU = 4,
 constexpr int GM_ADDT_PARTS = 4;
 static_assert(4 * GM_ADDT_PARTS == GM_EPI_WARPS + GM_GATHER_WARPS, "the gather warps join the epilogue");
 // Shared memory beside the operand ring: the bf16 outputs pass 32 columns (training path: 16
-// of up to three arrays) of 32 rows per warp, ECLS_ADD stages 16 rows per warp, ECLS_ADDT keeps
-// the {token, scale} pairs of 32 rows per warp; each gives up one of the 7 stages.  The
-// activation derivatives buffer two 16-column steps of u, a (and v) per warp, two stages.
+// of up to three arrays) of 32 rows per warp, the fp32 stores 32 columns of 32 rows, ECLS_ADD
+// stages 16 rows per warp, ECLS_ADDT keeps the {token, scale} pairs of 32 rows per warp: six
+// stages fit beside them.  The activation derivatives buffer two 16-column steps of u, a (and
+// v) per warp: five.
 __host__ __device__ constexpr int gm_bf16_warp_bytes(bool train) { return train ? 3 * 32 * 32 : 32 * 64; }
 __host__ __device__ constexpr int gm_stg_bytes(int ecls, bool train) {
     return ecls == ECLS_BF16 ? GM_EPI_WARPS * gm_bf16_warp_bytes(train)
+           : ecls == ECLS_F32 ? GM_EPI_WARPS * 32 * 128
            : ecls == ECLS_ADD ? GM_EPI_WARPS * GM_STG_ROWS * GM_STG_LD * 4
            : ecls == ECLS_ADDT ? 4 * GM_ADDT_PARTS * 32 * 8
            : ecls == ECLS_DGELU ? GM_EPI_WARPS * 2 * 2 * 1024
            : ecls == ECLS_DSWIGLU ? GM_EPI_WARPS * 2 * 3 * 1024 : 0;
 }
 __host__ __device__ constexpr int gm_stages(int ecls, bool) {
-    return ecls == ECLS_DGELU || ecls == ECLS_DSWIGLU ? 5 : ecls == ECLS_F32 ? 7 : 6;
+    return ecls == ECLS_DGELU || ecls == ECLS_DSWIGLU ? 5 : 6;
 }
 __host__ __device__ constexpr int gm_smem_bytes(int ecls, bool train) {
     return gm_stages(ecls, train) * (GM_A_BYTES + GM_B_BYTES) + gm_stg_bytes(ecls, train) + GM_OVERHEAD_BYTES;
