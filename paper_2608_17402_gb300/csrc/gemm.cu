@@ -304,8 +304,7 @@ struct Smem {
     uint32_t drain;
     uint32_t sink;            // 16 bytes: target / source of the peer's stage signals
     int nstages;              // operand ring depth of this launch
-    float* stg;               // ECLS_ADD: GM_STG_ROWS staged rows of GM_STG_LD floats per warp;
-                              // ECLS_ADDT: 32 {token, scale} pairs per warp
+    float* stg;               // the epilogue's buffers (gm_stg_bytes)
     uint32_t rank;            // rank of this CTA in its pair
     int64_t pair, npairs;     // pair index and count
 };
@@ -666,44 +665,6 @@ __device__ void mma_issuer(const GemmArgs& p, const Smem& sm, uint32_t tmem, int
 
 // -------------------------------------------------------------- epilogue
 
-// One 32-column chunk of the staged reductions (band-ordered rows, weight gradients) of one
-// warp: each lane holds its row's 32 values; GM_STG_ROWS rows at a time go to the warp's staging
-// buffer, scaled and with the row's offset; then
-// every lane reduces 4 columns of one of 4 rows per instruction, so 8 lanes cover a
-// row's 128 contiguous bytes (a whole L2 line).
-__device__ __forceinline__ void reduce_chunk(const GemmArgs& p, float* stg_all, int warp, int lane,
-                                             const uint32_t (&v)[32], float sc, int64_t my_yoff,
-                                             int n, bool store) {
-    constexpr int ROWS = GM_STG_ROWS;
-    float* stg = stg_all + warp * (ROWS * GM_STG_LD);
-    const int col = n + 4 * (lane & 7);
-#pragma unroll
-    for (int hh = 0; hh < 32 / ROWS; ++hh) {
-        if (lane / ROWS == hh) {
-            float* row = stg + (lane - hh * ROWS) * GM_STG_LD;
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                *reinterpret_cast<float4*>(row + 4 * c) =
-                    make_float4(sc * __uint_as_float(v[4 * c]), sc * __uint_as_float(v[4 * c + 1]),
-                                sc * __uint_as_float(v[4 * c + 2]), sc * __uint_as_float(v[4 * c + 3]));
-            *reinterpret_cast<int64_t*>(row + 32) = my_yoff;
-        }
-        __syncwarp();
-#pragma unroll
-        for (int r = 0; r < ROWS / 4; ++r) {
-            const float* row = stg + (4 * r + (lane >> 3)) * GM_STG_LD;
-            const int64_t yo = *reinterpret_cast<const int64_t*>(row + 32);
-            const float4 val = *reinterpret_cast<const float4*>(row + 4 * (lane & 7));
-            if (yo >= 0 && col < p.N) {
-                float4* dst = reinterpret_cast<float4*>(p.yacc + yo + col);
-                if (store) *dst = val;   // the only contribution to these elements
-                else atomicAdd(dst, val);
-            }
-        }
-        __syncwarp();
-    }
-}
-
 // Epilogue of the transposed product (EPI_ADD_F32 of rows): the accumulator holds D^T, so
 // TMEM lane l of the CTA is output column n0 + 128 rank + l and TMEM column j is row j of
 // the tile.  A warp takes 32 columns and every fourth chunk of 32 rows; register i of all
@@ -817,44 +778,47 @@ __device__ void epilogue_addt(const GemmArgs& p, const Smem& sm, uint32_t tmem, 
     }
 }
 
-// One 32-column chunk of fp32 stores of one warp: each lane holds its row's 32 values (scaled
-// by sc; tok < 0: no row); the 32 rows pass the warp's buffer (16-byte piece q of row r at
-// r * 128 + 16 (q ^ (r & 7)): no bank conflicts either way) so that eight lanes store the
-// 128 contiguous bytes of a row.  Stored by each lane from its own registers the pieces of 32
-// different lines an instruction held the router GEMM up: moevie_route at T = 65536, E = 256
-// 235 -> 219 us, at T = 32768, E = 128 92.0 -> 86.7.
-__device__ __forceinline__ void store_chunk(const GemmArgs& p, uint8_t* buf, int lane, const float (&f)[32], float sc,
-                                            int tok, int64_t base, int col0, int ncols) {
+// One 32-column chunk of the fp32 outputs of one warp: each lane holds its row's 32 values
+// (scaled by sc; tok < 0: no row).  The 32 rows pass the warp's 4 KB buffer (16-byte piece q of
+// row r at r * 128 + 16 (q ^ (r & 7)): no bank conflicts either way), so that eight lanes store
+// or reduce the 128 contiguous bytes of a row, whole L2 lines.  Stored by each lane from its own
+// registers the pieces of 32 different lines an instruction held the router GEMM up:
+// moevie_route at T = 65536, E = 256 235 -> 219 us, at T = 32768, E = 128 92.0 -> 86.7.  Reduced 16
+// rows at a time through rows of 36 floats (half the lanes idle, bank conflicts) the band-ordered
+// down-projection took 397 us at T = 32768, E = 128, this way 373.
+__device__ __forceinline__ void out_chunk(const GemmArgs& p, uint8_t* buf, int lane, const float (&f)[32], float sc,
+                                          int tok, int64_t base, int col0, int ncols, bool add) {
 #pragma unroll
     for (int q = 0; q < 8; ++q)
         *reinterpret_cast<float4*>(buf + lane * 128 + 16 * (q ^ (lane & 7))) =
             make_float4(sc * f[4 * q], sc * f[4 * q + 1], sc * f[4 * q + 2], sc * f[4 * q + 3]);
     __syncwarp();
     const int q = lane & 7;
+    const bool col_ok = col0 + 4 * q < ncols;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int r = 4 * i + (lane >> 3);
         const int tk = __shfl_sync(0xffffffffu, tok, r);
         const float4 v = *reinterpret_cast<const float4*>(buf + r * 128 + 16 * (q ^ (r & 7)));
-        if (tk >= 0 && col0 + 4 * q < ncols)
-            *reinterpret_cast<float4*>(p.yacc + base + (int64_t)tk * p.ldy + col0 + 4 * q) = v;
+        if (tk >= 0 && col_ok) {
+            float4* dst = reinterpret_cast<float4*>(p.yacc + base + (int64_t)tk * p.ldy + col0 + 4 * q);
+            if (add) atomicAdd(dst, v);
+            else *dst = v;
+        }
     }
     __syncwarp();
 }
 
 // Epilogue of the fp32 outputs.  Warp w reads TMEM lanes 32 (w % 4) .. +31 (its rows) and
-// the 32-column chunks c = w / 4, w / 4 + 2, ... of each tile.  fp32 stores: see store_chunk.
-// fp32 reductions: the rows pass a small
-// per-warp staging buffer so that each 16-byte vector reduction instruction of a
-// warp covers four rows x 128 contiguous bytes, i.e. whole L2 lines.  When a warp has read
-// its last chunk of the accumulator it arrives (once) on the leader's tempty barrier.
+// the 32-column chunks c = w / 4, w / 4 + 2, ... of each tile (out_chunk).  When a warp
+// has read its last chunk of the accumulator it arrives (once) on the leader's tempty barrier.
 template <int ECLS, bool TRAIN>
 __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64_t n_work,
                          volatile int* abort_flag) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int quad = warp & 3, half = warp >> 2;
     const int nchunk = p.BN / 32;
-    uint8_t* buf = reinterpret_cast<uint8_t*>(sm.stg) + warp * 4096;   // ECLS_F32: 32 rows x 128 bytes
+    uint8_t* buf = reinterpret_cast<uint8_t*>(sm.stg) + warp * 4096;   // 32 rows x 128 bytes
     const uint32_t tempty_leader = peer_addr(sm.tempty, 0);
     int it = 0;
     if (sm.pair >= n_work) return;
@@ -909,7 +873,7 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
                 }
 #pragma unroll
                 for (int i = 0; i < 32; ++i) s2[i] += __uint_as_float(v[i]);
-                store_chunk(p, buf, lane, s2, sc, ok_row ? (int)tok : -1, t.ks * p.y_split_stride, ch * 32, p.N / 2);
+                out_chunk(p, buf, lane, s2, sc, ok_row ? (int)tok : -1, t.ks * p.y_split_stride, ch * 32, p.N / 2, false);
             }
             continue;
         }
@@ -920,20 +884,6 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
         }
         for (int ch = half; ch < nchunk; ch += 2) {
             const int c0 = ch * 32;
-            if constexpr (ECLS == ECLS_ADD) {   // staged reductions
-                uint32_t v[32];
-                tmem_ld_32x32b_x32(tbase + c0, v);
-                tmem_wait_ld();
-                if (ch + 2 >= nchunk) {   // this warp's last read of the accumulator
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive_remote(tempty_leader + 8 * acc);
-                }
-                const int n = t.n0 + c0;
-                const int64_t my_yoff = ok_row ? t.ks * p.y_split_stride + tok * p.ldy : -1;
-                reduce_chunk(p, sm.stg, warp, lane, v, sc, my_yoff, n, TRAIN && t.store);
-                continue;
-            }
             uint32_t v[32];
             tmem_ld_32x32b_x32(tbase + c0, v);
             tmem_wait_ld();
@@ -945,7 +895,9 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
             float f[32];
 #pragma unroll
             for (int i = 0; i < 32; ++i) f[i] = __uint_as_float(v[i]);
-            store_chunk(p, buf, lane, f, sc, ok_row ? (int)tok : -1, t.ks * p.y_split_stride, t.n0 + c0, p.N);
+            // weight-gradient items that are their tile's only one store instead of adding
+            out_chunk(p, buf, lane, f, sc, ok_row ? (int)tok : -1, t.ks * p.y_split_stride, t.n0 + c0, p.N,
+                      ECLS == ECLS_ADD && !(TRAIN && t.store));
         }
     }
 }

@@ -199,8 +199,6 @@ constexpr int GM_GATHER_RSTEP = GM_GATHER_WARPS * 32 / 8;
 constexpr int GM_GATHER_ROWS = 128 / GM_GATHER_RSTEP;
 constexpr int GM_A_BYTES = GM_HALF * GM_BK * 2;           // one CTA's A rows per stage
 constexpr int GM_B_BYTES = GM_BK * (GM_MAXBN / 2) * 2;    // one CTA's half of B per stage
-constexpr int GM_STG_ROWS = 16;    // ECLS_ADD: rows per warp in the reduction staging buffer
-constexpr int GM_STG_LD = 36;      // floats per staged row: 32 values, the row's y offset, pad
 constexpr int GM_OVERHEAD_BYTES = 1024 + 512;   // alignment, barriers / TMEM slot / flags / sink
 // Epilogue classes of the grouped GEMM's kernel instances: bf16 outputs (GELU, SwiGLU,
 // plain), fp32 stores (plain, two-group sums), staged fp32 reductions (weight-gradient
@@ -213,15 +211,14 @@ enum { ECLS_BF16 = 0, ECLS_F32 = 1, ECLS_ADD = 2, ECLS_ADDT = 3, ECLS_DGELU = 4,
 constexpr int GM_ADDT_PARTS = 4;
 static_assert(4 * GM_ADDT_PARTS == GM_EPI_WARPS + GM_GATHER_WARPS, "the gather warps join the epilogue");
 // Shared memory beside the operand ring: the bf16 outputs pass 32 columns (training path: 16
-// of up to three arrays) of 32 rows per warp, the fp32 stores 32 columns of 32 rows, ECLS_ADD
-// stages 16 rows per warp, ECLS_ADDT keeps the {token, scale} pairs of 32 rows per warp: six
+// of up to three arrays) of 32 rows per warp, the other fp32 outputs 32 columns of 32 rows,
+// ECLS_ADDT keeps the {token, scale} pairs of 32 rows per warp: six
 // stages fit beside them.  The activation derivatives buffer two 16-column steps of u, a (and
 // v) per warp: five.
 __host__ __device__ constexpr int gm_bf16_warp_bytes(bool train) { return train ? 3 * 32 * 32 : 32 * 64; }
 __host__ __device__ constexpr int gm_stg_bytes(int ecls, bool train) {
     return ecls == ECLS_BF16 ? GM_EPI_WARPS * gm_bf16_warp_bytes(train)
-           : ecls == ECLS_F32 ? GM_EPI_WARPS * 32 * 128
-           : ecls == ECLS_ADD ? GM_EPI_WARPS * GM_STG_ROWS * GM_STG_LD * 4
+           : ecls == ECLS_F32 || ecls == ECLS_ADD ? GM_EPI_WARPS * 32 * 128
            : ecls == ECLS_ADDT ? 4 * GM_ADDT_PARTS * 32 * 8
            : ecls == ECLS_DGELU ? GM_EPI_WARPS * 2 * 2 * 1024
            : ecls == ECLS_DSWIGLU ? GM_EPI_WARPS * 2 * 3 * 1024 : 0;
