@@ -79,7 +79,7 @@ moevie_status moevie_workspace_init(void* ws, size_t ws_bytes, void* stream);
 
 /* Router (Eqs. 1, 7, 4-5).  x bf16 [T, d], W_r fp32 [d, E], b fp32 [E].
  * Out: idx int32 [T, k] (ascending ids per token), gate fp32 [T, k] (same order).
- * Logits are fp32 (tensor cores); a token whose selection the fp32 logits cannot
+ * Logits are fp32 (tensor cores; small problems: fp32 FMA); a token whose selection the fp32 logits cannot
  * certify (its k-th and (k+1)-th keys closer than their error bounds) is re-decided
  * from exact logits of the experts near its boundary -- an integer long accumulator
  * of the bf16 x fp32 products, within d 2^-64 sum|x_i w_i| of the exact dot product --

@@ -134,8 +134,8 @@ Layout make_layout(int64_t T, int64_t d, int64_t E, int64_t k, int64_t h, int64_
     L.items = take(16 * max_mtiles(n, E) * n_nt);   // band-ordered down-projection items
     L.n_items = take(4);
     L.n_tiles = take(4);
-    L.perm = take(4 * n);
-    L.inv = take(4 * n);
+    L.perm = take(4 * n);   // (room of earlier layouts: the forward writes perm and inv only to the
+    L.inv = take(4 * n);    //  caller's arrays; the size that callers ask for stays what it was)
     L.row_tok = take(4 * n2);
     L.row_gate = take(4 * n2);
     L.H = take(2 * n2 * row_ld(h));

@@ -351,7 +351,10 @@ __global__ void __launch_bounds__(1024) tile_table_kernel(const int32_t* __restr
     if (g == 0) *n_tiles = s_total;
 }
 
-// One CTA of 1024 threads.  Orders the (m-tile, n-tile) work items of a grouped GEMM
+constexpr int ITEM_CTAS = 8;
+// ITEM_CTAS CTAs of 1024 threads; each ranks every m-tile itself and writes its share of the
+// items (one CTA alone spent most of its time on the 16-byte scattered writes: 19 us for 15 k
+// items, 13 this way).  Orders the (m-tile, n-tile) work items of a grouped GEMM
 // in nb token bands x column groups of gsz n-tiles: band b holds the m-tiles whose
 // middle row's token lies in [b T / nb, (b + 1) T / nb) (expert-major order kept
 // inside a band).  Items run band-major, then column group, then m-tile, then n-tile,
@@ -414,10 +417,10 @@ __global__ void __launch_bounds__(1024) item_order_kernel(
             run += c;
         }
         s_cnt[nb] = run;
-        *n_items = run * n_ntiles;
+        if (blockIdx.x == 0) *n_items = run * n_ntiles;
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < nt; i += blockDim.x) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nt; i += gridDim.x * blockDim.x) {
         const int4 t = tiles[i];
         const int b = band[i];
         const int cnt_b = s_cnt[b + 1] - s_cnt[b];
@@ -578,7 +581,7 @@ cudaError_t launch_item_order(const int4* tiles, const int32_t* n_tiles, const i
         if (err != cudaSuccess) return err;
         attr_set[dev].store(true, std::memory_order_release);
     }
-    const cudaError_t err = launch_pdl(item_order_kernel, dim3(1), dim3(1024), smem, s, tiles, n_tiles,
+    const cudaError_t err = launch_pdl(item_order_kernel, dim3(ITEM_CTAS), dim3(1024), smem, s, tiles, n_tiles,
                                        row_tok, T, nb, n_ntiles, gsz, BN, max_tiles, items, n_items);
     count_launches(1);
     return err;

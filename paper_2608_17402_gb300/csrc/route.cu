@@ -31,6 +31,9 @@
 //     times a power of two; the CTA sums them in 128-bit fixed-point accumulators on
 //     the integer pipes, see long_acc_term), and the remaining places are filled from
 //     their keys (fp64), ties to the lower id.
+//
+// Small problems take one launch instead (route_small_kernel, launch_route_small): fp32 logits
+// on the FMA pipes, the same certified selection and the same exact re-decision.
 #include <math.h>
 
 #include "internal.h"
