@@ -238,6 +238,12 @@ __device__ __forceinline__ void st_global_v4_hint(void* p, const uint4& v, uint6
                  "r"(v.y), "r"(v.z), "r"(v.w), "l"(pol)
                  : "memory");
 }
+// *p += v (16 bytes, relaxed) with an L2 cache policy.  p: 16-byte aligned global memory.
+__device__ __forceinline__ void red_add_v4_hint(float4* p, const float4& v, uint64_t pol) {
+    asm volatile("red.relaxed.gpu.global.add.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p),
+                 "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "l"(pol)
+                 : "memory");
+}
 // *p += v as a relaxed reduction when sel >= 0 (predicated, no branch).  No memory clobber:
 // loads may move across it (nothing in the kernels that use it reads what it adds to).
 __device__ __forceinline__ void red_add_f32_if(float* p, float v, int sel) {

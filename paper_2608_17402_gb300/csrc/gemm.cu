@@ -25,17 +25,19 @@
 // arithmetic.
 //
 // Warp roles (608 threads per CTA, one CTA per SM):
-//   warps 0-7   epilogue: tcgen05.ld of the CTA's 128 accumulator rows (warp w:
-//               TMEM lanes 32 (w%4)..+31, every other 32-column chunk), fused math,
-//               and 16-byte stores / reductions of each thread's own row
-//   warp 8      TMEM allocation (both CTAs, jointly); leader lane 0 issues the MMAs
+//   warps 0-7   epilogue: tcgen05.ld of the CTA's 128 accumulator rows (warp w: TMEM lanes
+//               32 (w%4)..+31, every other 32-column chunk), fused math, and stores or
+//               reductions of whole sectors through a buffer per warp.  (The transposed
+//               product, epilogue_addt: with warps 10-17, straight from registers.)
+//   warp 8      TMEM allocation (both CTAs, jointly); the leader's issues the MMAs (the
+//               issuing roles run as whole warps, one elected lane issues)
 //   warp 9      TMA loads of the B half and, for contiguous A rows, of A; the leader
 //               posts the byte count of both CTAs on its full barrier.  With contiguous A
 //               warp 18 takes turns with it, stage by stage
 //   warps 10-17 token gather: 16-byte cp.async of A rows straight into the 128-byte
 //               swizzled K-major layout; each thread hands the completion of its
 //               copies to the stage's local afull barrier and moves on
-//   warp 18     lane 0: waits for afull, fences the stage to the async proxy and
+//   warp 18     waits for afull, fences the stage to the async proxy and
 //               publishes it on the leader's full barrier (from the peer: a 16-byte
 //               bulk copy that completes transaction bytes there)
 // Shared memory: 6 stages and an epilogue buffer (5 for the activation-derivative
@@ -787,7 +789,7 @@ __device__ void epilogue_addt(const GemmArgs& p, const Smem& sm, uint32_t tmem, 
 // rows at a time through rows of 36 floats (half the lanes idle, bank conflicts) the band-ordered
 // down-projection took 397 us at T = 32768, E = 128, this way 373.
 __device__ __forceinline__ void out_chunk(const GemmArgs& p, uint8_t* buf, int lane, const float (&f)[32], float sc,
-                                          int tok, int64_t base, int col0, int ncols, bool add) {
+                                          int tok, int64_t base, int col0, int ncols, bool add, bool banded, uint64_t keep) {
 #pragma unroll
     for (int q = 0; q < 8; ++q)
         *reinterpret_cast<float4*>(buf + lane * 128 + 16 * (q ^ (lane & 7))) =
@@ -802,7 +804,8 @@ __device__ __forceinline__ void out_chunk(const GemmArgs& p, uint8_t* buf, int l
         const float4 v = *reinterpret_cast<const float4*>(buf + r * 128 + 16 * (q ^ (r & 7)));
         if (tk >= 0 && col_ok) {
             float4* dst = reinterpret_cast<float4*>(p.yacc + base + (int64_t)tk * p.ldy + col0 + 4 * q);
-            if (add) atomicAdd(dst, v);
+            if (add && banded) red_add_v4_hint(dst, v, keep);
+            else if (add) atomicAdd(dst, v);
             else *dst = v;
         }
     }
@@ -820,6 +823,13 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
     const int nchunk = p.BN / 32;
     uint8_t* buf = reinterpret_cast<uint8_t*>(sm.stg) + warp * 4096;   // 32 rows x 128 bytes
     const uint32_t tempty_leader = peer_addr(sm.tempty, 0);
+    // Band-ordered reductions keep the accumulator's lines in L2 (evict-last) beside the streamed
+    // weights and rows: down-projection at T = 65536, d = 1664, E = 256 with loads after Zipf's
+    // law 1048 -> 926 us, the conversion that reads the accumulator next 96 -> 90; at T = 32768,
+    // d = 1536, E = 128 369-380 -> 365-387 (no difference beyond the runs'), conversion 43 -> 39.
+    // (Operand rows evict-first instead: 903 -> 1113 on a skewed T = 65536 layer.)
+    const bool banded = ECLS == ECLS_ADD && p.item_table == 1;
+    const uint64_t keep = banded ? l2_policy_evict_last() : 0;
     int it = 0;
     if (sm.pair >= n_work) return;
     TileLd nl = tile_load(p, sm.pair);   // one item ahead
@@ -873,7 +883,7 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
                 }
 #pragma unroll
                 for (int i = 0; i < 32; ++i) s2[i] += __uint_as_float(v[i]);
-                out_chunk(p, buf, lane, s2, sc, ok_row ? (int)tok : -1, t.ks * p.y_split_stride, ch * 32, p.N / 2, false);
+                out_chunk(p, buf, lane, s2, sc, ok_row ? (int)tok : -1, t.ks * p.y_split_stride, ch * 32, p.N / 2, false, false, 0);
             }
             continue;
         }
@@ -897,7 +907,7 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
             for (int i = 0; i < 32; ++i) f[i] = __uint_as_float(v[i]);
             // weight-gradient items that are their tile's only one store instead of adding
             out_chunk(p, buf, lane, f, sc, ok_row ? (int)tok : -1, t.ks * p.y_split_stride, t.n0 + c0, p.N,
-                      ECLS == ECLS_ADD && !(TRAIN && t.store));
+                      ECLS == ECLS_ADD && !(TRAIN && t.store), banded, keep);
         }
     }
 }
