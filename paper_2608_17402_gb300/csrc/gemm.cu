@@ -825,7 +825,7 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
     const uint32_t tempty_leader = peer_addr(sm.tempty, 0);
     // Band-ordered reductions keep the accumulator's lines in L2 (evict-last) beside the streamed
     // weights and rows: down-projection at T = 65536, d = 1664, E = 256 with loads after Zipf's
-    // law 1048 -> 926 us, the conversion that reads the accumulator next 96 -> 90; at T = 32768,
+    // law 1048 -> 926-950 us, the conversion that reads the accumulator next 96 -> 90; at T = 32768,
     // d = 1536, E = 128 369-380 -> 365-387 (no difference beyond the runs'), conversion 43 -> 39.
     // (Operand rows evict-first instead: 903 -> 1113 on a skewed T = 65536 layer.)
     const bool banded = ECLS == ECLS_ADD && p.item_table == 1;
