@@ -196,18 +196,37 @@ __device__ __forceinline__ void warp_kth_values(const float (&v)[NPL], int E, in
 __device__ __forceinline__ int bf16_exp_field(uint32_t hx) { return (int)((hx >> 7) & 0xffu); }
 __device__ __forceinline__ int f32_exp_field(uint32_t uw) { return (int)((uw >> 23) & 0xffu); }
 
+// x as its signed mantissa and its exponent (1 at least), w the same way.
+__device__ __forceinline__ void long_acc_x(uint32_t hx, int& mx, int& ex) {
+    const int e = bf16_exp_field(hx), m = (int)((hx & 0x7fu) | (e ? 0x80u : 0u));
+    mx = hx & 0x8000u ? -m : m;
+    ex = max(e, 1);
+}
+__device__ __forceinline__ void long_acc_w(uint32_t uw, int& mw, int& ew) {
+    const int e = f32_exp_field(uw), m = (int)((uw & 0x7fffffu) | (e ? 0x800000u : 0u));
+    mw = (int)uw < 0 ? -m : m;
+    ew = max(e, 1);
+}
+// acc += mx mw 2^sh (sh <= 64; below 0 the magnitude's dropped bits are less than one unit).  The
+// product (33 bits with its sign) and its two shifts are 64-bit; PTX clamps a shift by 64 or more.
+__device__ __forceinline__ void long_acc_add(int mx, int mw, int sh, unsigned __int128& acc) {
+    int64_t p = (int64_t)mx * mw;
+    if (sh < 0) {   // rare: a term 2^64 times smaller than the largest it might have been
+        const int64_t m = (p < 0 ? -p : p) >> min(-sh, 63);
+        p = p < 0 ? -m : m;
+        sh = 0;
+    }
+    uint64_t lo, hi;
+    asm("shl.b64 %0, %1, %2;" : "=l"(lo) : "l"(p), "r"(sh));
+    asm("shr.s64 %0, %1, %2;" : "=l"(hi) : "l"(p), "r"(64 - sh));
+    acc += ((unsigned __int128)hi << 64) | lo;
+}
 // acc += x w in units of 2^(Q - 348) (hx: bf16 bits of x, uw: fp32 bits of w).
 __device__ __forceinline__ void long_acc_term(uint32_t hx, uint32_t uw, int Q, unsigned __int128& acc) {
-    const int ex = bf16_exp_field(hx), ew = f32_exp_field(uw);
-    const uint64_t mx = (hx & 0x7fu) | (ex ? 0x80u : 0u);
-    const uint64_t mw = (uw & 0x7fffffu) | (ew ? 0x800000u : 0u);
-    const uint64_t P = mx * mw;
-    const int sh = 64 - (Q - (max(ex, 1) + max(ew, 1)));   // <= 64
-    unsigned __int128 t;
-    if (sh >= 0) t = (unsigned __int128)P << sh;
-    else t = sh > -64 ? (unsigned __int128)(P >> -sh) : (unsigned __int128)0;
-    if ((hx ^ (uw >> 16)) & 0x8000u) acc -= t;
-    else acc += t;
+    int mx, ex, mw, ew;
+    long_acc_x(hx, mx, ex);
+    long_acc_w(uw, mw, ew);
+    long_acc_add(mx, mw, 64 - Q + ex + ew, acc);
 }
 
 __device__ __forceinline__ unsigned __int128 warp_sum_u128(unsigned __int128 v) {
@@ -378,7 +397,72 @@ __global__ void __launch_bounds__(256) route_topk_kernel(
 }
 
 
-// Exact re-decision of one uncertified token by a CTA of 8 warps.  The CTA stages
+// The two warp steps of an exact re-decision.  First, from the fast logits sv and their error
+// bounds ts (slots past E get anything): the experts that are surely in, and the candidates for
+// the remaining places.
+template <int NPL>
+__device__ __forceinline__ void bound_candidates(const float (&sv)[NPL], const float (&ts)[NPL],
+                                                 const float* __restrict__ b, int E, int k, int lane,
+                                                 uint32_t& sure_in, uint32_t& cand) {
+    float up[NPL], lo[NPL];
+#pragma unroll
+    for (int i = 0; i < NPL; ++i) {
+        const int e = lane + 32 * i;
+        if (e < E) {
+            const float key = sigmoid_fast(sv[i]) + b[e];
+            const float tk = key_tau_exact_slope(sv[i], ts[i]);
+            up[i] = key + tk;
+            lo[i] = key - tk;
+        } else {
+            up[i] = lo[i] = -INFINITY;
+        }
+    }
+    // k-th / (k+1)-th largest upper ends and k-th largest lower end
+    float u_k, u_k1, l_k, l_k1;
+    warp_kth_values<NPL>(up, E, k, lane, u_k, u_k1);
+    warp_kth_values<NPL>(lo, E, k, lane, l_k, l_k1);
+    sure_in = cand = 0;
+#pragma unroll
+    for (int i = 0; i < NPL; ++i) {
+        const int e = lane + 32 * i;
+        if (e >= E) continue;
+        // k-th largest upper end among the others (u_k when e may sit at rank k: conservative)
+        const float thr = up[i] > u_k ? u_k1 : u_k;
+        if (k >= E || lo[i] > thr) sure_in |= 1u << i;
+        else if (!(up[i] < l_k)) cand |= 1u << i;
+    }
+}
+// Then, with the candidates' exact keys: `need` of them by key, ties to the lower id.
+template <int NPL>
+__device__ __forceinline__ uint32_t choose_exact(const double (&exk)[NPL], uint32_t sure_in, uint32_t cand, int need,
+                                                 int lane) {
+    uint32_t chosen = sure_in;
+    for (int r = 0; r < need; ++r) {
+        double bv = -INFINITY;
+        int bi = 0x7fffffff;
+#pragma unroll
+        for (int i = 0; i < NPL; ++i) {
+            const int e = lane + 32 * i;
+            if (((cand >> i) & 1u) && !((chosen >> i) & 1u) && (exk[i] > bv || bi == 0x7fffffff)) {
+                bv = exk[i];
+                bi = e;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            if (ov > bv || (ov == bv && oi < bi)) {
+                bv = ov;
+                bi = oi;
+            }
+        }
+        if ((bi & 31) == lane) chosen |= 1u << (bi >> 5);
+    }
+    return chosen;
+}
+
+// Exact re-decision of the uncertified tokens, a CTA of 8 warps per token.  The CTA stages
 // the token's x row in shared memory (16-byte loads) and finds its largest exponent
 // field; warp 0 bounds the keys and lists the candidates; then the candidates' exact
 // logits are formed FB_BATCH at a time by all 256 threads (threads over the d terms,
@@ -397,183 +481,14 @@ constexpr int FB_X_SMEM = 16384;  // largest d whose x row is staged in shared m
 // CTAs per SM the re-decision keeps resident for E <= 256 (its registers allow five), so
 // that up to five tokens per SM are re-decided at once
 constexpr int FB_CTAS_PER_SM = 5;
-template <int NPL>
-struct FbShared {
-    int cand[32 * NPL];
-    double key[32 * NPL];
-    unsigned long long acc[8][FB_BATCH][2];
-    int q[FB_BATCH];
-    int ncand;
-    int qx;
-};
 
-// Token t: xg its x row, fb_x its staging buffer (staged), logits(sv, ts) this lane's fast
-// logits and their error bounds (called by warp 0; slots past E get anything), window(e) the
-// largest exponent field of W_r[:, e] (called by a warp), weight(e, i) = W_r[i, e].  The caller
-// synchronises the CTA before sh and fb_x are used again.
-template <int NPL, class Logits, class Window, class Weight>
-__device__ __forceinline__ void redecide_token(FbShared<NPL>& sh, const uint16_t* __restrict__ xg, uint16_t* fb_x,
-                                               bool staged, const float* __restrict__ b, int64_t t, int d, int E,
-                                               int k, int32_t* __restrict__ idx, float* __restrict__ gate,
-                                               DevStatus* st, Logits logits, Window window, Weight weight) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t lt = (1u << lane) - 1u;
-    if (threadIdx.x == 0) sh.qx = 1;
-    __syncthreads();
-    if (warp > 0 || !staged) {   // warps 1-7 stage x_t while warp 0 bounds the keys
-        int m = 1;
-        const int nthr = staged ? (int)blockDim.x - 32 : (int)blockDim.x;
-        const int tid = staged ? (int)threadIdx.x - 32 : (int)threadIdx.x;
-        for (int i = tid; i < d / 8; i += nthr) {   // d % 8 == 0, rows 16-byte aligned
-            const uint4 v = reinterpret_cast<const uint4*>(xg)[i];
-            if (staged) reinterpret_cast<uint4*>(fb_x)[i] = v;
-            const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+// Largest exponent field of the eight bf16 values in v.
+__device__ __forceinline__ int bf16x8_exp_max(const uint4& v) {
+    const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+    int m = 0;
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                m = max(m, max((int)((w4[j] >> 7) & 0xffu), (int)((w4[j] >> 23) & 0xffu)));
-        }
-        m = __reduce_max_sync(0xffffffffu, m);
-        if (lane == 0) atomicMax(&sh.qx, m);
-    }
-    float sv[NPL], ts[NPL];
-    uint32_t sure_in = 0, cand = 0;
-    int need = 0;
-    if (warp == 0) {
-        float up[NPL], lo[NPL];
-        logits(sv, ts);
-#pragma unroll
-        for (int i = 0; i < NPL; ++i) {
-            const int e = lane + 32 * i;
-            if (e < E) {
-                const float key = sigmoid_fast(sv[i]) + b[e];
-                const float tk = key_tau_exact_slope(sv[i], ts[i]);
-                up[i] = key + tk;
-                lo[i] = key - tk;
-            } else {
-                up[i] = lo[i] = -INFINITY;
-            }
-        }
-        // k-th / (k+1)-th largest upper ends and k-th largest lower end
-        float u_k, u_k1, l_k, l_k1;
-        warp_kth_values<NPL>(up, E, k, lane, u_k, u_k1);
-        warp_kth_values<NPL>(lo, E, k, lane, l_k, l_k1);
-#pragma unroll
-        for (int i = 0; i < NPL; ++i) {
-            const int e = lane + 32 * i;
-            if (e >= E) continue;
-            // k-th largest upper end among the others (u_k when e may sit at rank k: conservative)
-            const float thr = up[i] > u_k ? u_k1 : u_k;
-            if (k >= E || lo[i] > thr) sure_in |= 1u << i;
-            else if (!(up[i] < l_k)) cand |= 1u << i;
-        }
-        int n_in = 0, n_cand = 0;
-#pragma unroll
-        for (int i = 0; i < NPL; ++i) {
-            n_in += __popc(__ballot_sync(0xffffffffu, (sure_in >> i) & 1u));
-            const uint32_t m = __ballot_sync(0xffffffffu, (cand >> i) & 1u);
-            if ((cand >> i) & 1u) sh.cand[n_cand + __popc(m & lt)] = lane + 32 * i;
-            n_cand += __popc(m);
-        }
-        need = k - n_in;
-        const bool bad = need < 0 || need > n_cand;
-        if (lane == 0) {
-            if (bad) report(st, MOEVIE_ERR_DEVICE, SITE_ROUTE_FALLBACK, t, need);
-            sh.ncand = bad ? -1 : (need == 0 ? 0 : n_cand);
-        }
-    }
-    __syncthreads();
-    const int nc = sh.ncand;
-    const int qx = sh.qx;
-    const uint16_t* xs = staged ? fb_x : xg;
-    for (int c0 = 0; c0 < nc; c0 += FB_BATCH) {
-        const int cn = min(FB_BATCH, nc - c0);
-        if (warp < cn) {   // warp c: the window of candidate c0 + c
-            const int e = sh.cand[c0 + warp];
-            const int qw = window(e);
-            if (lane == 0) sh.q[warp] = (qx == 255 || qw == 255) ? -1 : qx + qw;   // -1: NaN
-        }
-        __syncthreads();
-        unsigned __int128 acc[FB_BATCH];
-        int Q[FB_BATCH];
-        int ec[FB_BATCH];
-#pragma unroll
-        for (int c = 0; c < FB_BATCH; ++c) {
-            acc[c] = 0;
-            Q[c] = c < cn ? sh.q[c] : -1;
-            ec[c] = sh.cand[c0 + (c < cn ? c : 0)];
-        }
-        for (int i = threadIdx.x; i < d; i += blockDim.x) {
-            const uint32_t hx = xs[i];
-            uint32_t uw[FB_BATCH];
-#pragma unroll
-            for (int c = 0; c < FB_BATCH; ++c) uw[c] = Q[c] > 0 ? __float_as_uint(weight(ec[c], i)) : 0u;
-#pragma unroll
-            for (int c = 0; c < FB_BATCH; ++c)
-                if (Q[c] > 0) long_acc_term(hx, uw[c], Q[c], acc[c]);
-        }
-#pragma unroll
-        for (int c = 0; c < FB_BATCH; ++c) {
-            if (Q[c] <= 0) continue;   // uniform over the CTA
-            const unsigned __int128 a = warp_sum_u128(acc[c]);
-            if (lane == 0) {
-                sh.acc[warp][c][0] = (unsigned long long)(uint64_t)a;
-                sh.acc[warp][c][1] = (unsigned long long)(uint64_t)(a >> 64);
-            }
-        }
-        __syncthreads();
-        if (warp == 0 && lane < cn) {   // candidate c0 + lane: the sum over the 8 warps
-            const int q = sh.q[lane];
-            double v = __longlong_as_double(0x7ff8000000000000ll);
-            if (q > 0) {
-                unsigned __int128 u = 0;
-#pragma unroll
-                for (int w = 0; w < 8; ++w)
-                    u += ((unsigned __int128)sh.acc[w][lane][1] << 64) | sh.acc[w][lane][0];
-                v = long_acc_value(u, q);
-            }
-            sh.key[c0 + lane] = 1.0 / (1.0 + exp(-v)) + (double)b[sh.cand[c0 + lane]];
-        }
-        __syncthreads();
-    }
-    if (warp == 0 && nc >= 0) {
-        double exk[NPL];
-        int base = 0;
-#pragma unroll
-        for (int i = 0; i < NPL; ++i) {
-            const uint32_t m = __ballot_sync(0xffffffffu, (cand >> i) & 1u);
-            exk[i] = ((cand >> i) & 1u && nc > 0) ? sh.key[base + __popc(m & lt)] : -INFINITY;
-            base += __popc(m);
-        }
-        // choose `need` candidates by exact key, ties to the lower id
-        uint32_t chosen = sure_in;
-        for (int r = 0; r < need; ++r) {
-            double bv = -INFINITY;
-            int bi = 0x7fffffff;
-#pragma unroll
-            for (int i = 0; i < NPL; ++i) {
-                const int e = lane + 32 * i;
-                if (((cand >> i) & 1u) && !((chosen >> i) & 1u) &&
-                    (exk[i] > bv || bi == 0x7fffffff)) {
-                    bv = exk[i];
-                    bi = e;
-                }
-            }
-#pragma unroll
-            for (int o = 16; o; o >>= 1) {
-                const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (ov > bv || (ov == bv && oi < bi)) {
-                    bv = ov;
-                    bi = oi;
-                }
-            }
-            if ((bi & 31) == lane) chosen |= 1u << (bi >> 5);
-        }
-        float sg[NPL];
-#pragma unroll
-        for (int i = 0; i < NPL; ++i) sg[i] = ((chosen >> i) & 1u) ? sigmoid_fast(sv[i]) : 0.f;
-        write_selection<NPL>(chosen, sg, t, k, lane, idx, gate);
-    }
+    for (int j = 0; j < 4; ++j) m = max(m, max((int)((w4[j] >> 7) & 0xffu), (int)((w4[j] >> 23) & 0xffu)));
+    return m;
 }
 
 template <int NPL>
@@ -586,30 +501,132 @@ __global__ void __launch_bounds__(256, (NPL <= 8 ? FB_CTAS_PER_SM : 1)) route_fa
     DevStatus* st) {
     pdl_wait();
     extern __shared__ __align__(16) uint16_t fb_x[];   // the token's x row when d <= FB_X_SMEM
-    __shared__ FbShared<NPL> sh;
-    const int lane = threadIdx.x & 31;
+    __shared__ int s_cand[32 * NPL];
+    __shared__ double s_key[32 * NPL];
+    __shared__ unsigned long long s_acc[8][FB_BATCH][2];
+    __shared__ int s_q[FB_BATCH];
+    __shared__ int s_ncand, s_qx;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
     const int nfb = st->fb_count;
     const bool staged = d <= FB_X_SMEM;
     for (int f = blockIdx.x; f < nfb; f += gridDim.x) {
         const int t = fb_tokens[f];
-        redecide_token<NPL>(
-            sh, reinterpret_cast<const uint16_t*>(x) + (int64_t)t * d, fb_x, staged, b, t, d, E, k, idx, gate, st,
-            [&](float (&sv)[NPL], float (&ts)[NPL]) {
-                const float xn = xnorm[t];
+        const uint16_t* xg = reinterpret_cast<const uint16_t*>(x) + (int64_t)t * d;
+        if (threadIdx.x == 0) s_qx = 1;
+        __syncthreads();
+        if (warp > 0 || !staged) {   // warps 1-7 stage x_t while warp 0 bounds the keys
+            int m = 1;
+            const int nthr = staged ? (int)blockDim.x - 32 : (int)blockDim.x;
+            const int tid = staged ? (int)threadIdx.x - 32 : (int)threadIdx.x;
+            for (int i = tid; i < d / 8; i += nthr) {   // d % 8 == 0, rows 16-byte aligned
+                const uint4 v = reinterpret_cast<const uint4*>(xg)[i];
+                if (staged) reinterpret_cast<uint4*>(fb_x)[i] = v;
+                m = max(m, bf16x8_exp_max(v));
+            }
+            m = __reduce_max_sync(0xffffffffu, m);
+            if (lane == 0) atomicMax(&s_qx, m);
+        }
+        float sv[NPL];
+        uint32_t sure_in = 0, cand = 0;
+        int need = 0;
+        if (warp == 0) {
+            float ts[NPL];
+            const float xn = xnorm[t];
 #pragma unroll
-                for (int i = 0; i < NPL; ++i) {
-                    const int e = lane + 32 * i;
-                    sv[i] = e < E ? s[(int64_t)t * ld + e] : 0.f;
-                    ts[i] = e < E ? logit_tau(xn, wnorm[e], wnorm[E + e]) : 0.f;
-                }
-            },
-            [&](int e) {
+            for (int i = 0; i < NPL; ++i) {
+                const int e = lane + 32 * i;
+                sv[i] = e < E ? s[(int64_t)t * ld + e] : 0.f;
+                ts[i] = e < E ? logit_tau(xn, wnorm[e], wnorm[E + e]) : 0.f;
+            }
+            bound_candidates<NPL>(sv, ts, b, E, k, lane, sure_in, cand);
+            int n_in = 0, n_cand = 0;
+#pragma unroll
+            for (int i = 0; i < NPL; ++i) {
+                n_in += __popc(__ballot_sync(0xffffffffu, (sure_in >> i) & 1u));
+                const uint32_t m = __ballot_sync(0xffffffffu, (cand >> i) & 1u);
+                if ((cand >> i) & 1u) s_cand[n_cand + __popc(m & lt)] = lane + 32 * i;
+                n_cand += __popc(m);
+            }
+            need = k - n_in;
+            const bool bad = need < 0 || need > n_cand;
+            if (lane == 0) {
+                if (bad) report(st, MOEVIE_ERR_DEVICE, SITE_ROUTE_FALLBACK, t, need);
+                s_ncand = bad ? -1 : (need == 0 ? 0 : n_cand);
+            }
+        }
+        __syncthreads();
+        const int nc = s_ncand;
+        const int qx = s_qx;
+        const uint16_t* xs = staged ? fb_x : xg;
+        for (int c0 = 0; c0 < nc; c0 += FB_BATCH) {
+            const int cn = min(FB_BATCH, nc - c0);
+            if (warp < cn) {   // warp c: the window of candidate c0 + c
+                const int e = s_cand[c0 + warp];
                 int qw = 1;
                 for (int pp = lane; pp < wexp_parts; pp += 32) qw = max(qw, __ldg(wexp + (int64_t)pp * Ep + e));
-                return (int)__reduce_max_sync(0xffffffffu, qw);
-            },
-            [&](int e, int i) { return __ldg(wrt + (int64_t)e * dp + i); });
-        __syncthreads();   // sh / fb_x are reused by the next token
+                qw = __reduce_max_sync(0xffffffffu, qw);
+                if (lane == 0) s_q[warp] = (qx == 255 || qw == 255) ? -1 : qx + qw;   // -1: NaN
+            }
+            __syncthreads();
+            unsigned __int128 acc[FB_BATCH];
+            int Q[FB_BATCH];
+            int ec[FB_BATCH];
+#pragma unroll
+            for (int c = 0; c < FB_BATCH; ++c) {
+                acc[c] = 0;
+                Q[c] = c < cn ? s_q[c] : -1;
+                ec[c] = s_cand[c0 + (c < cn ? c : 0)];
+            }
+            for (int i = threadIdx.x; i < d; i += blockDim.x) {
+                const uint32_t hx = xs[i];
+                uint32_t uw[FB_BATCH];
+#pragma unroll
+                for (int c = 0; c < FB_BATCH; ++c) uw[c] = Q[c] > 0 ? __float_as_uint(__ldg(wrt + (int64_t)ec[c] * dp + i)) : 0u;
+#pragma unroll
+                for (int c = 0; c < FB_BATCH; ++c)
+                    if (Q[c] > 0) long_acc_term(hx, uw[c], Q[c], acc[c]);
+            }
+#pragma unroll
+            for (int c = 0; c < FB_BATCH; ++c) {
+                if (Q[c] <= 0) continue;   // uniform over the CTA
+                const unsigned __int128 a = warp_sum_u128(acc[c]);
+                if (lane == 0) {
+                    s_acc[warp][c][0] = (unsigned long long)(uint64_t)a;
+                    s_acc[warp][c][1] = (unsigned long long)(uint64_t)(a >> 64);
+                }
+            }
+            __syncthreads();
+            if (warp == 0 && lane < cn) {   // candidate c0 + lane: the sum over the 8 warps
+                const int q = s_q[lane];
+                double v = __longlong_as_double(0x7ff8000000000000ll);
+                if (q > 0) {
+                    unsigned __int128 u = 0;
+#pragma unroll
+                    for (int ww = 0; ww < 8; ++ww)
+                        u += ((unsigned __int128)s_acc[ww][lane][1] << 64) | s_acc[ww][lane][0];
+                    v = long_acc_value(u, q);
+                }
+                s_key[c0 + lane] = 1.0 / (1.0 + exp(-v)) + (double)b[s_cand[c0 + lane]];
+            }
+            __syncthreads();
+        }
+        if (warp == 0 && nc >= 0) {
+            double exk[NPL];
+            int base = 0;
+#pragma unroll
+            for (int i = 0; i < NPL; ++i) {
+                const uint32_t m = __ballot_sync(0xffffffffu, (cand >> i) & 1u);
+                exk[i] = ((cand >> i) & 1u && nc > 0) ? s_key[base + __popc(m & lt)] : -INFINITY;
+                base += __popc(m);
+            }
+            const uint32_t chosen = choose_exact<NPL>(exk, sure_in, cand, need, lane);
+            float sg[NPL];
+#pragma unroll
+            for (int i = 0; i < NPL; ++i) sg[i] = ((chosen >> i) & 1u) ? sigmoid_fast(sv[i]) : 0.f;
+            write_selection<NPL>(chosen, sg, t, k, lane, idx, gate);
+        }
+        __syncthreads();   // the shared arrays are reused by the next token
     }
 }
 
@@ -617,7 +634,7 @@ __global__ void __launch_bounds__(256, (NPL <= 8 ? FB_CTAS_PER_SM : 1)) route_fa
 // FMA pipes straight from W_r, the certified top-k, and the exact re-decision.  The
 // tensor-core route (split of W_r, GEMM, top-k, re-decision) is four dependent launches, 17.5
 // us at T = 512, d = 768, E = 16 and 18.0 at T = 256, E = 31 (back to back calls); this kernel
-// takes 10.5 (the rate of the calls) and 12.8.  A CTA of 8 warps takes 8 tokens, each warp an
+// takes 10.5 (the rate of the calls) and 12.8.  A CTA of 8 warps takes up to 8 tokens, each warp an
 // eighth of d: chunks of CH rows of W_r and columns of x go through registers (one chunk
 // ahead) into the warp's shared memory as fp32, and each lane forms one token x 8 NE experts
 // with packed FMAs (lane = 4 token + expert group).  What bounds it is the L2 latency of the
@@ -628,16 +645,202 @@ __global__ void __launch_bounds__(256, (NPL <= 8 ? FB_CTAS_PER_SM : 1)) route_fa
 // to first order (one more unit covers the rest): rigorous.  The loading lanes also form
 // |W_r[:, e]|, the columns' largest exponent fields and |x_t|.
 constexpr int RS_TB = 8, RS_NW = 8;   // tokens and warps per CTA
+constexpr int ROUTE_SMALL_ED = 32768;   // largest 32 ceil(E / 32) d (route_small)
+template <int NE>
+constexpr int RS_G = 4 / NE;            // tokens whose exact logits are formed together
+template <int NE>
+constexpr size_t route_small_sums = 16 * RS_NW * 32 * NE * RS_G<NE>;
 template <int NE>
 constexpr size_t route_small_smem() {
     constexpr size_t EP = 32 * NE, CH = 16 / NE;
-    return 4 * RS_NW * (CH * (RS_TB + EP) > RS_TB * EP ? CH * (RS_TB + EP) : RS_TB * EP);
+    constexpr size_t logits = 4 * RS_NW * (CH * (RS_TB + EP) > RS_TB * EP ? CH * (RS_TB + EP) : RS_TB * EP);
+    constexpr size_t exact = route_small_sums<NE> + 4 * RS_G<NE> * (ROUTE_SMALL_ED / EP);   // route_small_exact's sums and xp
+    return logits > exact ? logits : exact;
 }
+// Exact logits of the uncertified tokens of a CTA of route_small_kernel (RS_TB tokens from xg, RS_NW
+// warps): logit[tt][e] for the candidates cand[tt], from the same long accumulators as
+// route_fallback_kernel's and with the same windows (wmax: the columns' largest exponent fields).
+// A token with at most FB_BATCH candidates takes the threads over the d terms.  Tokens with more go
+// RS_G together, lanes over the experts: the weights are read as whole rows of W_r and taken
+// apart once for those tokens, the warps (with E <= 16 also the parts of a warp) share the
+// terms, and a pass costs the same however many of the experts tie.  The integer instructions bound
+// it (about 20 a term).  The whole router on tokens that tie in every key (W_r = 0, b = 0): 32 us at
+// T = 64, d = 1024, E = 32 and 98 us at T = 1216, d = 512, E = 64, against 57 and 186 of the
+// tensor-core route, and 330 and 470 with the threads over the terms for any number of candidates
+// and the eight tokens of a CTA one after another through all of their steps.  Not inlined: its
+// registers are not to crowd the kernel's main loop.
+// sums: the warps' sums, [2][RS_NW][EP] (two tokens in turn) or [RS_G][RS_NW][EP]; xp: the
+// tokens' x as (mantissa << 16 | exponent), [RS_G][d].
+template <int NE>
+__device__ __noinline__ void route_small_exact(const __nv_bfloat16* __restrict__ xg, const float* __restrict__ Wr,
+                                               int d, int E, const uint32_t (*cand)[NE], const int* qx,
+                                               const uint32_t* wmax, ulonglong2* sums, int* xp,
+                                               double (*logit)[32 * NE]) {
+    constexpr int EP = 32 * NE, NW = RS_NW, G = RS_G<NE>;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto window = [&](int tt, int e) { return qx[tt] == 255 || wmax[e] == 255u ? -1 : qx[tt] + (int)wmax[e]; };   // -1: NaN
+    auto put = [&](int at, const unsigned __int128& a) {
+        sums[at] = make_ulonglong2((unsigned long long)(uint64_t)a, (unsigned long long)(uint64_t)(a >> 64));
+    };
+    // the sum over the warps of token tt, expert e (part `from` of sums)
+    auto finish = [&](int tt, int e, int from) {
+        if (!((cand[tt][e / 32] >> (e & 31)) & 1u)) return;
+        const int Q = window(tt, e);
+        double v = __longlong_as_double(0x7ff8000000000000ll);
+        if (Q > 0) {
+            unsigned __int128 u = 0;
+#pragma unroll
+            for (int q = 0; q < NW; ++q) {
+                const ulonglong2 a = sums[(from * NW + q) * EP + e];
+                u += ((unsigned __int128)a.y << 64) | a.x;
+            }
+            v = long_acc_value(u, Q);
+        }
+        logit[tt][e] = v;
+    };
+    uint32_t wide = 0;   // tokens with more than FB_BATCH candidates (the same for the whole CTA, as all that branches on it)
+    int buf = 0;
+    for (int tt = 0; tt < RS_TB; ++tt) {
+        uint32_t cm[NE];
+        int n = 0;
+#pragma unroll
+        for (int i = 0; i < NE; ++i) {
+            cm[i] = cand[tt][i];
+            n += __popc(cm[i]);
+        }
+        if (n > FB_BATCH) wide |= 1u << tt;
+        if (n == 0 || n > FB_BATCH) continue;
+        const uint16_t* xr = reinterpret_cast<const uint16_t*>(xg) + (int64_t)tt * d;
+        unsigned __int128 acc[FB_BATCH];
+        int ec[FB_BATCH], Q[FB_BATCH];
+#pragma unroll
+        for (int c = 0; c < FB_BATCH; ++c) {   // candidate c: the lowest id left
+            acc[c] = 0;
+            ec[c] = -1;
+#pragma unroll
+            for (int i = 0; i < NE; ++i)
+                if (ec[c] < 0 && cm[i]) {
+                    ec[c] = 32 * i + __ffs(cm[i]) - 1;
+                    cm[i] &= cm[i] - 1u;
+                }
+            Q[c] = ec[c] >= 0 ? window(tt, ec[c]) : -1;
+        }
+        for (int i = threadIdx.x; i < d; i += 32 * NW) {
+            const uint32_t hx = xr[i];
+            uint32_t uw[FB_BATCH];
+#pragma unroll
+            for (int c = 0; c < FB_BATCH; ++c)
+                uw[c] = Q[c] > 0 ? __float_as_uint(__ldg(Wr + (int64_t)i * E + ec[c])) : 0u;
+#pragma unroll
+            for (int c = 0; c < FB_BATCH; ++c)
+                if (Q[c] > 0) long_acc_term(hx, uw[c], Q[c], acc[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < FB_BATCH; ++c) {
+            if (Q[c] <= 0) continue;
+            const unsigned __int128 a = warp_sum_u128(acc[c]);
+            if (lane == 0) put((buf * NW + warp) * EP + ec[c], a);
+        }
+        __syncthreads();
+        // (the token after the next writes this half again: after the next token's barrier)
+        if (threadIdx.x < EP) finish(tt, threadIdx.x, buf);
+        buf ^= 1;
+    }
+    const int W = NE > 1 || E > 16 ? 32 : E > 8 ? 16 : 8;   // lanes over the experts; 32 / W parts of a warp
+    const int sub = lane / W, le = lane % W, step = NW * (32 / W);
+    while (wide) {
+        int tok[G];   // -1: none left
+        unsigned __int128 acc[G][NE];
+        int base[G][NE];   // 64 - Q; 128: not a candidate, or its logit is NaN
+#pragma unroll
+        for (int u = 0; u < G; ++u) {
+            tok[u] = __ffs(wide) - 1;
+            wide &= wide - 1u;
+#pragma unroll
+            for (int i = 0; i < NE; ++i) {
+                acc[u][i] = 0;
+                base[u][i] = 128;
+                if (tok[u] >= 0 && ((cand[tok[u]][i] >> le) & 1u)) {
+                    const int Q = window(tok[u], le + 32 * i);
+                    if (Q > 0) base[u][i] = 64 - Q;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+            if (tok[u] >= 0)
+                for (int g = threadIdx.x; g < d / 8; g += 32 * NW) {
+                    const uint4 v = reinterpret_cast<const uint4*>(xg + (int64_t)tok[u] * d)[g];
+                    const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+                    int o[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        int mx, ex;
+                        long_acc_x(w4[j / 2] >> (16 * (j & 1)), mx, ex);
+                        o[j] = mx * 65536 + ex;
+                    }
+                    int4* to = reinterpret_cast<int4*>(xp + u * d + 8 * g);
+                    to[0] = make_int4(o[0], o[1], o[2], o[3]);
+                    to[1] = make_int4(o[4], o[5], o[6], o[7]);
+                }
+        // four terms a step, the next step's weights loaded ahead of them
+        uint32_t un[4][NE];
+        auto load = [&](int g) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int i = 0; i < NE; ++i)
+                    un[j][i] = g < d / 4 && le + 32 * i < E ? __float_as_uint(__ldg(Wr + (int64_t)(4 * g + j) * E + le + 32 * i)) : 0u;
+        };
+        load(warp * (32 / W) + sub);
+        __syncthreads();   // xp; and the sums of the tokens before have been taken
+        for (int g = warp * (32 / W) + sub; g < d / 4; g += step) {
+            int mw[4][NE], ew[4][NE];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int i = 0; i < NE; ++i) long_acc_w(un[j][i], mw[j][i], ew[j][i]);
+            load(g + step);
+#pragma unroll
+            for (int u = 0; u < G; ++u) {
+                if (tok[u] < 0) break;
+                const int4 x4 = *reinterpret_cast<const int4*>(xp + u * d + 4 * g);
+                const int xq[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                    for (int i = 0; i < NE; ++i)
+                        if (base[u][i] < 128)
+                            long_acc_add(xq[j] >> 16, mw[j][i], base[u][i] + (xq[j] & 0xffff) + ew[j][i], acc[u][i]);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < G; ++u)
+#pragma unroll
+            for (int i = 0; i < NE; ++i) {
+                for (int o = W; o < 32; o <<= 1) {
+                    const uint64_t lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)(uint64_t)acc[u][i], o);
+                    const uint64_t hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)(uint64_t)(acc[u][i] >> 64), o);
+                    acc[u][i] += ((unsigned __int128)hi << 64) | lo;
+                }
+                if (sub == 0 && base[u][i] < 128) put((u * NW + warp) * EP + le + 32 * i, acc[u][i]);
+            }
+        __syncthreads();
+        if (threadIdx.x < G * EP) {
+            const int u = threadIdx.x / EP;
+            int tt = -1;
+#pragma unroll
+            for (int v = 0; v < G; ++v) tt = u == v ? tok[v] : tt;
+            if (tt >= 0) finish(tt, threadIdx.x % EP, u);
+        }
+    }
+}
+
 // Units of 2^-24 |x_t| |W_r[:, e]| certified at least: twice the sum's own bound at d = 192.
 constexpr int ROUTE_SMALL_TAU_MIN = 64;
 template <int NE>
-__global__ void __launch_bounds__(256, 2) route_small_kernel(
-    const __nv_bfloat16* __restrict__ x, const float* __restrict__ Wr, const float* __restrict__ b, int T, int d,
+__global__ void __launch_bounds__(256, 1) route_small_kernel(
+    const __nv_bfloat16* __restrict__ x, const float* __restrict__ Wr, const float* __restrict__ b, int T, int tb, int d,
     int E, int k, int32_t* __restrict__ idx, float* __restrict__ gate, DevStatus* st, float4* __restrict__ zero,
     int64_t zero_n4) {
     pdl_wait();
@@ -657,10 +860,12 @@ __global__ void __launch_bounds__(256, 2) route_small_kernel(
     __shared__ float s_w2[NW][EP];      // partial sums of squares of W_r's columns, then |W_r[:, e]|
     __shared__ uint32_t s_wmax[NW][EP]; // largest |w| bits, then exponent fields
     __shared__ float s_x2[NW][TB];
-    __shared__ int s_list[TB], s_nlist;
-    __shared__ FbShared<NE> sh;
+    __shared__ uint32_t s_cand[TB][NE];    // uncertified tokens: candidates of each 32-expert slot
+    __shared__ int s_qx[TB], s_nlist;      //   largest exponent field of x_t; their number
+    __shared__ double s_logit[TB][EP];     //   the candidates' exact logits
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t t0 = (int64_t)blockIdx.x * TB;
+    const int64_t t0 = (int64_t)blockIdx.x * tb;
+    const int nt = min(tb, (int)(T - t0));   // tokens of this CTA
     if (threadIdx.x == 0) s_nlist = 0;
     float* xs = buf + warp * WBUF;
     float* ws = xs + CH * TB;
@@ -669,8 +874,8 @@ __global__ void __launch_bounds__(256, 2) route_small_kernel(
     const int xt = lane % TB, xk = 8 * (lane / TB);   // this lane's piece of x: its token, its first column
     uint4 xr;
     float wv[CH][NE];
-    auto load = [&](int k0) {   // chunk k0 .. k0 + CH - 1 into registers (zeros past kend, T and E)
-        const bool ok = lane < XPC && k0 + xk < kend && t0 + xt < T;
+    auto load = [&](int k0) {   // chunk k0 .. k0 + CH - 1 into registers (zeros past kend, nt and E)
+        const bool ok = lane < XPC && k0 + xk < kend && xt < nt;
         xr = ok ? *reinterpret_cast<const uint4*>(x + (t0 + xt) * d + k0 + xk) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
         for (int u = 0; u < CH; ++u)
@@ -760,51 +965,84 @@ __global__ void __launch_bounds__(256, 2) route_small_kernel(
     }
     __syncthreads();
     const float tau = (float)max(per + NW + 1, ROUTE_SMALL_TAU_MIN) * 5.9604645e-8f * 1.001f;
-    auto token_tau = [&](int tt, float (&ts)[NE]) {
+    static_assert(TB == NW, "a warp per token");
+    const int64_t t = t0 + warp;
+    float sv[NE];
+    uint32_t sure_in = 0, cand = 0;
+    int need = 0;
+    bool again = false;   // this warp's token is re-decided
+    uint32_t cm[NE];      // its candidates, bit e of slot i (none: certified, or no exact keys needed)
+#pragma unroll
+    for (int i = 0; i < NE; ++i) cm[i] = 0u;
+    if (warp < nt) {
+        float ts[NE], sg[NE];
         float q2 = 0.f;
 #pragma unroll
-        for (int q = 0; q < NW; ++q) q2 += s_x2[q][tt];
+        for (int q = 0; q < NW; ++q) q2 += s_x2[q][warp];
         const float xn = sqrtf(q2);
-#pragma unroll
-        for (int i = 0; i < NE; ++i) ts[i] = tau * s_w2[0][lane + 32 * i] * xn;
-    };
-    static_assert(TB == NW, "a warp per token");
-    const int tt = warp;
-    if (t0 + tt < T) {
-        float sv[NE], ts[NE], sg[NE];
 #pragma unroll
         for (int i = 0; i < NE; ++i) {
             float v = 0.f;
 #pragma unroll
-            for (int q = 0; q < NW; ++q) v += buf[(q * TB + tt) * EP + lane + 32 * i];
+            for (int q = 0; q < NW; ++q) v += buf[(q * TB + warp) * EP + lane + 32 * i];
             sv[i] = v;
+            ts[i] = tau * s_w2[0][lane + 32 * i] * xn;
         }
-        token_tau(tt, ts);
         uint32_t taken;
         if (select_certified<NE>(sv, ts, b, E, k, lane, sg, taken)) {
-            write_selection<NE>(taken, sg, t0 + tt, k, lane, idx, gate);
-        } else {   // listed; its logits stay in the first partial array
-            __syncwarp();
+            write_selection<NE>(taken, sg, t, k, lane, idx, gate);
+        } else {
+            again = true;
+            bound_candidates<NE>(sv, ts, b, E, k, lane, sure_in, cand);
+            int n_in = 0, n_cand = 0;
 #pragma unroll
-            for (int i = 0; i < NE; ++i) buf[tt * EP + lane + 32 * i] = sv[i];
-            if (lane == 0) s_list[atomicAdd(&s_nlist, 1)] = tt;
+            for (int i = 0; i < NE; ++i) {
+                n_in += __popc(__ballot_sync(0xffffffffu, (sure_in >> i) & 1u));
+                cm[i] = __ballot_sync(0xffffffffu, (cand >> i) & 1u);
+                n_cand += __popc(cm[i]);
+            }
+            need = k - n_in;
+            if (need < 0 || need > n_cand) {
+                if (lane == 0) report(st, MOEVIE_ERR_DEVICE, SITE_ROUTE_FALLBACK, (int)t, need);
+                need = -1;
+            }
+            if (need <= 0) {
+#pragma unroll
+                for (int i = 0; i < NE; ++i) cm[i] = 0u;
+            }
+            int m = 1;
+            for (int i = lane; i < d / 8; i += 32) m = max(m, bf16x8_exp_max(reinterpret_cast<const uint4*>(x + t * d)[i]));
+            m = __reduce_max_sync(0xffffffffu, m);
+            if (lane == 0) {
+                atomicAdd(&s_nlist, 1);
+                s_qx[warp] = m;
+            }
         }
     }
-    __syncthreads();
-    const int nlist = s_nlist;
-    for (int f = 0; f < nlist; ++f) {
-        const int tt = s_list[f];
-        redecide_token<NE>(
-            sh, reinterpret_cast<const uint16_t*>(x) + (t0 + tt) * d, nullptr, false, b, t0 + tt, d, E, k, idx, gate,
-            st,
-            [&](float (&sv)[NE], float (&ts)[NE]) {
+    if (lane == 0) {
 #pragma unroll
-                for (int i = 0; i < NE; ++i) sv[i] = buf[tt * EP + lane + 32 * i];
-                token_tau(tt, ts);
-            },
-            [&](int e) { return (int)s_wmax[0][e]; },
-            [&](int e, int i) { return __ldg(Wr + (int64_t)i * E + e); });
-        __syncthreads();   // sh is reused
+        for (int i = 0; i < NE; ++i) s_cand[warp][i] = cm[i];
+    }
+    __syncthreads();   // the fast logits in buf are done with, too
+    const int nlist = s_nlist;
+    if (nlist) {
+        route_small_exact<NE>(x + t0 * d, Wr, d, E, s_cand, s_qx, s_wmax[0],
+                              reinterpret_cast<ulonglong2*>(buf),
+                              reinterpret_cast<int*>(buf) + route_small_sums<NE> / 4, s_logit);
+        __syncthreads();
+        if (again && need >= 0) {
+            double exk[NE];
+            float sg[NE];
+#pragma unroll
+            for (int i = 0; i < NE; ++i) {
+                const int e = lane + 32 * i;
+                exk[i] = (cm[i] >> lane) & 1u ? 1.0 / (1.0 + exp(-s_logit[warp][e])) + (double)b[e] : -INFINITY;
+            }
+            const uint32_t chosen = choose_exact<NE>(exk, sure_in, cand, need, lane);
+#pragma unroll
+            for (int i = 0; i < NE; ++i) sg[i] = ((chosen >> i) & 1u) ? sigmoid_fast(sv[i]) : 0.f;
+            write_selection<NE>(chosen, sg, t, k, lane, idx, gate);
+        }
     }
     // tokens re-decided in this call: the last CTA publishes the sum and clears the counters
     if (threadIdx.x == 0) {
@@ -877,22 +1115,27 @@ cudaError_t launch_route_sum_parts(const float* logits, int64_t part_stride, int
 }
 
 // The one-launch router takes up to eight tokens for each SM (one wave of CTAs) and chunks
-// few enough: 32 ceil(E / 32) d <= 32768, so at most eight chunks a warp.  Measured against the
+// few enough: 32 ceil(E / 32) d <= ROUTE_SMALL_ED, so at most eight chunks a warp.  Measured against the
 // tensor-core route, back to back calls: T = 512, d = 768, E = 16 10.5 against 17.5 us, T = 256,
 // E = 31 12.8 against 18.0; past the line, T = 1024, d = 1536, E = 64 (24 chunks) 31 against 24.
+constexpr int ROUTE_SMALL_SMS = 152;
 bool route_small(int64_t T, int d, int E) {
-    return T >= 1 && T <= 8 * 152 && E <= 64 && (int64_t)(E + 31) / 32 * 32 * d <= 32768;
+    return T >= 1 && T <= RS_TB * ROUTE_SMALL_SMS && E <= 64 && (int64_t)(E + 31) / 32 * 32 * d <= ROUTE_SMALL_ED;
 }
 
 cudaError_t launch_route_small(const __nv_bfloat16* x, const float* Wr, const float* b, int T, int d, int E, int k,
                                int32_t* idx, float* gate, DevStatus* st, cudaStream_t s, float* zero,
                                int64_t zero_n) {
     if (!route_small(T, d, E)) return cudaErrorInvalidValue;
-    static_assert(route_small_smem<1>() <= 48 * 1024 && route_small_smem<2>() <= 48 * 1024, "no opt-in needed");
+    static_assert(route_small_smem<1>() <= 38 * 1024 && route_small_smem<2>() <= 38 * 1024,
+                  "no opt-in needed beside the static arrays (9 KB)");
+    // as few tokens a CTA as one wave of the SMs allows (a CTA takes as long with one as with eight),
+    // so that tokens that need the exact logits are spread over the SMs
+    const int tb = (T + ROUTE_SMALL_SMS - 1) / ROUTE_SMALL_SMS;
     const auto kern = E <= 32 ? route_small_kernel<1> : route_small_kernel<2>;
-    const cudaError_t e = launch_pdl(kern, dim3((unsigned)((T + RS_TB - 1) / RS_TB)), dim3(256),
-                                     E <= 32 ? route_small_smem<1>() : route_small_smem<2>(), s, x, Wr, b, T, d, E, k,
-                                     idx, gate, st, reinterpret_cast<float4*>(zero), zero ? zero_n / 4 : (int64_t)0);
+    const cudaError_t e = launch_pdl(kern, dim3((unsigned)((T + tb - 1) / tb)), dim3(256),
+                                     E <= 32 ? route_small_smem<1>() : route_small_smem<2>(), s, x, Wr, b, T, tb, d, E,
+                                     k, idx, gate, st, reinterpret_cast<float4*>(zero), zero ? zero_n / 4 : (int64_t)0);
     count_launches(1);
     return e;
 }
