@@ -33,60 +33,68 @@ __device__ __forceinline__ float warp_sum_f(float v) {
     return v;
 }
 
-// One warp per token: s_j = x_t . W_r[:, e_j] for its k experts (fp32, lanes over d; the
-// k dot products advance together, four steps' loads ahead of their sums: with one step's
-// loads in flight the chain of d / 32 load latencies took 30 us at T = 8192, d = 1024),
-// sigma_j = 1 / (1 + e^-s_j), S = sum_j sigma_j, g_j = sigma_j / S.  KB >= k.
-template <int KB>
-__global__ void __launch_bounds__(256) bwd_gates_kernel(const __nv_bfloat16* __restrict__ x,
-                                                        const float* __restrict__ wrt, int dp,
-                                                        const int32_t* __restrict__ idx, int64_t T,
-                                                        int d, int E, int k, float* __restrict__ sig,
-                                                        float* __restrict__ gate, DevStatus* st) {
+// One warp per token: s_j = x_t . W_r[:, e_j] for its k experts (fp32, lanes over d; KB dot
+// products advance together, U steps' loads ahead of their sums; KB = k up to 8, then passes of
+// 8 with MORE), sigma_j = 1 / (1 + e^-s_j), S = sum_j sigma_j, g_j = sigma_j / S.  The selected
+// rows of W_r come from L2; what bounds it is how many of their loads are in flight, so the
+// loads are unconditional and the registers leave room for four CTAs on an SM.  At T =
+// 8192, d = 1024, E = 64, in us:                   k = 1     4     8     9    16    32
+//   this form                                        6.4  11.6  17.7  28.1  31.8  57.3
+//   KB = 4, 8 or 32 >= k, U = 4, 4, 1 (116 to 204
+//   registers from KB = 8 on)                       16.6  17.7  30.4   158   184   268
+//   loads skipped where j >= k, U = 1               16.9  21.8  23.3   107   123   159
+template <int KB, bool MORE, int U, int CTAS>
+__global__ void __launch_bounds__(256, CTAS) bwd_gates_kernel(const __nv_bfloat16* __restrict__ x,
+                                                              const float* __restrict__ wrt, int dp,
+                                                              const int32_t* __restrict__ idx, int64_t T,
+                                                              int d, int E, int k, float* __restrict__ sig,
+                                                              float* __restrict__ gate, DevStatus* st) {
     pdl_wait();
     const int lane = threadIdx.x & 31;
     const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (t >= T) return;
     const __nv_bfloat16* xr = x + t * d;
-    const float* w[KB];   // past k and for bad ids: any row, unused
-    float acc[KB];
-    uint32_t okm = 0;
+    const int n = MORE ? k : KB;
+    float ssum = 0.f, mine = 0.f;   // lane j keeps sigma_j
+    for (int j0 = 0; j0 < n; j0 += KB) {
+        int w[KB];   // offsets of the rows (E dp < 2^31: E <= 1024, d < 2^16); bad ids and past k: row 0, unused
+        float acc[KB];
+        uint32_t okm = 0;
 #pragma unroll
-    for (int j = 0; j < KB; ++j) {
-        acc[j] = 0.f;
-        const int e = j < k ? idx[t * k + j] : 0;
-        const bool ok = e >= 0 && e < E;
-        if (j < k && !ok && lane == 0) report(st, MOEVIE_ERR_DEVICE, SITE_PERMUTE_ID, (int)(t * k + j), e);
-        if (j < k && ok) okm |= 1u << j;
-        w[j] = wrt + (int64_t)(ok ? e : 0) * dp;
-    }
-    constexpr int U = KB <= 8 ? 4 : 1;
-    int i = lane;
-    for (; i + 32 * (U - 1) < d; i += 32 * U) {
-        float xi[U], wv[U][KB];
+        for (int j = 0; j < KB; ++j) {
+            acc[j] = 0.f;
+            const int e = !MORE || j0 + j < k ? idx[t * k + j0 + j] : 0;
+            const bool ok = e >= 0 && e < E;
+            if (!ok && lane == 0) report(st, MOEVIE_ERR_DEVICE, SITE_PERMUTE_ID, (int)(t * k + j0 + j), e);
+            if (ok) okm |= 1u << j;
+            w[j] = (ok ? e : 0) * dp;
+        }
+        int i = lane;
+        for (; i + 32 * (U - 1) < d; i += 32 * U) {
+            float xi[U], wv[U][KB];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            xi[u] = __bfloat162float(xr[i + 32 * u]);
+            for (int u = 0; u < U; ++u) {
+                xi[u] = __bfloat162float(xr[i + 32 * u]);
 #pragma unroll
-            for (int j = 0; j < KB; ++j) wv[u][j] = __ldg(w[j] + i + 32 * u);
+                for (int j = 0; j < KB; ++j) wv[u][j] = __ldg(wrt + w[j] + i + 32 * u);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int j = 0; j < KB; ++j) acc[j] = fmaf(xi[u], wv[u][j], acc[j]);
+        }
+        for (; i < d; i += 32) {
+            const float xi = __bfloat162float(xr[i]);
+#pragma unroll
+            for (int j = 0; j < KB; ++j) acc[j] = fmaf(xi, __ldg(wrt + w[j] + i), acc[j]);
         }
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-#pragma unroll
-            for (int j = 0; j < KB; ++j) acc[j] = fmaf(xi[u], wv[u][j], acc[j]);
-    }
-    for (; i < d; i += 32) {
-        const float xi = __bfloat162float(xr[i]);
-#pragma unroll
-        for (int j = 0; j < KB; ++j) acc[j] = fmaf(xi, __ldg(w[j] + i), acc[j]);
-    }
-    float ssum = 0.f, mine = 0.f;   // lane j keeps sigma_j
-#pragma unroll
-    for (int j = 0; j < KB; ++j) {
-        if (j >= k) break;
-        const float sgm = 1.0f / (1.0f + expf(-warp_sum_f((okm >> j) & 1u ? acc[j] : 0.f)));
-        if (lane == j) mine = sgm;
-        ssum += sgm;
+        for (int j = 0; j < KB; ++j) {
+            if (MORE && j0 + j >= k) break;
+            const float sgm = 1.0f / (1.0f + expf(-warp_sum_f((okm >> j) & 1u ? acc[j] : 0.f)));
+            if (lane == j0 + j) mine = sgm;
+            ssum += sgm;
+        }
     }
     if (lane < k) {
         sig[t * k + lane] = mine;
@@ -346,10 +354,15 @@ cudaError_t launch_bwd_gates(const __nv_bfloat16* x, const float* wrt, int dp, c
                              int d, int E, int k, float* sig, float* gate, DevStatus* st, cudaStream_t s) {
     const dim3 grid((unsigned)((T * 32 + 255) / 256));
     cudaError_t e;
-    if (k <= 4) e = launch_pdl(bwd_gates_kernel<4>, grid, dim3(256), 0, s, x, wrt, dp, idx, T, d, E, k, sig, gate, st);
-    else if (k <= 8) e = launch_pdl(bwd_gates_kernel<8>, grid, dim3(256), 0, s, x, wrt, dp, idx, T, d, E, k, sig, gate, st);
-    else if (k <= 32) e = launch_pdl(bwd_gates_kernel<32>, grid, dim3(256), 0, s, x, wrt, dp, idx, T, d, E, k, sig, gate, st);
-    else return cudaErrorInvalidValue;
+    using Kern = decltype(&bwd_gates_kernel<1, false, 4, 4>);
+    static const Kern kerns[9] = {
+        bwd_gates_kernel<8, true, 2, 4>,
+        bwd_gates_kernel<1, false, 8, 4>, bwd_gates_kernel<2, false, 4, 4>, bwd_gates_kernel<3, false, 4, 4>,
+        bwd_gates_kernel<4, false, 4, 4>, bwd_gates_kernel<5, false, 2, 4>, bwd_gates_kernel<6, false, 2, 4>,
+        bwd_gates_kernel<7, false, 2, 4>, bwd_gates_kernel<8, false, 2, 4>};
+    if (k < 1 || k > 32) return cudaErrorInvalidValue;
+    const Kern kern = kerns[k <= 8 ? k : 0];
+    e = launch_pdl(kern, grid, dim3(256), 0, s, x, wrt, dp, idx, T, d, E, k, sig, gate, st);
     count_launches(1);
     return e;
 }
