@@ -912,23 +912,29 @@ __device__ void epilogue(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64
     }
 }
 
-// Epilogue of the bf16 outputs (GELU, SwiGLU, plain; the training path's also keep the
-// pre-activations).  Warp w reads TMEM lanes 32 (w % 4) .. +31 (its rows); each thread forms
-// 32 (training path 16) columns of its own row at a time, and the warp's 32 rows pass a buffer in shared
-// memory, from which whole sectors are stored, 64 (training path 32) bytes of a row by
-// neighbouring lanes.  Stored by each thread straight from its registers they left as
-// 16-byte pieces of 32 different lines an instruction; staged, for one stage of the operand
-// ring: up-projection T = 65536, d = 1664, E = 256 612 -> 593 us, T = 32768, E = 128 287 -> 268,
-// T = 8192, d = 1280, h = 854 (SwiGLU) 208 -> 203, T = 8192, d = 1024, E = 64 unchanged (84).
-template <bool TRAIN>
+// Epilogue of the bf16 outputs (gathered rows: GELU or SwiGLU; dense rows: GELU or plain; the
+// training path's also keep the pre-activations).  Warp w reads TMEM lanes 32 (w % 4) .. +31 (its
+// rows); each thread forms 32 (training path 16) columns of its own row at a time, and the warp's 32
+// rows pass a buffer in shared memory, from which whole sectors are stored, 64 (training path 32)
+// bytes of a row by neighbouring lanes.  (Stored by each thread straight from its registers they
+// leave as 16-byte pieces of 32 different lines an instruction: up-projection T = 65536, d =
+// 1664, E = 256 612 us against 593, T = 32768, E = 128 287 against 268.)  Below about 1024 columns of K
+// the instructions of this epilogue bound the launch, 256 columns a tile against K / 64 stages, so
+// what does not change is formed once a tile or a launch: the copies' addresses, and whether
+// there is an activation (a template parameter).  Up-projection, addresses formed and the
+// activation looked up at every piece -> this form, T = 8192: d = 512, E = 8, k = 2, h = 1000
+// 33.1 -> 29.1 us (straight from registers 29.0), d = 512, E = 64, h = 256 33.7 -> 29.0, d = 768 36.6 -> 34.9,
+// d = 1024, E = 64, h = 512 66.2 -> 61.9 (70.5); T = 1024, d = 1536 41.7 -> 40.0 (42.8).
+template <bool TRAIN, bool GATHER, bool GELU>
 __device__ void epilogue_bf16(const GemmArgs& p, const Smem& sm, uint32_t tmem, int64_t n_work,
                               volatile int* abort_flag) {
     constexpr int COLS = TRAIN ? 16 : 32, NP = COLS / 8;   // columns a step, 16-byte pieces of a row
     constexpr int ARR = 32 * COLS * 2;                     // bytes of one array's step
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int quad = warp & 3, half = warp >> 2;
-    const int nchunk = p.swiglu ? p.BN / 64 : p.BN / 32;   // 32-column chunks of the output
-    const int up0 = p.swiglu ? p.BN / 2 : 0;               // SwiGLU: first accumulator column of the up projection
+    const bool swiglu = GATHER && p.swiglu;
+    const int nchunk = swiglu ? p.BN / 64 : p.BN / 32;   // 32-column chunks of the output
+    const int up0 = swiglu ? p.BN / 2 : 0;               // SwiGLU: first accumulator column of the up projection
     // bf16 results are written once and read back later: let them leave L2 first
     const uint64_t stream_pol = l2_policy_evict_first();
     const uint32_t tempty_leader = peer_addr(sm.tempty, 0);
@@ -936,6 +942,10 @@ __device__ void epilogue_bf16(const GemmArgs& p, const Smem& sm, uint32_t tmem, 
     // piece q of row r at r * 2 COLS + 16 (q ^ swizzle(r)): eight consecutive rows' pieces (the
     // threads' writes) and eight consecutive pieces (the copies out) hit all banks
     auto place = [](int r, int q) { return r * (2 * COLS) + 16 * (q ^ (NP == 4 ? (r >> 1) & 3 : (r >> 2) & 1)); };
+    // copied out: piece q0 of rows r0, r0 + RS, ... (RS rows on the swizzle is the same)
+    constexpr int RS = 32 / NP, STEP = RS * 2 * COLS;
+    const int r0 = lane / NP, q0 = lane % NP;
+    const uint8_t* from = buf + place(r0, q0);
     if (sm.pair >= n_work) return;
     TileLd nl = tile_load(p, sm.pair);   // one item ahead
     int it = 0;
@@ -956,69 +966,86 @@ __device__ void epilogue_bf16(const GemmArgs& p, const Smem& sm, uint32_t tmem, 
             __syncwarp();
             if (lane == 0) mbar_arrive_remote(tempty_leader + 8 * acc);
         }
+        const int64_t off0 = (row0 + r0) * p.ldo + t.n0 + 8 * q0;
+        auto put = [&](int arr, int at, const float (&o)[8]) {
+            uint4 u;
+            u.x = pack_bf16x2(o[0], o[1]);
+            u.y = pack_bf16x2(o[2], o[3]);
+            u.z = pack_bf16x2(o[4], o[5]);
+            u.w = pack_bf16x2(o[6], o[7]);
+            *reinterpret_cast<uint4*>(buf + arr * ARR + at) = u;
+        };
+        // eight accumulator columns x (SwiGLU: the gate's, y the up projection's) into piece q of the lane's row
+        auto act8 = [&](const uint32_t* x, const uint32_t* y, int q) {
+            float f[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(x[i]);
+            const int at = place(lane, q);
+            if (TRAIN && p.out2) put(1, at, f);   // the pre-activation (SwiGLU: the gate's) as well
+            if (swiglu) {
+                float g[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) g[i] = __uint_as_float(y[i]);
+                if (TRAIN && p.out2) put(2, at, g);
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    // SiLU(u) v = u v / (1 + e^-u); e^-u = inf for u far below 0 gives 0
+                    f[i] = __fdividef(f[i], 1.0f + __expf(-f[i])) * g[i];
+            } else if (GELU) {
+#pragma unroll
+                for (int i = 0; i < 8; i += 2) gelu_erf2(f[i], f[i + 1]);
+            }
+            put(0, at, f);
+        };
+        auto release = [&]() {   // this warp's last read of the accumulator
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_remote(tempty_leader + 8 * acc);
+        };
+        auto copy_out = [&](int c) {   // the step's rows, written by all lanes, to columns t.n0 + c ..
+            __syncwarp();
+            const bool ok = t.n0 + c + 8 * q0 < p.N;
+            uint4 m[NP];
+#pragma unroll
+            for (int i = 0; i < NP; ++i) {
+                m[i] = *reinterpret_cast<const uint4*>(from + i * STEP);
+                if (TRAIN && p.out2 && ok && r0 + RS * i < nrow) {
+                    const int64_t off = off0 + c + i * (RS * p.ldo);
+                    *reinterpret_cast<uint4*>(p.out2 + off) = *reinterpret_cast<const uint4*>(from + i * STEP + ARR);
+                    if (swiglu)
+                        *reinterpret_cast<uint4*>(p.out3 + off) = *reinterpret_cast<const uint4*>(from + i * STEP + 2 * ARR);
+                }
+            }
+            __syncwarp();   // read before the next step overwrites it
+#pragma unroll
+            for (int i = 0; i < NP; ++i)
+                if (ok && r0 + RS * i < nrow) st_global_v4_hint(p.out + off0 + c + i * (RS * p.ldo), m[i], stream_pol);
+        };
         for (int ch = half; ch < nchunk; ch += 2) {
+            if (!TRAIN && !swiglu) {
+                uint32_t v[32];
+                tmem_ld_32x32b_x32(tbase + ch * 32, v);
+                tmem_wait_ld();
+                if (ch + 2 >= nchunk) release();
 #pragma unroll
-            for (int c0 = 0; c0 < 32; c0 += COLS) {
-                const int c = ch * 32 + c0;
+                for (int q = 0; q < 4; ++q) act8(v + 8 * q, v + 8 * q, q);
+                copy_out(ch * 32);
+            } else {
 #pragma unroll
-                for (int s0 = 0; s0 < COLS; s0 += 16) {
-                    uint32_t x[16], y[16];
-                    tmem_ld_32x32b_x16(tbase + c + s0, x);
-                    if (p.swiglu) tmem_ld_32x32b_x16(tbase + up0 + c + s0, y);
-                    tmem_wait_ld();
-                    if (ch + 2 >= nchunk && c0 + s0 + 16 == 32) {   // this warp's last read of the accumulator
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive_remote(tempty_leader + 8 * acc);
+                for (int c0 = 0; c0 < 32; c0 += COLS) {
+                    const int c = ch * 32 + c0;
+#pragma unroll
+                    for (int s0 = 0; s0 < COLS; s0 += 16) {
+                        uint32_t x[16], y[16];
+                        tmem_ld_32x32b_x16(tbase + c + s0, x);
+                        if (swiglu) tmem_ld_32x32b_x16(tbase + up0 + c + s0, y);
+                        tmem_wait_ld();
+                        if (ch + 2 >= nchunk && c0 + s0 + 16 == 32) release();
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) act8(x + 8 * q, y + 8 * q, s0 / 8 + q);
                     }
-#pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        float f[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(x[8 * q + i]);
-                        const int at = place(lane, s0 / 8 + q);
-                        auto put = [&](int arr, const float (&o)[8]) {
-                            uint4 u;
-                            u.x = pack_bf16x2(o[0], o[1]);
-                            u.y = pack_bf16x2(o[2], o[3]);
-                            u.z = pack_bf16x2(o[4], o[5]);
-                            u.w = pack_bf16x2(o[6], o[7]);
-                            *reinterpret_cast<uint4*>(buf + arr * ARR + at) = u;
-                        };
-                        if (TRAIN && p.out2) put(1, f);   // the pre-activation (SwiGLU: the gate's) as well
-                        if (p.swiglu) {
-                            float g[8];
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) g[i] = __uint_as_float(y[8 * q + i]);
-                            if (TRAIN && p.out2) put(2, g);
-#pragma unroll
-                            for (int i = 0; i < 8; ++i)
-                                // SiLU(u) v = u v / (1 + e^-u); e^-u = inf for u far below 0 gives 0
-                                f[i] = __fdividef(f[i], 1.0f + __expf(-f[i])) * g[i];
-                        } else if (p.epi == EPI_GELU_BF16 || (TRAIN && p.epi == EPI_GELU2_BF16)) {
-#pragma unroll
-                            for (int i = 0; i < 8; i += 2) gelu_erf2(f[i], f[i + 1]);
-                        }
-                        put(0, f);
-                    }
+                    copy_out(c);
                 }
-                __syncwarp();   // the step's rows, written by all lanes
-                const int n = t.n0 + c;
-#pragma unroll
-                for (int i = 0; i < NP; ++i) {
-                    const int r = (lane + 32 * i) / NP, q = (lane + 32 * i) % NP;
-                    if (r < nrow && n + 8 * q < p.N) {
-                        const int64_t off = (row0 + r) * p.ldo + n + 8 * q;
-                        const uint8_t* from = buf + place(r, q);
-                        st_global_v4_hint(p.out + off, *reinterpret_cast<const uint4*>(from), stream_pol);
-                        if (TRAIN && p.out2) {
-                            *reinterpret_cast<uint4*>(p.out2 + off) = *reinterpret_cast<const uint4*>(from + ARR);
-                            if (p.swiglu)
-                                *reinterpret_cast<uint4*>(p.out3 + off) = *reinterpret_cast<const uint4*>(from + 2 * ARR);
-                        }
-                    }
-                }
-                __syncwarp();   // copied out before the next step overwrites it
             }
         }
     }
@@ -1240,7 +1267,10 @@ __global__ void __launch_bounds__(GM_THREADS, 1) grouped_gemm_kernel(const __gri
         if constexpr (ECLS == ECLS_ADDT) epilogue_addt<TRAIN>(p, sm, tmem, n_work, warp, abort_flag);
         else if constexpr (ECLS == ECLS_DGELU) epilogue_dact<false>(p, sm, tmem, n_work, abort_flag);
         else if constexpr (ECLS == ECLS_DSWIGLU) epilogue_dact<true>(p, sm, tmem, n_work, abort_flag);
-        else if constexpr (ECLS == ECLS_BF16) epilogue_bf16<TRAIN>(p, sm, tmem, n_work, abort_flag);
+        else if constexpr (ECLS == ECLS_BF16) {
+            if (GATHER || p.epi == EPI_GELU_BF16) epilogue_bf16<TRAIN, GATHER, true>(p, sm, tmem, n_work, abort_flag);
+            else epilogue_bf16<TRAIN, GATHER, false>(p, sm, tmem, n_work, abort_flag);
+        }
         else epilogue<ECLS, TRAIN>(p, sm, tmem, n_work, abort_flag);
     } else if (warp == GM_WARP_MMA) {
         if (sm.rank == 0) mma_issuer<TRAIN, ECLS == ECLS_F32, ECLS == ECLS_ADDT>(p, sm, tmem, n_work, abort_flag);
@@ -1413,7 +1443,7 @@ cudaError_t launch_grouped_gemm(const GemmArgs& a, int grid, cudaStream_t s) {
                        a.epi == EPI_DGELU_BF16 || a.epi == EPI_DSWIGLU_BF16 || a.out2 != nullptr;
     const bool bf16_out = a.epi == EPI_GELU_BF16 || a.epi == EPI_STORE_BF16 || a.epi == EPI_SWIGLU_BF16 ||
                           a.epi == EPI_GELU2_BF16 || a.epi == EPI_DGELU_BF16 || a.epi == EPI_DSWIGLU_BF16;
-    if (gathered && !bf16_out) return cudaErrorInvalidValue;
+    if (gathered && (!bf16_out || a.epi == EPI_STORE_BF16)) return cudaErrorInvalidValue;
     if (!gathered && a.epi == EPI_SWIGLU_BF16) return cudaErrorInvalidValue;
     if (a.trans && (a.epi != EPI_ADD_F32 || a.item_table)) return cudaErrorInvalidValue;
     int which;
