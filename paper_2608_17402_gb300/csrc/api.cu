@@ -312,7 +312,7 @@ moevie_status run_gemm(const GemmSpec& g, DevStatus* st, cudaStream_t s) {
     a.A = static_cast<const __nv_bfloat16*>(g.A);
     a.lda = g.lda;
     a.a_rows = g.a_rows;
-    a.a_div = g.a_div > 0 ? g.a_div : 1;
+    div_by_mul(g.a_div > 0 ? g.a_div : 1, &a.a_div_mul, &a.a_div_shift);
     a.a_kperiod = g.a_kperiod;
     a.a_nrows = g.a_nrows;
     a.m_total = g.m_total;

@@ -257,6 +257,16 @@ enum Epilogue : int {
     EPI_DSWIGLU_BF16 = 8,// SwiGLU a = SiLU(u) v: out = du = bf16(scale acc v SiLU'(u)), out2 = dv =
                          //   bf16(scale acc SiLU(u)), and the row dot sum_n acc a as for EPI_DGELU_BF16
 };
+// Division of 0 <= r < 2^31 by a constant as a multiplication (Granlund and Montgomery, "Division
+// by Invariant Integers using Multiplication", 1994): with 2^(l - 1) < div <= 2^l, shift = 31 + l and mul
+// = floor(2^shift / div) + 1 < 2^32, r mul exceeds r 2^shift / div by at most r < 2^31 <= 2^shift / div.
+inline void div_by_mul(int div, uint32_t* mul, int* shift) {
+    int l = 0;
+    while ((int64_t(1) << l) < div) ++l;
+    *shift = 31 + l;
+    *mul = (uint32_t)((uint64_t(1) << *shift) / (uint64_t)div + 1);
+}
+
 struct GemmArgs {
     CUtensorMap tmB;            // B = weights [G][K][N] bf16 (N contiguous), 3-D map {N, K, G}
     CUtensorMap tmB2;           // groups g >= g_split: B from this map, group g - g_split
@@ -271,7 +281,8 @@ struct GemmArgs {
     const __nv_bfloat16* A;     // A rows, for the token gather
     int64_t lda;
     const int32_t* a_rows;      // A row of GEMM row r: a_rows ? a_rows[r] / a_div : r (gather)
-    int a_div;
+    uint32_t a_div_mul;         // r / a_div as r a_div_mul >> a_div_shift for 0 <= r < 2^31 (div_by_mul)
+    int a_div_shift;
     int a_kperiod;              // 0, or a multiple of 64: column of K index kk in A is kk % a_kperiod
     int64_t a_nrows;            // rows of A; a gathered row outside [0, a_nrows) is a device error
     int64_t m_total;            // GEMM rows that may be written
