@@ -657,94 +657,112 @@ constexpr size_t route_small_smem() {
     constexpr size_t exact = route_small_sums<NE> + 4 * RS_G<NE> * (ROUTE_SMALL_ED / EP);   // route_small_exact's sums and xp
     return logits > exact ? logits : exact;
 }
-// Exact logits of the uncertified tokens of a CTA of route_small_kernel (RS_TB tokens from xg, RS_NW
-// warps): logit[tt][e] for the candidates cand[tt], from the same long accumulators as
+// Exact keys of the uncertified tokens `list` of a CTA of route_small_kernel (x rows from xg on, ldx
+// apart, RS_NW warps): key[tt][e] for the candidates cand[tt], from the same long accumulators as
 // route_fallback_kernel's and with the same windows (wmax: the columns' largest exponent fields).
-// A token with at most FB_BATCH candidates takes the threads over the d terms.  Tokens with more go
-// RS_G together, lanes over the experts: the weights are read as whole rows of W_r and taken
-// apart once for those tokens, the warps (with E <= 16 also the parts of a warp) share the
-// terms, and a pass costs the same however many of the experts tie.  The integer instructions bound
-// it (about 20 a term).  The whole router on tokens that tie in every key (W_r = 0, b = 0): 32 us at
-// T = 64, d = 1024, E = 32 and 98 us at T = 1216, d = 512, E = 64, against 57 and 186 of the
-// tensor-core route, and 330 and 470 with the threads over the terms for any number of candidates
-// and the eight tokens of a CTA one after another through all of their steps.  Not inlined: its
-// registers are not to crowd the kernel's main loop.
-// sums: the warps' sums, [2][RS_NW][EP] (two tokens in turn) or [RS_G][RS_NW][EP]; xp: the
+// The tokens with at most FB_BATCH candidates go all at once, the eight warps shared among them, lanes
+// over the d terms: a call with one such token takes 4 us longer than one with none, mostly to
+// fetch this code (four terms unrolled: 0.3 us more).  Tokens with more candidates go RS_G together,
+// lanes over the experts: the weights are read as whole rows of W_r and taken apart once for those
+// tokens, the warps (with E <= 16 also the parts of a warp) share the terms, and a pass costs
+// the same however many of the experts tie; the integer instructions bound it (about 20 a term).
+// The whole router on tokens that tie in every key (W_r = 0, b = 0): 32 us at T = 64, d = 1024, E =
+// 32, 98 at T = 1216, d = 512, E = 64, against 57 and 186 of the tensor-core route; on 1216 tokens
+// with two candidates each (d = 1024, E = 32) 27 against 31.  One token after another through all of
+// its steps, the threads over the terms for any number of candidates: 330, 470 and 57.
+// sums: the warps' sums, [RS_NW][FB_BATCH] and the candidates' ids, or [RS_G][RS_NW][EP]; xp: the
 // tokens' x as (mantissa << 16 | exponent), [RS_G][d].
 template <int NE>
-__device__ __noinline__ void route_small_exact(const __nv_bfloat16* __restrict__ xg, const float* __restrict__ Wr,
-                                               int d, int E, const uint32_t (*cand)[NE], const int* qx,
-                                               const uint32_t* wmax, ulonglong2* sums, int* xp,
-                                               double (*logit)[32 * NE]) {
+__device__ __forceinline__ void route_small_exact(uint32_t list, const __nv_bfloat16* __restrict__ xg, int64_t ldx,
+                                                  const float* __restrict__ Wr, int d, int E,
+                                                  const uint32_t (*cand)[NE], const int* qx, const uint32_t* wmax,
+                                                  const float* __restrict__ b, ulonglong2* sums, int* xp,
+                                                  double (*key)[32 * NE]) {
     constexpr int EP = 32 * NE, NW = RS_NW, G = RS_G<NE>;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     auto window = [&](int tt, int e) { return qx[tt] == 255 || wmax[e] == 255u ? -1 : qx[tt] + (int)wmax[e]; };   // -1: NaN
     auto put = [&](int at, const unsigned __int128& a) {
         sums[at] = make_ulonglong2((unsigned long long)(uint64_t)a, (unsigned long long)(uint64_t)(a >> 64));
     };
-    // the sum over the warps of token tt, expert e (part `from` of sums)
-    auto finish = [&](int tt, int e, int from) {
-        if (!((cand[tt][e / 32] >> (e & 31)) & 1u)) return;
+    // the key of token tt, expert e from its n parts sums[at], sums[at + by], ...
+    auto finish = [&](int tt, int e, int at, int by, int n) {
         const int Q = window(tt, e);
         double v = __longlong_as_double(0x7ff8000000000000ll);
         if (Q > 0) {
             unsigned __int128 u = 0;
-#pragma unroll
-            for (int q = 0; q < NW; ++q) {
-                const ulonglong2 a = sums[(from * NW + q) * EP + e];
+            for (int q = 0; q < n; ++q) {
+                const ulonglong2 a = sums[at + q * by];
                 u += ((unsigned __int128)a.y << 64) | a.x;
             }
             v = long_acc_value(u, Q);
         }
-        logit[tt][e] = v;
+        key[tt][e] = 1.0 / (1.0 + exp(-v)) + (double)b[e];
     };
-    uint32_t wide = 0;   // tokens with more than FB_BATCH candidates (the same for the whole CTA, as all that branches on it)
-    int buf = 0;
-    for (int tt = 0; tt < RS_TB; ++tt) {
-        uint32_t cm[NE];
+    // (the same for the whole CTA, as all that branches on them)
+    uint32_t few = 0, wide = 0;   // tokens with at most FB_BATCH candidates; with more
+    for (; list; list &= list - 1u) {
+        const int tt = __ffs(list) - 1;
         int n = 0;
 #pragma unroll
-        for (int i = 0; i < NE; ++i) {
-            cm[i] = cand[tt][i];
-            n += __popc(cm[i]);
-        }
+        for (int i = 0; i < NE; ++i) n += __popc(cand[tt][i]);
         if (n > FB_BATCH) wide |= 1u << tt;
-        if (n == 0 || n > FB_BATCH) continue;
-        const uint16_t* xr = reinterpret_cast<const uint16_t*>(xg) + (int64_t)tt * d;
-        unsigned __int128 acc[FB_BATCH];
-        int ec[FB_BATCH], Q[FB_BATCH];
+        else if (n > 0) few |= 1u << tt;
+    }
+    if (few) {
+        const int n = __popc(few), P = n > 4 ? 8 : n > 2 ? 4 : n;   // P tokens at once, NW / P warps each
+        static_assert(RS_TB == 8 && NW == 8, "a warp a token at least");
+        int* ids = reinterpret_cast<int*>(sums + NW * FB_BATCH);    // [NW][FB_BATCH] the candidates, -1: none
+        auto token = [&](int j) {   // the j-th of them
+            uint32_t m = few;
+            for (; j > 0; --j) m &= m - 1u;
+            return __ffs(m) - 1;
+        };
+        if (warp % P < n) {
+            const int tt = token(warp % P);
+            const uint16_t* xr = reinterpret_cast<const uint16_t*>(xg) + tt * ldx;
+            uint32_t cm[NE];
 #pragma unroll
-        for (int c = 0; c < FB_BATCH; ++c) {   // candidate c: the lowest id left
-            acc[c] = 0;
-            ec[c] = -1;
+            for (int i = 0; i < NE; ++i) cm[i] = cand[tt][i];
+            const int step = 32 * (NW / P);
+#pragma unroll 1
+            for (int c = 0; c < FB_BATCH; c += 2) {   // mostly there are two; one copy of the code, which is fetched cold
+                int e[2], Q[2];
+                unsigned __int128 acc[2];
 #pragma unroll
-            for (int i = 0; i < NE; ++i)
-                if (ec[c] < 0 && cm[i]) {
-                    ec[c] = 32 * i + __ffs(cm[i]) - 1;
-                    cm[i] &= cm[i] - 1u;
+                for (int v = 0; v < 2; ++v) {   // the lowest id left
+                    e[v] = -1;
+#pragma unroll
+                    for (int i = 0; i < NE; ++i)
+                        if (e[v] < 0 && cm[i]) {
+                            e[v] = 32 * i + __ffs(cm[i]) - 1;
+                            cm[i] &= cm[i] - 1u;
+                        }
+                    if (lane == 0) ids[warp * FB_BATCH + c + v] = e[v];
+                    Q[v] = e[v] >= 0 ? window(tt, e[v]) : -1;
+                    acc[v] = 0;
                 }
-            Q[c] = ec[c] >= 0 ? window(tt, ec[c]) : -1;
-        }
-        for (int i = threadIdx.x; i < d; i += 32 * NW) {
-            const uint32_t hx = xr[i];
-            uint32_t uw[FB_BATCH];
+                if (Q[0] <= 0 && Q[1] <= 0) continue;
+#pragma unroll 1
+                for (int i = warp / P * 32 + lane; i < d; i += step) {
+                    const uint32_t hx = xr[i];
+                    uint32_t uw[2];
 #pragma unroll
-            for (int c = 0; c < FB_BATCH; ++c)
-                uw[c] = Q[c] > 0 ? __float_as_uint(__ldg(Wr + (int64_t)i * E + ec[c])) : 0u;
+                    for (int v = 0; v < 2; ++v) uw[v] = Q[v] > 0 ? __float_as_uint(__ldg(Wr + (int64_t)i * E + e[v])) : 0u;
 #pragma unroll
-            for (int c = 0; c < FB_BATCH; ++c)
-                if (Q[c] > 0) long_acc_term(hx, uw[c], Q[c], acc[c]);
-        }
+                    for (int v = 0; v < 2; ++v) long_acc_term(hx, uw[v], Q[v], acc[v]);   // (Q < 0: not used)
+                }
 #pragma unroll
-        for (int c = 0; c < FB_BATCH; ++c) {
-            if (Q[c] <= 0) continue;
-            const unsigned __int128 a = warp_sum_u128(acc[c]);
-            if (lane == 0) put((buf * NW + warp) * EP + ec[c], a);
+                for (int v = 0; v < 2; ++v) {
+                    acc[v] = warp_sum_u128(acc[v]);
+                    if (lane == 0) put(warp * FB_BATCH + c + v, acc[v]);
+                }
+            }
         }
         __syncthreads();
-        // (the token after the next writes this half again: after the next token's barrier)
-        if (threadIdx.x < EP) finish(tt, threadIdx.x, buf);
-        buf ^= 1;
+        if (threadIdx.x < n * FB_BATCH) {
+            const int j = threadIdx.x / FB_BATCH, c = threadIdx.x % FB_BATCH, e = ids[j * FB_BATCH + c];
+            if (e >= 0) finish(token(j), e, j * FB_BATCH + c, P * FB_BATCH, NW / P);
+        }
     }
     const int W = NE > 1 || E > 16 ? 32 : E > 8 ? 16 : 8;   // lanes over the experts; 32 / W parts of a warp
     const int sub = lane / W, le = lane % W, step = NW * (32 / W);
@@ -770,7 +788,7 @@ __device__ __noinline__ void route_small_exact(const __nv_bfloat16* __restrict__
         for (int u = 0; u < G; ++u)
             if (tok[u] >= 0)
                 for (int g = threadIdx.x; g < d / 8; g += 32 * NW) {
-                    const uint4 v = reinterpret_cast<const uint4*>(xg + (int64_t)tok[u] * d)[g];
+                    const uint4 v = reinterpret_cast<const uint4*>(xg + tok[u] * ldx)[g];
                     const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
                     int o[8];
 #pragma unroll
@@ -831,7 +849,8 @@ __device__ __noinline__ void route_small_exact(const __nv_bfloat16* __restrict__
             int tt = -1;
 #pragma unroll
             for (int v = 0; v < G; ++v) tt = u == v ? tok[v] : tt;
-            if (tt >= 0) finish(tt, threadIdx.x % EP, u);
+            const int e = threadIdx.x % EP;
+            if (tt >= 0 && ((cand[tt][e / 32] >> (e & 31)) & 1u)) finish(tt, e, u * NW * EP + e, EP, NW);
         }
     }
 }
@@ -840,7 +859,7 @@ __device__ __noinline__ void route_small_exact(const __nv_bfloat16* __restrict__
 constexpr int ROUTE_SMALL_TAU_MIN = 64;
 template <int NE>
 __global__ void __launch_bounds__(256, 1) route_small_kernel(
-    const __nv_bfloat16* __restrict__ x, const float* __restrict__ Wr, const float* __restrict__ b, int T, int tb, int d,
+    const __nv_bfloat16* __restrict__ x, const float* __restrict__ Wr, const float* __restrict__ b, int T, int d,
     int E, int k, int32_t* __restrict__ idx, float* __restrict__ gate, DevStatus* st, float4* __restrict__ zero,
     int64_t zero_n4) {
     pdl_wait();
@@ -861,22 +880,25 @@ __global__ void __launch_bounds__(256, 1) route_small_kernel(
     __shared__ uint32_t s_wmax[NW][EP]; // largest |w| bits, then exponent fields
     __shared__ float s_x2[NW][TB];
     __shared__ uint32_t s_cand[TB][NE];    // uncertified tokens: candidates of each 32-expert slot
-    __shared__ int s_qx[TB], s_nlist;      //   largest exponent field of x_t; their number
-    __shared__ double s_logit[TB][EP];     //   the candidates' exact logits
+    __shared__ int s_qx[TB];               //   largest exponent field of x_t
+    __shared__ uint32_t s_again;           //   which of the CTA's tokens they are
+    __shared__ double s_key[TB][EP];       //   the candidates' exact keys
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t t0 = (int64_t)blockIdx.x * tb;
-    const int nt = min(tb, (int)(T - t0));   // tokens of this CTA
-    if (threadIdx.x == 0) s_nlist = 0;
+    // this CTA's tokens: blockIdx.x + tt gridDim.x, so that neighbours that are alike fall to different CTAs
+    const int nt = ((int)T - 1 - (int)blockIdx.x) / (int)gridDim.x + 1;
+    auto token = [&](int tt) { return (int64_t)blockIdx.x + tt * (int64_t)gridDim.x; };
+    if (threadIdx.x == 0) s_again = 0u;
     float* xs = buf + warp * WBUF;
     float* ws = xs + CH * TB;
     const int per = (d / 8 + NW - 1) / NW * 8;   // d % 8 == 0: slices of whole groups of 8
     const int kbeg = warp * per, kend = min(d, kbeg + per);
     const int xt = lane % TB, xk = 8 * (lane / TB);   // this lane's piece of x: its token, its first column
+    const __nv_bfloat16* xp = x + token(xt) * d + xk;   // (xt past nt: not read)
     uint4 xr;
     float wv[CH][NE];
     auto load = [&](int k0) {   // chunk k0 .. k0 + CH - 1 into registers (zeros past kend, nt and E)
         const bool ok = lane < XPC && k0 + xk < kend && xt < nt;
-        xr = ok ? *reinterpret_cast<const uint4*>(x + (t0 + xt) * d + k0 + xk) : make_uint4(0u, 0u, 0u, 0u);
+        xr = ok ? *reinterpret_cast<const uint4*>(xp + k0) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
         for (int u = 0; u < CH; ++u)
 #pragma unroll
@@ -966,7 +988,7 @@ __global__ void __launch_bounds__(256, 1) route_small_kernel(
     __syncthreads();
     const float tau = (float)max(per + NW + 1, ROUTE_SMALL_TAU_MIN) * 5.9604645e-8f * 1.001f;
     static_assert(TB == NW, "a warp per token");
-    const int64_t t = t0 + warp;
+    const int64_t t = token(warp);
     float sv[NE];
     uint32_t sure_in = 0, cand = 0;
     int need = 0;
@@ -993,6 +1015,11 @@ __global__ void __launch_bounds__(256, 1) route_small_kernel(
             write_selection<NE>(taken, sg, t, k, lane, idx, gate);
         } else {
             again = true;
+            uint4 xv[4];   // the token's x row (d <= 1024), on its way while the keys are bounded
+            static_assert(ROUTE_SMALL_ED <= 32 * 4 * 32 * 8, "four pieces a lane");
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                xv[i] = lane + 32 * i < d / 8 ? reinterpret_cast<const uint4*>(x + t * d)[lane + 32 * i] : make_uint4(0u, 0u, 0u, 0u);
             bound_candidates<NE>(sv, ts, b, E, k, lane, sure_in, cand);
             int n_in = 0, n_cand = 0;
 #pragma unroll
@@ -1011,10 +1038,11 @@ __global__ void __launch_bounds__(256, 1) route_small_kernel(
                 for (int i = 0; i < NE; ++i) cm[i] = 0u;
             }
             int m = 1;
-            for (int i = lane; i < d / 8; i += 32) m = max(m, bf16x8_exp_max(reinterpret_cast<const uint4*>(x + t * d)[i]));
+#pragma unroll
+            for (int i = 0; i < 4; ++i) m = max(m, bf16x8_exp_max(xv[i]));
             m = __reduce_max_sync(0xffffffffu, m);
             if (lane == 0) {
-                atomicAdd(&s_nlist, 1);
+                atomicOr(&s_again, 1u << warp);
                 s_qx[warp] = m;
             }
         }
@@ -1024,11 +1052,11 @@ __global__ void __launch_bounds__(256, 1) route_small_kernel(
         for (int i = 0; i < NE; ++i) s_cand[warp][i] = cm[i];
     }
     __syncthreads();   // the fast logits in buf are done with, too
-    const int nlist = s_nlist;
-    if (nlist) {
-        route_small_exact<NE>(x + t0 * d, Wr, d, E, s_cand, s_qx, s_wmax[0],
+    const uint32_t list = s_again;
+    if (list) {
+        route_small_exact<NE>(list, x + token(0) * d, (int64_t)gridDim.x * d, Wr, d, E, s_cand, s_qx, s_wmax[0], b,
                               reinterpret_cast<ulonglong2*>(buf),
-                              reinterpret_cast<int*>(buf) + route_small_sums<NE> / 4, s_logit);
+                              reinterpret_cast<int*>(buf) + route_small_sums<NE> / 4, s_key);
         __syncthreads();
         if (again && need >= 0) {
             double exk[NE];
@@ -1036,7 +1064,7 @@ __global__ void __launch_bounds__(256, 1) route_small_kernel(
 #pragma unroll
             for (int i = 0; i < NE; ++i) {
                 const int e = lane + 32 * i;
-                exk[i] = (cm[i] >> lane) & 1u ? 1.0 / (1.0 + exp(-s_logit[warp][e])) + (double)b[e] : -INFINITY;
+                exk[i] = (cm[i] >> lane) & 1u ? s_key[warp][e] : -INFINITY;
             }
             const uint32_t chosen = choose_exact<NE>(exk, sure_in, cand, need, lane);
 #pragma unroll
@@ -1046,7 +1074,7 @@ __global__ void __launch_bounds__(256, 1) route_small_kernel(
     }
     // tokens re-decided in this call: the last CTA publishes the sum and clears the counters
     if (threadIdx.x == 0) {
-        if (nlist) atomicAdd(&st->route_sum, nlist);
+        if (list) atomicAdd(&st->route_sum, __popc(list));
         __threadfence();
         if (atomicAdd(&st->route_ticket, 1) == (int)gridDim.x - 1) {
             __threadfence();
@@ -1134,7 +1162,7 @@ cudaError_t launch_route_small(const __nv_bfloat16* x, const float* Wr, const fl
     const int tb = (T + ROUTE_SMALL_SMS - 1) / ROUTE_SMALL_SMS;
     const auto kern = E <= 32 ? route_small_kernel<1> : route_small_kernel<2>;
     const cudaError_t e = launch_pdl(kern, dim3((unsigned)((T + tb - 1) / tb)), dim3(256),
-                                     E <= 32 ? route_small_smem<1>() : route_small_smem<2>(), s, x, Wr, b, T, tb, d, E,
+                                     E <= 32 ? route_small_smem<1>() : route_small_smem<2>(), s, x, Wr, b, T, d, E,
                                      k, idx, gate, st, reinterpret_cast<float4*>(zero), zero ? zero_n / 4 : (int64_t)0);
     count_launches(1);
     return e;

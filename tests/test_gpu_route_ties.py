@@ -57,6 +57,28 @@ def test_groups_of_equal_experts(n, d, E):
     np.testing.assert_allclose(gate, ogate, rtol=0, atol=1e-5)
 
 
+@pytest.mark.parametrize("T", [152, 153, 305, 460, 610, 913, 1216])
+@pytest.mark.parametrize("d,E,some", [(200, 24, 1), (512, 40, 3)])
+def test_pairs_of_equal_experts_on_many_tokens(T, d, E, some):
+    """One to eight tokens a CTA, all of them (or every third) with two or four candidates for
+    the last place: odd k splits a pair of equal experts."""
+    rng = np.random.default_rng(T + E)
+    k = 3
+    xf = rng.standard_normal((T, d)).astype(np.float32)
+    xf[:, 0] = (np.arange(T) % some != 0) * 8.0     # moves the pairs apart on the other tokens
+    x = workloads.f32_to_bf16_bits(xf)
+    Wr = np.repeat((rng.standard_normal((d, E // 2)) * 0.02).astype(np.float32), 2, axis=1)
+    Wr[0, 1::2] += 0.05
+    b = np.repeat(rng.uniform(-0.1, 0.1, E // 2).astype(np.float32), 2)
+    b[2:4] = b[0:2]
+    Wr[:, 2:4] = Wr[:, 0:2]                         # and one group of four
+    idx, gate, nfb = _route(x, Wr, b, k)
+    oidx, ogate, _ = oracle.route(x, Wr, b, k)
+    assert nfb >= T // some
+    assert np.array_equal(idx, oidx)
+    np.testing.assert_allclose(gate, ogate, rtol=0, atol=1e-5)
+
+
 @pytest.mark.parametrize("pattern", ["halves", "alternating", "slices"])
 @pytest.mark.parametrize("d,E", [(1024, 32), (512, 64), (776, 31)])
 def test_rounding_errors_larger_than_the_gaps(pattern, d, E):
