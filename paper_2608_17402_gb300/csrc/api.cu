@@ -246,6 +246,21 @@ struct GemmSpec {
     float* dg_part;
 };
 
+// Whether the transposed product is the faster form of an accumulating GEMM of m_total rows in G
+// groups onto N columns.  Its tiles have 256 columns whatever N is, and their rows rounded up to
+// 64; the other form's have BN columns (choose_bn) and 256 rows.  So with r rows a group it does
+// (r + 32) 256 against (r + 128) BN of MMAs a group and n-tile on average, and it is taken up to
+// 1.1 times as many (its reductions are cheaper).  Transposed / staged, down-projections in us:
+// BN = 256 (T = 8192, E = 64, d = 1024) 72 / 76; BN = 224 (T = 8192, E = 32) d = 640 31.1 / 31.8, d =
+// 1288 63.2 / 59.8; BN = 192, d = 576: r = 1024 51.6 / 49.1, r = 503 13.7 / 13.3, r = 251 24.6 / 23.6, r
+// = 64 20.0 / 22.3.  Whole forwards at T = 32768, E = 64, k = 8, h = 128 (SwiGLU): d = 64 177 / 153, d =
+// 264 254 / 236.
+bool transposed_pays(int64_t m_total, int G, int N) {
+    int bn = 0, nnt = 0;
+    choose_bn(N, &bn, &nnt);
+    return 10 * (m_total + 32 * (int64_t)G) * GM_BM <= 11 * (m_total + 128 * (int64_t)G) * bn;
+}
+
 moevie_status run_gemm(const GemmSpec& g, DevStatus* st, cudaStream_t s) {
     GemmArgs a;
     memset(&a, 0, sizeof a);
@@ -253,12 +268,10 @@ moevie_status run_gemm(const GemmSpec& g, DevStatus* st, cudaStream_t s) {
     if (n_ld < g.N || n_ld % 8 != 0) return MOEVIE_ERR_UNSUPPORTED;
     const bool swiglu = g.epi == EPI_SWIGLU_BF16;
     // Rows reduced into their tokens' rows: the transposed product (256 output columns a tile,
-    // N = the tile's rows), unless the items are band-ordered.  Measured, down-projection with
-    // staged 16-byte reductions -> transposed: T = 8192, d = 1024, E = 64 100 -> 95 us;
-    // T = 1024, d = 1536, E = 64 (one partial tile an expert) 47 -> 41 us; band-ordered,
-    // where DRAM traffic bounds the launch: T = 32768, E = 128 397 -> 393 us, T = 65536,
-    // E = 256 925 -> 1010 us.
-    a.trans = g.epi == EPI_ADD_F32 && !g.item_table ? 1 : 0;
+    // N = the tile's rows) where it pays, unless the items are band-ordered.  Band-ordered, where DRAM
+    // traffic bounds the launch: T = 32768, E = 128 393 us transposed, 366 staged; T = 65536, E = 256
+    // 1010, 891.
+    a.trans = g.epi == EPI_ADD_F32 && !g.item_table && transposed_pays(g.m_total, g.G, g.N) ? 1 : 0;
     if (a.trans && (g.ksplit > 1 || g.o_div > 1 || g.a_rows || g.a_ident || g.ldy >= (int64_t(1) << 31) ||
                     (g.b_kmajor ? g.row_scale != nullptr : !g.o_rows || !g.row_scale)))
         return MOEVIE_ERR_UNSUPPORTED;
