@@ -166,7 +166,9 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, ui
     if (ONE) {
         int ok = 1;
         if ((threadIdx.x & 31) == 0) ok = ready || mbar_wait(bar, parity, limit_ns, abort_flag);
-        return __shfl_sync(0xffffffffu, ok, 0) != 0;
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        __syncwarp();   // orders what lane 0 has seen before what the elected lane issues (the shuffle orders no memory)
+        return ok != 0;
     }
     if (__all_sync(0xffffffffu, ready || mbar_try_wait(bar, parity))) return true;
     const uint64_t t0 = globaltimer_ns();

@@ -1,0 +1,29 @@
+"""Orderings between lanes that a run cannot show missing (the hardware happens to keep them), read
+from the sources."""
+import os
+import re
+
+from paper_2608_17402_gb300 import _build
+
+
+def _source(name):
+    with open(os.path.join(_build.CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())   # without comments
+
+
+def _body(src, head):
+    """The braces' content that follows the first match of `head`."""
+    i = src.index("{", re.search(head, src).end())
+    depth, j = 0, i
+    while True:
+        depth += {"{": 1, "}": -1}.get(src[j], 0)
+        j += 1
+        if depth == 0:
+            return src[i:j]
+
+
+def test_one_lane_wait_publishes_what_it_saw():
+    """Lane 0 alone waits on the barrier; another lane may issue what depends on it.  A shuffle
+    orders no memory accesses between lanes, __syncwarp does."""
+    one = _body(_body(_source("common.cuh"), r"bool mbar_wait_warp\("), r"if \(ONE\)")
+    assert re.search(r"__shfl_sync.*__syncwarp\(\)", one, re.S), one
