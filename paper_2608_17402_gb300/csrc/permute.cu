@@ -258,6 +258,7 @@ constexpr int64_t PERM_CLUSTER_SLOTS = 2048;   // 256 slots per CTA (T = 1024, k
 template <bool CLUSTER>
 __device__ __forceinline__ bool perm_barrier(DevStatus* st) {
     if constexpr (CLUSTER) {   // all threads of all CTAs; orders their global writes and reads
+        __syncwarp();   // .aligned: the whole warp, converged (it may come from loops that its lanes left one by one)
         asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
         return true;
     }
