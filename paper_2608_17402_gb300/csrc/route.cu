@@ -138,7 +138,7 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-// Order-preserving code of a float (larger float, larger code; no NaNs here).
+// Order-preserving code of a float (larger float, larger code; an arithmetic NaN above all).
 __device__ __forceinline__ uint32_t ord_f32(float f) {
     const uint32_t u = __float_as_uint(f);
     return u ^ ((u & 0x80000000u) ? 0xffffffffu : 0x80000000u);
@@ -324,8 +324,8 @@ __device__ __forceinline__ void write_selection(uint32_t taken, const float (&sg
 #pragma unroll
     for (int i = 0; i < NPL; ++i) {
         const uint32_t m = __ballot_sync(0xffffffffu, (taken >> i) & 1u);
-        if ((taken >> i) & 1u) {
-            const int pos = base + __popc(m & lt);
+        const int pos = base + __popc(m & lt);
+        if (((taken >> i) & 1u) && pos < k) {   // (there are k)
             idx[t * k + pos] = lane + 32 * i;
             gate[t * k + pos] = __fdividef(sg[i], ssum);
         }
@@ -432,32 +432,39 @@ __device__ __forceinline__ void bound_candidates(const float (&sv)[NPL], const f
         else if (!(up[i] < l_k)) cand |= 1u << i;
     }
 }
-// Then, with the candidates' exact keys: `need` of them by key, ties to the lower id.
+// Order code of a key in 64 bits (larger key, larger code, above 0); NaN above all, as in ord_f32:
+// the order has to be total, or the lanes would disagree on the choice.
+__device__ __forceinline__ uint64_t ord_f64(double v) {
+    const uint64_t u = (uint64_t)__double_as_longlong(v);
+    return v != v ? ~0ull : u ^ (u >> 63 ? ~0ull : 1ull << 63);
+}
+// Then, with the candidates' exact keys: `need` of them (no more than there are) by key, ties to
+// the lower id; exactly one a round, whatever the keys are.
 template <int NPL>
 __device__ __forceinline__ uint32_t choose_exact(const double (&exk)[NPL], uint32_t sure_in, uint32_t cand, int need,
                                                  int lane) {
     uint32_t chosen = sure_in;
     for (int r = 0; r < need; ++r) {
-        double bv = -INFINITY;
+        uint64_t bv = 0;
         int bi = 0x7fffffff;
 #pragma unroll
         for (int i = 0; i < NPL; ++i) {
-            const int e = lane + 32 * i;
-            if (((cand >> i) & 1u) && !((chosen >> i) & 1u) && (exk[i] > bv || bi == 0x7fffffff)) {
-                bv = exk[i];
-                bi = e;
+            const uint64_t v = ((cand & ~chosen) >> i) & 1u ? ord_f64(exk[i]) : 0;
+            if (v > bv) {
+                bv = v;
+                bi = lane + 32 * i;
             }
         }
 #pragma unroll
         for (int o = 16; o; o >>= 1) {
-            const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+            const uint64_t ov = __shfl_xor_sync(0xffffffffu, (unsigned long long)bv, o);
             const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
             if (ov > bv || (ov == bv && oi < bi)) {
                 bv = ov;
                 bi = oi;
             }
         }
-        if ((bi & 31) == lane) chosen |= 1u << (bi >> 5);
+        if ((bi & 31) == lane && bv) chosen |= 1u << (bi >> 5);
     }
     return chosen;
 }
