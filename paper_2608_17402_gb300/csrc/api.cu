@@ -35,7 +35,7 @@ inline int64_t row_ld(int64_t h) { return (h + 7) / 8 * 8; }
 // stage (which passes 0 for the sizes it does not use).
 struct Layout {
     size_t status, xnorm, wnorm, wpart, wexp, wsplit, wrt, logits, fb_tokens;
-    size_t idx, gate, hist, counts, offsets, tiles, n_tiles, items, n_items, perm, inv, row_tok,
+    size_t idx, gate, hist, counts, offsets, tiles, n_tiles, items, n_items, row_tok,
         row_gate;
     size_t H, Hs, yacc;
     size_t total;
@@ -134,8 +134,6 @@ Layout make_layout(int64_t T, int64_t d, int64_t E, int64_t k, int64_t h, int64_
     L.items = take(16 * max_mtiles(n, E) * n_nt);   // band-ordered down-projection items
     L.n_items = take(4);
     L.n_tiles = take(4);
-    L.perm = take(4 * n);   // (room of earlier layouts: the forward writes perm and inv only to the
-    L.inv = take(4 * n);    //  caller's arrays; the size that callers ask for stays what it was)
     L.row_tok = take(4 * n2);
     L.row_gate = take(4 * n2);
     L.H = take(2 * n2 * row_ld(h));
@@ -374,7 +372,6 @@ moevie_status run_gemm(const GemmSpec& g, DevStatus* st, cudaStream_t s) {
         a.n_ntiles = (g.N + a.n_step - 1) / a.n_step;
     }
     a.num_kb = (g.K + GM_BK - 1) / GM_BK;
-    a.nbox = (a.BN + 63) / 64;
     a.epi = g.epi;
     a.out = static_cast<__nv_bfloat16*>(g.out);
     a.ldo = g.ldo;
@@ -387,8 +384,7 @@ moevie_status run_gemm(const GemmSpec& g, DevStatus* st, cudaStream_t s) {
     a.scale = g.scale;
     a.ksplit = g.ksplit > 1 ? g.ksplit : 1;
     if (a.ksplit > a.num_kb) return MOEVIE_ERR_UNSUPPORTED;
-    if (a.ksplit > 1 && g.epi != EPI_STORE_F32 && g.epi != EPI_ADD_F32 && g.epi != EPI_SUM2_F32)
-        return MOEVIE_ERR_UNSUPPORTED;
+    if (a.ksplit > 1 && g.epi != EPI_STORE_F32 && g.epi != EPI_SUM2_F32) return MOEVIE_ERR_UNSUPPORTED;
     if (g.epi == EPI_SUM2_F32 && (g.N % 64 != 0 || g.N > GM_MAXBN)) return MOEVIE_ERR_UNSUPPORTED;
     a.y_split_stride = g.y_split_stride;
     a.status = st;

@@ -140,8 +140,8 @@ __device__ __forceinline__ int block_scan_1024(int v, int* s_w, int* total) {
 // their number (at most max_items; more is a device error and none are listed).  A group
 // of one chunk writes each of its gradient's elements once: its items carry BWD_STORE_BIT in
 // kb1 (the GEMM stores instead of adding) and gclear[g] = 0; a group with no rows or several
-// chunks has gclear[g] = 1 (its gradient is cleared first).  (Seven to nine launches of one
-// CTA each before, 3 - 4 us apiece.)
+// chunks has gclear[g] = 1 (its gradient is cleared first).  (One launch for all the
+// tables: of one CTA each they take 3 - 4 us apiece, seven to nine of them.)
 __global__ void __launch_bounds__(1024) bwd_plan_kernel(const __grid_constant__ BwdPlan p) {
     pdl_wait();
     __shared__ int s_w[33];

@@ -1196,7 +1196,7 @@ __global__ void __launch_bounds__(GM_THREADS, 1) grouped_gemm_kernel(const __gri
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(gm_smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint8_t* sA = smem;
-    constexpr int nst = gm_stages(ECLS, TRAIN);
+    constexpr int nst = gm_stages(ECLS);
     uint8_t* sB = smem + nst * GM_A_BYTES;
     uint8_t* sStg = sB + nst * GM_B_BYTES;                       // epilogue staging
     uint64_t* bars = reinterpret_cast<uint64_t*>(sStg + gm_stg_bytes(ECLS, TRAIN));

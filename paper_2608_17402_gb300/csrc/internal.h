@@ -223,11 +223,11 @@ __host__ __device__ constexpr int gm_stg_bytes(int ecls, bool train) {
            : ecls == ECLS_DGELU ? GM_EPI_WARPS * 2 * 2 * 1024
            : ecls == ECLS_DSWIGLU ? GM_EPI_WARPS * 2 * 3 * 1024 : 0;
 }
-__host__ __device__ constexpr int gm_stages(int ecls, bool) {
+__host__ __device__ constexpr int gm_stages(int ecls) {
     return ecls == ECLS_DGELU || ecls == ECLS_DSWIGLU ? 5 : 6;
 }
 __host__ __device__ constexpr int gm_smem_bytes(int ecls, bool train) {
-    return gm_stages(ecls, train) * (GM_A_BYTES + GM_B_BYTES) + gm_stg_bytes(ecls, train) + GM_OVERHEAD_BYTES;
+    return gm_stages(ecls) * (GM_A_BYTES + GM_B_BYTES) + gm_stg_bytes(ecls, train) + GM_OVERHEAD_BYTES;
 }
 static_assert(gm_smem_bytes(ECLS_BF16, true) <= 232448 && gm_smem_bytes(ECLS_BF16, false) <= 232448 &&
                   gm_smem_bytes(ECLS_F32, false) <= 232448 && gm_smem_bytes(ECLS_ADD, true) <= 232448 &&
@@ -292,7 +292,7 @@ struct GemmArgs {
     int a_ident;                // gathered path with A row r = r (contiguous rows through cp.async)
     const int32_t* n_tiles_dev; // number of entries of `tiles`
     int64_t max_mtiles;         // host bound on *n_tiles_dev
-    int G, K, N, BN, n_ntiles, num_kb, nbox;
+    int G, K, N, BN, n_ntiles, num_kb;
     int g_split;                // first group read through tmB2 (G when there is none)
     int swiglu;                 // EPI_SWIGLU_BF16: B half of CTA rank 1 from tmB2 (W3), same columns;
                                 // groups g >= g_split from tmB3 (rank 0) and tmB4 (rank 1)

@@ -354,8 +354,8 @@ __global__ void __launch_bounds__(1024) tile_table_kernel(const int32_t* __restr
 
 constexpr int ITEM_CTAS = 8;
 // ITEM_CTAS CTAs of 1024 threads; each ranks every m-tile itself and writes its share of the
-// items (one CTA alone spent most of its time on the 16-byte scattered writes: 19 us for 15 k
-// items, 13 this way).  Orders the (m-tile, n-tile) work items of a grouped GEMM
+// items (one CTA alone spends most of its time on the 16-byte scattered writes: 19 us for 15 k
+// items against 13).  Orders the (m-tile, n-tile) work items of a grouped GEMM
 // in nb token bands x column groups of gsz n-tiles: band b holds the m-tiles whose
 // middle row's token lies in [b T / nb, (b + 1) T / nb) (expert-major order kept
 // inside a band).  Items run band-major, then column group, then m-tile, then n-tile,
