@@ -1007,8 +1007,10 @@ __device__ void epilogue_bf16(const GemmArgs& p, const Smem& sm, uint32_t tmem, 
         auto copy_out = [&](int c) {   // the step's rows, written by all lanes, to columns t.n0 + c ..
             __syncwarp();
             const bool ok = t.n0 + c + 8 * q0 < p.N;
-            if (!TRAIN && swiglu) {   // a chunk's stores apart, each address formed before its store: at T =
-#pragma unroll                        // 8192, d = 1280, h = 854 196 us, with the form below 200
+            // SwiGLU: a chunk's stores apart, each address formed before its store (at T = 8192, d = 1280,
+            // h = 854 196 us; back to back as below 200)
+            if (!TRAIN && swiglu) {
+#pragma unroll
                 for (int i = 0; i < NP; ++i) {
                     const int row = (lane + 32 * i) / NP, q = (lane + 32 * i) % NP;
                     if (row < nrow && t.n0 + c + 8 * q < p.N)
