@@ -36,6 +36,8 @@
 // on the FMA pipes, the same certified selection and the same exact re-decision.
 #include <math.h>
 
+#include <algorithm>
+
 #include "internal.h"
 
 namespace mv {
@@ -673,8 +675,8 @@ constexpr size_t route_small_smem() {
 // lanes over the experts: the weights are read as whole rows of W_r and taken apart once for those
 // tokens, the warps (with E <= 16 also the parts of a warp) share the terms, and a pass costs
 // the same however many of the experts tie; the integer instructions bound it (about 20 a term).
-// The whole router on tokens that tie in every key (W_r = 0, b = 0): 32 us at T = 64, d = 1024, E =
-// 32, 98 at T = 1216, d = 512, E = 64, against 57 and 186 of the tensor-core route; on 1216 tokens
+// The whole router on tokens that tie in every key (W_r = 0, b = 0): 36 us at T = 64, d = 1024, E =
+// 32, 93 at T = 1216, d = 512, E = 64, against 57 and 186 of the tensor-core route; on 1216 tokens
 // with two candidates each (d = 1024, E = 32) 27 against 31.  One token after another through all of
 // its steps, the threads over the terms for any number of candidates: 330, 470 and 57.
 // sums: the warps' sums, [RS_NW][FB_BATCH] and the candidates' ids, or [RS_G][RS_NW][EP]; xp: the
@@ -1164,9 +1166,10 @@ cudaError_t launch_route_small(const __nv_bfloat16* x, const float* Wr, const fl
     if (!route_small(T, d, E)) return cudaErrorInvalidValue;
     static_assert(route_small_smem<1>() <= 38 * 1024 && route_small_smem<2>() <= 38 * 1024,
                   "no opt-in needed beside the static arrays (9 KB)");
-    // as few tokens a CTA as one wave of the SMs allows (a CTA takes as long with one as with eight),
-    // so that tokens that need the exact logits are spread over the SMs
-    const int tb = (T + ROUTE_SMALL_SMS - 1) / ROUTE_SMALL_SMS;
+    // as few tokens a CTA as one wave of the SMs allows (a CTA takes as long with two as with eight),
+    // so that tokens that need the exact keys are spread over the SMs: T = 16, d = 512, E = 64, all
+    // tied, 34 us with two tokens a CTA, 53 with four (one: 27, but 10.7 instead of 10.2 untied)
+    const int tb = std::max(2, (T + ROUTE_SMALL_SMS - 1) / ROUTE_SMALL_SMS);
     const auto kern = E <= 32 ? route_small_kernel<1> : route_small_kernel<2>;
     const cudaError_t e = launch_pdl(kern, dim3((unsigned)((T + tb - 1) / tb)), dim3(256),
                                      E <= 32 ? route_small_smem<1>() : route_small_smem<2>(), s, x, Wr, b, T, d, E,
